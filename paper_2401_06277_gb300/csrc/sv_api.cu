@@ -106,6 +106,8 @@ void free_all(stokes_hierarchy* h) {
   cudaFree(h->bt_buf);
   h->bt_GL = h->bt_GM = h->bt_buf = nullptr;
   h->lv.clear();
+  cudaFree(h->stencil_G);
+  h->stencil_G = nullptr;
   cudaFree(h->coarse_G);
   cudaFree(h->V);
   cudaFree(h->Z);
@@ -193,6 +195,8 @@ void sweep_f64(stokes_hierarchy* h, sv::Level& L, const double* x, const double*
     sv::launch_bs_sweep<double>(L.d, h->bs, static_cast<double*>(h->bs_buf), L.r, x, b, xo, h->stream);
   else if (h->prm.smoother == STOKES_SMOOTHER_PER_PATCH)
     sv::launch_simple_sweep(L.d, L.pinv, h->delta, L.r, x, b, xo, h->prm.omega, h->stream);
+  else if (L.vk_cfg == sv::VANKA_CFG_STENCIL)
+    sv::launch_vanka_stencil(L.d, h->stencil_G, x, b, xo, h->prm.omega, L.r, h->stream);
   else if (sv::vanka_cfg_split(L.vk_cfg))
     sv::launch_vanka_split<double>(L.d, L.cd, h->fd, x, b, xo, h->prm.omega, h->delta, L.vk_cfg == sv::VANKA_CFG_SPLIT2,
                            h->stream, L.r);
@@ -788,6 +792,7 @@ cudaError_t tune_level(stokes_hierarchy* h, sv::Level& L, int* cfg) {
   return cudaGetLastError();
 }
 
+constexpr int STENCIL_MAX_N = 160;
 cudaError_t choose_tiles(stokes_hierarchy* h) {
   for (sv::Level& L : h->lv) {
     if (h->prm.tile >= 0 || h->prm.smoother != STOKES_SMOOTHER_SHARED || h->prm.precond == 1) {
@@ -801,7 +806,8 @@ cudaError_t choose_tiles(stokes_hierarchy* h) {
     // only the precision the V-cycle runs in is tuned (the FP64 sweep of a
     // mixed hierarchy serves stokes_vanka_sweep alone and keeps 16x8)
     cudaError_t e = cudaSuccess;
-    if (h->prm.prec == STOKES_FP64) e = tune_level<double>(h, L, &L.vk_cfg);
+    if (h->prm.prec == STOKES_FP64 && L.d.n >= sv::VS_MIN_N && L.d.n <= STENCIL_MAX_N) L.vk_cfg = sv::VANKA_CFG_STENCIL;
+    else if (h->prm.prec == STOKES_FP64) e = tune_level<double>(h, L, &L.vk_cfg);
     else e = tune_level<float>(h, L, &L.vk_cfg_f);   // strip sweep vs SIMT shapes
     if (e != cudaSuccess) return e;
   }
@@ -1016,6 +1022,17 @@ stokes_status stokes_hierarchy_create(int n, double viscosity, const stokes_para
       free_all(h);
       delete h;
       return cuda_fail(e, "block-triangular set-up");
+    }
+  }
+  if (prm.prec == STOKES_FP64 && prm.smoother == STOKES_SMOOTHER_SHARED) {
+    const std::vector<long double>& G = sv::vanka_stencil();
+    const std::vector<double> Gd(G.begin(), G.end());
+    if ((e = dalloc(&h->stencil_G, Gd.size())) != cudaSuccess ||
+        (e = cudaMemcpy(h->stencil_G, Gd.data(), Gd.size() * sizeof(double), cudaMemcpyHostToDevice)) !=
+            cudaSuccess) {
+      free_all(h);
+      delete h;
+      return cuda_fail(e, "composite stencil upload");
     }
   }
   const size_t Nf = static_cast<size_t>(h->lv.back().d.N);

@@ -224,6 +224,7 @@ struct stokes_hierarchy {
   std::vector<sv::Level> lv;     // lv[0] = coarsest
   sv::FastDiag fd;               // interior patch factors (level independent)
   sv::FastDiagT<float> fdf;      // the same in FP32
+  double* stencil_G = nullptr;   // FP64 form: the composite Vanka stencil (VS_TAB doubles)
   double* coarse_G = nullptr;    // N0 x N0 dense inverse of the bordered coarse system
   int N0 = 0;
   // FGMRES workspace
@@ -322,10 +323,24 @@ constexpr int VANKA_CFG_14 = 3;
 constexpr int VANKA_CFG_SPLIT = 4;   // FP64 only: own-patch solves + separate update (launch_vanka_split)
 constexpr int VANKA_CFG_SPLIT2 = 5;  // the same, compiled for two CTAs per SM (at most 128 registers)
 constexpr int VANKA_CFG_4 = 6;       // fused 4x4 tiles: small levels, spread over more SMs
+constexpr int VANKA_CFG_STENCIL = 7; // FP64 only: the residual, then the composite stencil (launch_vanka_stencil)
 inline bool vanka_cfg_split(int cfg) { return cfg == VANKA_CFG_SPLIT || cfg == VANKA_CFG_SPLIT2; }
 template <typename R>
 void launch_vanka(const LevelDev& L, const R* cd, const FastDiagT<R>& fd, const R* x, const R* b, R* xo,
                   double omega, int cfg, cudaStream_t s, int skip_lo = 1, int skip_hi = 0);
+
+// The additive Vanka correction as one stencil (sv_vanka_stencil.cu).  Table layout:
+// [position_y][position_x] (0, 1, 2, interior, n-2, n-1, n per axis) x 9 outputs of a
+// cell (c * 4 + J parity * 2 + I parity, then p) x VS_OUT coefficients: velocity
+// residuals [9 node rows][9 node columns][component] from node (2i - 4, 2j - 4),
+// pressure residuals [3][3] from vertex (i - 1, j - 1), one pad.  Integer units.
+constexpr int VS_POS = 7, VS_OUT = 172, VS_TYPE = 9 * VS_OUT, VS_TAB = VS_POS * VS_POS * VS_TYPE;
+constexpr int VS_MIN_N = 6;   // below it the positions of a cell overlap
+const std::vector<long double>& vanka_stencil();
+// x_out = x + omega (stencil (b - A x)); x may be null (zero guess, the residual is b);
+// rscratch: a level vector.  G: the table in FP64 on the device.  n >= VS_MIN_N.
+void launch_vanka_stencil(const LevelDev& L, const double* G, const double* x, const double* b, double* xo,
+                          double omega, double* rscratch, cudaStream_t s);
 
 // Persistent coarse-level kernel (sv_vanka.cu): one cooperative launch of `grid`
 // CTAs runs the nops steps; err is set to 1 if a grid barrier gave up.

@@ -185,6 +185,11 @@ __global__ void k_coarse(const double* __restrict__ G, int N0, const double* __r
   if (lane == 0) e[row] = s;
 }
 
+// Threads of a per-vertex kernel on an np x np grid.  A block of 8 rows puts 8 warps
+// on one SM; on the small levels that leaves most SMs idle while those warps queue
+// for the FP64 pipe, so they take one row per block.
+dim3 vertex_block(int np) { return np > 257 ? dim3(32, 8) : np > 129 ? dim3(32, 2) : dim3(32, 1); }
+
 dim3 grid2(int nx, int ny, dim3 blk) {
   return dim3((nx + blk.x - 1) / blk.x, (ny + blk.y - 1) / blk.y);
 }
@@ -194,7 +199,7 @@ dim3 grid2(int nx, int ny, dim3 blk) {
 template <typename T>
 void launch_apply(const LevelDev& L, const T* x, const T* b, T* y, int residual, cudaStream_t s) {
   count_launches(1);
-  dim3 blk(32, 8);
+  const dim3 blk = vertex_block(L.np);
   launch_pdl(k_apply<T>, dim3(grid2(L.np, L.np, blk)), dim3(blk), 0, s, L, x, b, y, residual);
 }
 
@@ -214,14 +219,14 @@ void launch_rhs_transpose(const LevelDev& L, const double* lam, double* g, cudaS
 template <typename T>
 void launch_restrict(const LevelDev& F, const LevelDev& C, const T* rf, T* rc, cudaStream_t s) {
   count_launches(1);
-  dim3 blk(32, 8);
+  const dim3 blk = vertex_block(C.np);
   launch_pdl(k_restrict<T>, dim3(grid2(C.n + 1, C.n + 1, blk)), dim3(blk), 0, s, F, C, rf, rc);
 }
 
 template <typename T>
 void launch_prolong_add(const LevelDev& F, const LevelDev& C, const T* ec, T* xf, cudaStream_t s) {
   count_launches(1);
-  dim3 blk(32, 8);
+  const dim3 blk = vertex_block(C.np);
   launch_pdl(k_prolong_add<T>, dim3(grid2(C.n + 1, C.n + 1, blk)), dim3(blk), 0, s, F, C, ec, xf);
 }
 
