@@ -196,7 +196,7 @@ void sweep_f64(stokes_hierarchy* h, sv::Level& L, const double* x, const double*
   else if (h->prm.smoother == STOKES_SMOOTHER_PER_PATCH)
     sv::launch_simple_sweep(L.d, L.pinv, h->delta, L.r, x, b, xo, h->prm.omega, h->stream);
   else if (L.vk_cfg == sv::VANKA_CFG_STENCIL)
-    sv::launch_vanka_stencil(L.d, h->stencil_G, x, b, xo, h->prm.omega, L.r, h->stream);
+    sv::launch_vanka_stencil<double>(L.d, h->stencil_G, x, b, xo, h->prm.omega, L.r, h->stream);
   else if (sv::vanka_cfg_split(L.vk_cfg))
     sv::launch_vanka_split<double>(L.d, L.cd, h->fd, x, b, xo, h->prm.omega, h->delta, L.vk_cfg == sv::VANKA_CFG_SPLIT2,
                            h->stream, L.r);

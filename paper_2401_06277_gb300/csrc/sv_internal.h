@@ -338,9 +338,10 @@ constexpr int VS_POS = 7, VS_OUT = 172, VS_TYPE = 9 * VS_OUT, VS_TAB = VS_POS * 
 constexpr int VS_MIN_N = 6;   // below it the positions of a cell overlap
 const std::vector<long double>& vanka_stencil();
 // x_out = x + omega (stencil (b - A x)); x may be null (zero guess, the residual is b);
-// rscratch: a level vector.  G: the table in FP64 on the device.  n >= VS_MIN_N.
-void launch_vanka_stencil(const LevelDev& L, const double* G, const double* x, const double* b, double* xo,
-                          double omega, double* rscratch, cudaStream_t s);
+// rscratch: a level vector.  G: the table on the device in the element type.  n >= VS_MIN_N.
+template <typename T>
+void launch_vanka_stencil(const LevelDev& L, const T* G, const T* x, const T* b, T* xo, double omega, T* rscratch,
+                          cudaStream_t s);
 
 // Persistent coarse-level kernel (sv_vanka.cu): one cooperative launch of `grid`
 // CTAs runs the nops steps; err is set to 1 if a grid barrier gave up.

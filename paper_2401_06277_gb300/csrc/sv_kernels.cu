@@ -166,6 +166,72 @@ __global__ void k_prolong_add(LevelDev F, LevelDev C, const T* __restrict__ ec, 
   ops::prolong_elem<T>(F, C, ec, xf, ex, ey);
 }
 
+// One output per thread (small levels; sv_level_ops.cuh): a warp takes one output kind
+// of 32 consecutive cells, block.x = 32, output kind = blockIdx.y.
+template <typename T>
+__global__ void __launch_bounds__(32) k_apply_out(LevelDev L, const T* __restrict__ x, const T* __restrict__ b,
+                                                  T* __restrict__ y, int residual) {
+  pdl_begin();
+  const int k = blockIdx.x * 32 + threadIdx.x;
+  if (k >= L.np * L.np) return;
+  const int bb = k / L.np, a = k - bb * L.np;
+  switch (blockIdx.y) {
+    case 0: ops::apply_out<T, 0, 0, 0>(L, x, b, y, residual, a, bb); break;
+    case 1: ops::apply_out<T, 0, 0, 1>(L, x, b, y, residual, a, bb); break;
+    case 2: ops::apply_out<T, 0, 1, 0>(L, x, b, y, residual, a, bb); break;
+    case 3: ops::apply_out<T, 0, 1, 1>(L, x, b, y, residual, a, bb); break;
+    case 4: ops::apply_out<T, 1, 0, 0>(L, x, b, y, residual, a, bb); break;
+    case 5: ops::apply_out<T, 1, 0, 1>(L, x, b, y, residual, a, bb); break;
+    case 6: ops::apply_out<T, 1, 1, 0>(L, x, b, y, residual, a, bb); break;
+    case 7: ops::apply_out<T, 1, 1, 1>(L, x, b, y, residual, a, bb); break;
+    default: ops::apply_out<T, 2, 0, 0>(L, x, b, y, residual, a, bb); break;
+  }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(32) k_restrict_out(LevelDev F, LevelDev C, const T* __restrict__ rf,
+                                                     T* __restrict__ rc) {
+  pdl_begin();
+  const int k = blockIdx.x * 32 + threadIdx.x;
+  if (k >= C.np * C.np) return;
+  const int ey = k / C.np, ex = k - ey * C.np;
+  switch (blockIdx.y) {
+    case 0: ops::restrict_out<T, 0, 0, 0>(F, C, rf, rc, ex, ey); break;
+    case 1: ops::restrict_out<T, 0, 0, 1>(F, C, rf, rc, ex, ey); break;
+    case 2: ops::restrict_out<T, 0, 1, 0>(F, C, rf, rc, ex, ey); break;
+    case 3: ops::restrict_out<T, 0, 1, 1>(F, C, rf, rc, ex, ey); break;
+    case 4: ops::restrict_out<T, 1, 0, 0>(F, C, rf, rc, ex, ey); break;
+    case 5: ops::restrict_out<T, 1, 0, 1>(F, C, rf, rc, ex, ey); break;
+    case 6: ops::restrict_out<T, 1, 1, 0>(F, C, rf, rc, ex, ey); break;
+    case 7: ops::restrict_out<T, 1, 1, 1>(F, C, rf, rc, ex, ey); break;
+    default: ops::restrict_out<T, 2, 0, 0>(F, C, rf, rc, ex, ey); break;
+  }
+}
+
+// blockIdx.y: 0..31 = component * 16 + fy * 4 + fx, 32..35 = the fine vertices
+template <typename T, int K>
+__device__ __forceinline__ void prolong_case(const LevelDev& F, const LevelDev& C, const T* ec, T* xf, int ex, int ey,
+                                             int kind) {
+  if constexpr (K < 36) {
+    if (kind == K) {
+      if constexpr (K < 32) ops::prolong_out<T, (K >> 4), ((K >> 2) & 3), (K & 3)>(F, C, ec, xf, ex, ey);
+      else ops::prolong_out<T, 2, (K >> 1) & 1, K & 1>(F, C, ec, xf, ex, ey);
+    } else {
+      prolong_case<T, K + 1>(F, C, ec, xf, ex, ey, kind);
+    }
+  }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(32) k_prolong_out(LevelDev F, LevelDev C, const T* __restrict__ ec,
+                                                    T* __restrict__ xf) {
+  pdl_begin();
+  const int k = blockIdx.x * 32 + threadIdx.x;
+  if (k >= C.np * C.np) return;
+  const int ey = k / C.np, ex = k - ey * C.np;
+  prolong_case<T, 0>(F, C, ec, xf, ex, ey, blockIdx.y);
+}
+
 template <typename TI, typename TO>
 __global__ void k_convert(const TI* __restrict__ in, TO* __restrict__ out, long long N) {
   pdl_begin();
@@ -185,10 +251,10 @@ __global__ void k_coarse(const double* __restrict__ G, int N0, const double* __r
   if (lane == 0) e[row] = s;
 }
 
-// Threads of a per-vertex kernel on an np x np grid.  A block of 8 rows puts 8 warps
-// on one SM; on the small levels that leaves most SMs idle while those warps queue
-// for the FP64 pipe, so they take one row per block.
-dim3 vertex_block(int np) { return np > 257 ? dim3(32, 8) : np > 129 ? dim3(32, 2) : dim3(32, 1); }
+// Levels whose per-vertex kernels run one output per thread.  At np = 129 the operator
+// has 4680 such warps for 608 sub-partitions; above, a thread per vertex fills them.
+constexpr int OUT_MAX_NP = 129;
+dim3 out_grid(int np, int kinds) { return dim3((np * np + 31) / 32, kinds); }
 
 dim3 grid2(int nx, int ny, dim3 blk) {
   return dim3((nx + blk.x - 1) / blk.x, (ny + blk.y - 1) / blk.y);
@@ -199,7 +265,11 @@ dim3 grid2(int nx, int ny, dim3 blk) {
 template <typename T>
 void launch_apply(const LevelDev& L, const T* x, const T* b, T* y, int residual, cudaStream_t s) {
   count_launches(1);
-  const dim3 blk = vertex_block(L.np);
+  if (L.np <= OUT_MAX_NP) {
+    launch_pdl(k_apply_out<T>, out_grid(L.np, 9), dim3(32), 0, s, L, x, b, y, residual);
+    return;
+  }
+  dim3 blk(32, 8);
   launch_pdl(k_apply<T>, dim3(grid2(L.np, L.np, blk)), dim3(blk), 0, s, L, x, b, y, residual);
 }
 
@@ -219,14 +289,22 @@ void launch_rhs_transpose(const LevelDev& L, const double* lam, double* g, cudaS
 template <typename T>
 void launch_restrict(const LevelDev& F, const LevelDev& C, const T* rf, T* rc, cudaStream_t s) {
   count_launches(1);
-  const dim3 blk = vertex_block(C.np);
+  if (C.np <= OUT_MAX_NP) {
+    launch_pdl(k_restrict_out<T>, out_grid(C.np, 9), dim3(32), 0, s, F, C, rf, rc);
+    return;
+  }
+  dim3 blk(32, 8);
   launch_pdl(k_restrict<T>, dim3(grid2(C.n + 1, C.n + 1, blk)), dim3(blk), 0, s, F, C, rf, rc);
 }
 
 template <typename T>
 void launch_prolong_add(const LevelDev& F, const LevelDev& C, const T* ec, T* xf, cudaStream_t s) {
   count_launches(1);
-  const dim3 blk = vertex_block(C.np);
+  if (C.np <= OUT_MAX_NP / 2 + 1) {
+    launch_pdl(k_prolong_out<T>, out_grid(C.np, 36), dim3(32), 0, s, F, C, ec, xf);
+    return;
+  }
+  dim3 blk(32, 8);
   launch_pdl(k_prolong_add<T>, dim3(grid2(C.n + 1, C.n + 1, blk)), dim3(blk), 0, s, F, C, ec, xf);
 }
 

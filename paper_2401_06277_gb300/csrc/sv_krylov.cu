@@ -31,6 +31,36 @@ __device__ __forceinline__ double warp_sum(double v) {
 template <int K>
 constexpr int orth_unroll() { return K <= 1 ? 4 : (K <= 4 ? 2 : 1); }
 
+// red[OFF + k] = sum over the warp of acc[OFF + k], k < NO - OFF.  In chunks of C (a
+// power of two) values: each of the first log2 C steps exchanges half of the values
+// still held, so a chunk costs C - 1 + 5 - log2 C additions instead of 5 C.  An FP64
+// addition holds a sub-partition's unit for 64 clocks, and the block sums of nine
+// values by nine separate trees were most of a small grid's pass.
+template <int NO, int OFF = 0>
+__device__ __forceinline__ void warp_sums(const double (&acc)[NO], int lane, double* red) {
+  if constexpr (OFF < NO) {
+    constexpr int R = NO - OFF;
+    constexpr int C = R >= 16 ? 16 : R >= 8 ? 8 : R >= 4 ? 4 : R >= 2 ? 2 : 1;
+    double v[C];
+#pragma unroll
+    for (int k = 0; k < C; ++k) v[k] = acc[OFF + k];
+    int idx = 0, o = 16;
+#pragma unroll
+    for (int h = C / 2; h >= 1; h /= 2, o /= 2) {
+      const bool up = (lane & o) != 0;
+#pragma unroll
+      for (int k = 0; k < h; ++k) {
+        const double send = up ? v[k] : v[k + h], keep = up ? v[k + h] : v[k];
+        v[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+      }
+      idx += up ? h : 0;
+    }
+    for (; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+    if ((lane & (32 / C - 1)) == 0) red[OFF + idx] = v[0];
+    warp_sums<NO, OFF + C>(acc, lane, red);
+  }
+}
+
 // Reduces acc[0..NO) over the block into partials[t * npart + blockIdx.x] and
 // returns, in every thread, whether this block is the last of the grid to
 // finish (its partials then see all others').  The last block resets *ticket.
@@ -40,11 +70,7 @@ __device__ __forceinline__ bool block_partials(const double (&acc)[NO], double* 
   __shared__ double red[DOT_NT / 32][NO];
   __shared__ unsigned last;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-  for (int k = 0; k < NO; ++k) {
-    const double v = warp_sum(acc[k]);
-    if (lane == 0) red[wid][k] = v;
-  }
+  warp_sums<NO>(acc, lane, red[wid]);
   __syncthreads();
   if (threadIdx.x < NO) {
     double s = 0.0;
@@ -469,6 +495,14 @@ std::atomic<long long> g_tc_launches{0};
 
 int dot_blocks() { return DOT_BLOCKS; }
 
+// Blocks of a reduction over N elements: at least two elements per thread, so that a
+// small grid does not spend its time on the block sums and the last block's total of
+// 608 partials (N = 9539: 608 -> 19 blocks).
+static int dot_blocks_for(long long N, int npart) {
+  const long long b = (N + 2 * DOT_NT - 1) / (2 * DOT_NT);
+  return b < 1 ? 1 : b < npart ? static_cast<int>(b) : npart;
+}
+
 template <int K>
 void dots_k(bool norm, const double* V, long long ld, const double* w, long long N, double* partials,
             int npart, unsigned* ticket, double* dots, double* norm2, const double* gate, cudaStream_t s) {
@@ -531,6 +565,7 @@ void update_dots_k(double* w, const double* V, long long ld, const double* coef,
 void launch_orth_dots(const double* V, long long ld, int nk, const double* w, long long N, double* partials,
                       int npart, unsigned* ticket, double* dots, double* norm2, const double* gate,
                       cudaStream_t s) {
+  npart = dot_blocks_for(N, npart);
   // chunks of ORTH_KMAX vectors; the first chunk also takes ||w||^2
   int k0 = 0;
   do {
@@ -545,6 +580,7 @@ void launch_orth_dots(const double* V, long long ld, int nk, const double* w, lo
 void launch_orth_update(double* w, const double* V, long long ld, int nk, const double* coef, long long N,
                         double* partials, int npart, unsigned* ticket, double* norm2, const double* gate,
                         const double* dgks_ref, double* flag, double* hacc, cudaStream_t s) {
+  npart = dot_blocks_for(N, npart);
   // chunks of ORTH_KMAX vectors; the last chunk takes the norm, the flag and hacc
   int k0 = 0;
   do {
@@ -560,6 +596,7 @@ void launch_orth_update(double* w, const double* V, long long ld, int nk, const 
 bool launch_orth_update_dots(double* w, const double* V, long long ld, int nk, const double* coef, long long N,
                              double* partials, int npart, unsigned* ticket, double* dots, double* norm2,
                              const double* dgks_ref, double* flag, cudaStream_t s) {
+  npart = dot_blocks_for(N, npart);
   if (nk < 1 || nk > ORTH_KMAX) return false;   // one launch holds at most ORTH_KMAX vectors
   const int kk = nk;
   count_launches(1);
@@ -571,6 +608,7 @@ bool launch_orth_update_dots(double* w, const double* V, long long ld, int nk, c
 
 void launch_mgs_step(double* w, const double* Va, const double* Vb, const double* coef, long long N,
                      double* partials, int npart, unsigned* ticket, double* dots, double* norm2, cudaStream_t s) {
+  npart = dot_blocks_for(N, npart);
   if (Va == nullptr && Vb == nullptr) return;   // a step reads at least one basis vector
   count_launches(1);
   const dim3 g(npart), b(DOT_NT);

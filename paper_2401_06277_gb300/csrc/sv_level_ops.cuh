@@ -275,6 +275,170 @@ __device__ __forceinline__ void prolong_elem(const LevelDev& F, const LevelDev& 
   }
 }
 
+// ---------------------------------------------------------------------------
+// The same operations with one output per thread, for the small levels: an FP64
+// instruction of a warp holds its sub-partition's unit for 64 clocks, so a thread
+// that evaluates a whole cell (170 multiply-adds) takes microseconds however few
+// cells there are; one output is at most 25 + 6.  Terms are added in the order of
+// the per-cell bodies above, so the values are equal bit for bit.
+// ---------------------------------------------------------------------------
+
+// y = A x or b - A x at output o (C component, PJ, PI node parity; C = 2: the
+// pressure row) of vertex (a, bb)
+template <typename T, int C, int PJ, int PI>
+__device__ __forceinline__ void apply_out(const LevelDev& L, const T* x, const T* b, T* y, int residual, int a,
+                                          int bb) {
+  const int nq = L.nq, np = L.np, n = L.n;
+  const long long nv = L.nv;
+  if constexpr (C == 2) {
+    T X[2][5][5];
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+#pragma unroll
+      for (int r = 0; r < 5; ++r)
+#pragma unroll
+        for (int q = 0; q < 5; ++q) {
+          const double w = c == 0 ? crow(q - 2) * nrow(r - 2) : nrow(q - 2) * crow(r - 2);
+          const int I = 2 * a - 2 + q, J = 2 * bb - 2 + r;
+          X[c][r][q] = (w != 0.0 && is_free(I, J, nq)) ? x[c * nv + static_cast<long long>(J) * nq + I] : T(0);
+        }
+    T bu = T(0);
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+#pragma unroll
+      for (int dJ = -2; dJ <= 2; ++dJ)
+#pragma unroll
+        for (int dI = -2; dI <= 2; ++dI) {
+          const T w = T(c == 0 ? crow(dI) * nrow(dJ) : nrow(dI) * crow(dJ));
+          if (w != T(0)) bu = fma(w, X[c][dJ + 2][dI + 2], bu);
+        }
+    const T ap = level_cb<T>(L) * bu;
+    const long long k = 2 * nv + static_cast<long long>(bb) * np + a;
+    y[k] = residual ? b[k] - ap : ap;
+  } else {
+    const int I = 2 * a + PI, J = 2 * bb + PJ;
+    if (I >= nq || J >= nq) return;
+    const T* xc = x + C * nv;
+    const long long k = C * nv + static_cast<long long>(J) * nq + I;
+    T v;
+    if (!is_free(I, J, nq)) {
+      v = x[k];   // Dirichlet row: identity
+    } else {
+      T X[5][5], P[3][3];
+#pragma unroll
+      for (int dJ = -2; dJ <= 2; ++dJ)
+#pragma unroll
+        for (int dI = -2; dI <= 2; ++dI) {
+          const double cf = k1(PI, dI) * m1(PJ, dJ) + m1(PI, dI) * k1(PJ, dJ);
+          X[dJ + 2][dI + 2] = (cf != 0.0 && is_free(I + dI, J + dJ, nq))
+                                  ? xc[static_cast<long long>(J + dJ) * nq + I + dI] : T(0);
+        }
+#pragma unroll
+      for (int dj = -1; dj <= 1; ++dj)
+#pragma unroll
+        for (int di = -1; di <= 1; ++di) {
+          const double w = C == 0 ? ccol(2 + PI, 1 + di) * ncol(2 + PJ, 1 + dj)
+                                  : ncol(2 + PI, 1 + di) * ccol(2 + PJ, 1 + dj);
+          const int pi = a + di, pj = bb + dj;
+          P[dj + 1][di + 1] = (w != 0.0 && pi >= 0 && pj >= 0 && pi <= n && pj <= n)
+                                  ? x[2 * nv + static_cast<long long>(pj) * np + pi] : T(0);
+        }
+      T sl = T(0), g = T(0);
+#pragma unroll
+      for (int dJ = -2; dJ <= 2; ++dJ)
+#pragma unroll
+        for (int dI = -2; dI <= 2; ++dI) {
+          const T cf = T(k1(PI, dI) * m1(PJ, dJ) + m1(PI, dI) * k1(PJ, dJ));
+          if (cf != T(0)) sl = fma(cf, X[dJ + 2][dI + 2], sl);
+        }
+#pragma unroll
+      for (int dj = -1; dj <= 1; ++dj)
+#pragma unroll
+        for (int di = -1; di <= 1; ++di) {
+          const T w = T(C == 0 ? ccol(2 + PI, 1 + di) * ncol(2 + PJ, 1 + dj)
+                               : ncol(2 + PI, 1 + di) * ccol(2 + PJ, 1 + dj));
+          if (w != T(0)) g = fma(w, P[dj + 1][di + 1], g);
+        }
+      v = level_cl<T>(L) * sl + level_cb<T>(L) * g;
+    }
+    y[k] = residual ? b[k] - v : v;
+  }
+}
+
+// rc = P^T rf at output (C, gy, gx) of coarse element (ex, ey); C = 2: its vertex
+template <typename T, int C, int GY, int GX>
+__device__ __forceinline__ void restrict_out(const LevelDev& F, const LevelDev& Co, const T* rf, T* rc, int ex,
+                                             int ey) {
+  if constexpr (C == 2) {
+    const T* pf = rf + 2 * F.nv;
+    T s = T(0);
+#pragma unroll
+    for (int dj = -1; dj <= 1; ++dj)
+#pragma unroll
+      for (int di = -1; di <= 1; ++di) {
+        const int fi = 2 * ex + di, fj = 2 * ey + dj;
+        if (fi < 0 || fj < 0 || fi >= F.np || fj >= F.np) continue;
+        s = fma(T((di == 0 ? 1.0 : 0.5) * (dj == 0 ? 1.0 : 0.5)), pf[static_cast<long long>(fj) * F.np + fi], s);
+      }
+    rc[2 * Co.nv + static_cast<long long>(ey) * Co.np + ex] = s;
+  } else {
+    const int cq = Co.nq, I = 2 * ex + GX, J = 2 * ey + GY;
+    if (I >= cq || J >= cq) return;
+    T acc = T(0);
+    if (is_free(I, J, cq)) {
+#pragma unroll
+      for (int k2 = 0; k2 < 7; ++k2) {
+        if (rw(GY, k2) == 0.0) continue;
+        T h = T(0);
+#pragma unroll
+        for (int k = 0; k < 7; ++k) {
+          if (rw(GX, k) == 0.0) continue;
+          const int Fi = 4 * ex - 3 + k, Fj = 4 * ey - 3 + k2;
+          const T v = is_free(Fi, Fj, F.nq) ? rf[C * F.nv + static_cast<long long>(Fj) * F.nq + Fi] : T(0);
+          h = fma(T(rw(GX, k)), v, h);
+        }
+        acc = fma(T(rw(GY, k2)), h, acc);
+      }
+    }
+    rc[C * Co.nv + static_cast<long long>(J) * cq + I] = acc;
+  }
+}
+
+// xf += P ec at fine Q2 node (4 ex + FX, 4 ey + FY) of component C; C = 2: at fine
+// vertex (2 ex + FX, 2 ey + FY), FX, FY < 2
+template <typename T, int C, int FY, int FX>
+__device__ __forceinline__ void prolong_out(const LevelDev& F, const LevelDev& Co, const T* ec, T* xf, int ex,
+                                            int ey) {
+  if constexpr (C == 2) {
+    const int I = 2 * ex + FX, J = 2 * ey + FY;
+    if (I >= F.np || J >= F.np) return;
+    const T* p = ec + 2 * Co.nv + static_cast<long long>(ey) * Co.np + ex;   // fx, fy = 1 stay inside the grid
+    T v = p[0];
+    if (FX == 1 && FY == 0) v = T(0.5) * (p[0] + p[1]);
+    if (FX == 0 && FY == 1) v = T(0.5) * (p[0] + p[Co.np]);
+    if (FX == 1 && FY == 1) v = T(0.25) * ((p[0] + p[1]) + (p[Co.np] + p[Co.np + 1]));
+    xf[2 * F.nv + static_cast<long long>(J) * F.np + I] += v;
+  } else {
+    const int cq = Co.nq, I = 4 * ex + FX, J = 4 * ey + FY;
+    if (!is_free(I, J, F.nq)) return;
+    T acc = T(0);
+#pragma unroll
+    for (int gy = 0; gy < 3; ++gy) {
+      if (pw(FY, gy) == 0.0) continue;
+      T h = T(0);
+#pragma unroll
+      for (int gx = 0; gx < 3; ++gx) {
+        if (pw(FX, gx) == 0.0) continue;
+        const int Ci = 2 * ex + gx, Cj = 2 * ey + gy;
+        const T v = is_free(Ci, Cj, cq) ? ec[C * Co.nv + static_cast<long long>(Cj) * cq + Ci] : T(0);
+        h = fma(T(pw(FX, gx)), v, h);
+      }
+      acc = fma(T(pw(FY, gy)), h, acc);
+    }
+    xf[C * F.nv + static_cast<long long>(J) * F.nq + I] += acc;
+  }
+}
+
 // e[row] = sum_k G[row][k] r[k] by one warp (lanes along the row, a fixed
 // shuffle tree: deterministic); r converted to double on the fly
 template <typename TR>

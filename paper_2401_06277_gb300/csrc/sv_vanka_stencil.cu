@@ -125,99 +125,95 @@ std::vector<long double> build_stencil() {
 // ---------------------------------------------------------------------------
 // One sweep from the residual r: x_out = x + omega (stencil r), Dirichlet rows
 // x + omega r (their patch rows are identities and every patch holding the node
-// adds r / m).  A CTA takes 8 x 4 cells and three of the nine outputs per cell,
-// one warp per output (so that loop bounds and coefficients are uniform in a warp
-// of interior cells), one lane per cell.  An output takes 81 x 2, 63 x 2 or 49 x 2
-// residuals and 9, 6 or 4 pressures (the patches holding the node), the pressure
-// 25 x 2 + 1.  Bound: the FP64 pipe (one warp instruction in 16 clocks per SM), on
-// the small levels by how evenly the outputs spread over the SMs, which is why
-// three CTAs share the outputs of a tile.
+// adds r / m).  An output takes 81 x 2, 63 x 2 or 49 x 2 residuals and 9, 6 or 4
+// pressures (the patches holding the node), the pressure 25 x 2 + 1.
+//
+// What bounds it is the FP64 pipe: a warp's FP64 instruction holds the unit of its
+// SM sub-partition for 64 clocks, so on the small levels the time is the longest
+// chain a warp runs, not the work.  Hence a warp takes one output kind of 4 x 2
+// cells with four lanes per output, each lane every fourth coefficient (at most 42
+// multiply-adds), summed by shuffles; three warps per CTA and three CTAs per tile
+// spread the nine outputs of a cell over the SMs.
 // ---------------------------------------------------------------------------
-constexpr int GX = 8, GY = 4, GW = GX + 4, GH = GY + 4;
+constexpr int GX = 4, GY = 2, GW = GX + 4, GH = GY + 4, PARTS = 4;
+static_assert(GX * GY * PARTS == 32, "a warp is one output kind of a tile");
 
-__global__ void __launch_bounds__(96) k_vanka_stencil(LevelDev L, const double* __restrict__ G,
-                                                      const double* __restrict__ x, const double* __restrict__ r,
-                                                      double* __restrict__ xo, double su, double sp, double rps,
-                                                      double omega) {
+template <typename T>
+struct Pair;
+template <>
+struct Pair<double> { using type = double2; };
+template <>
+struct Pair<float> { using type = float2; };
+
+template <typename T>
+__global__ void __launch_bounds__(96) k_vanka_stencil(LevelDev L, const T* __restrict__ G, const T* __restrict__ x,
+                                                      const T* __restrict__ r, T* __restrict__ xo, T su, T sp, T rps,
+                                                      T omega) {
+  using T2 = typename Pair<T>::type;
   pdl_begin();
-  __shared__ double V[2][2][2][GH][GW];   // [component][J parity][I parity][cell row][cell column]
-  __shared__ double P[GH][GW];            // (cl / cb) r_p
+  __shared__ T V[2][2 * GH][2 * GW];   // residual of the window's nodes, 0 off the free nodes
+  __shared__ T P[GH][GW];              // (cl / cb) r_p
   const int nq = L.nq, np = L.np, n = L.n;
   const long long nv = L.nv;
   const int i0 = GX * blockIdx.x, j0 = GY * blockIdx.y;
-  {
-    const int cx = threadIdx.x % GW, cy = threadIdx.x / GW;   // 96 threads: 12 x 8 cells
-    const int gi = i0 - 2 + cx, gj = j0 - 2 + cy;
-#pragma unroll
-    for (int PJ = 0; PJ < 2; ++PJ)
-#pragma unroll
-      for (int PI = 0; PI < 2; ++PI) {
-        const int I = 2 * gi + PI, J = 2 * gj + PJ;
-        const bool ok = is_free(I, J, nq);
-        const double* p = r + static_cast<long long>(J) * nq + I;
-        V[0][PJ][PI][cy][cx] = ok ? p[0] : 0.0;
-        V[1][PJ][PI][cy][cx] = ok ? p[nv] : 0.0;
-      }
-    P[cy][cx] = (gi >= 0 && gj >= 0 && gi <= n && gj <= n) ? rps * r[2 * nv + static_cast<long long>(gj) * np + gi] : 0.0;
+  for (int t = threadIdx.x; t < 4 * GW * GH; t += 96) {
+    const int c = t % (2 * GW), w = t / (2 * GW), I = 2 * (i0 - 2) + c, J = 2 * (j0 - 2) + w;
+    const bool ok = is_free(I, J, nq);
+    const long long k = static_cast<long long>(J) * nq + I;
+    V[0][w][c] = ok ? r[k] : T(0);
+    V[1][w][c] = ok ? r[nv + k] : T(0);
+  }
+  if (threadIdx.x < GW * GH) {
+    const int c = threadIdx.x % GW, w = threadIdx.x / GW, gi = i0 - 2 + c, gj = j0 - 2 + w;
+    const bool ok = gi >= 0 && gj >= 0 && gi <= n && gj <= n;
+    P[w][c] = ok ? rps * r[2 * nv + static_cast<long long>(gj) * np + gi] : T(0);
   }
   __syncthreads();
-  const int o = 3 * blockIdx.z + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  const int lx = lane & (GX - 1), ly = lane / GX, i = i0 + lx, j = j0 + ly;
+  const int o = 3 * blockIdx.z + (threadIdx.x >> 5), part = (threadIdx.x & 31) / (GX * GY);
+  const int lx = threadIdx.x % GX, ly = (threadIdx.x / GX) % GY, i = i0 + lx, j = j0 + ly;
   auto pos = [n](int a) { return a < 3 ? a : a <= n - 3 ? 3 : a >= n ? 6 : a - (n - 2) + 4; };
-  const double* g = G + static_cast<size_t>(pos(j) * VS_POS + pos(i)) * VS_TYPE + o * VS_OUT;
-  double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-  if (o < 8) {
-    const int c = o >> 2, py = (o >> 1) & 1, px = o & 1;
-    for (int J = 2 * py; J < 9; ++J) {
-      const double* v = &V[0][J & 1][0][ly + (J >> 1)][lx];
-      const double2* gj = reinterpret_cast<const double2*>(g + J * 18);
+  const T* g = G + static_cast<size_t>(pos(j) * VS_POS + pos(i)) * VS_TYPE + o * VS_OUT;
+  const T* v = &V[0][2 * ly][2 * lx];
+  T a0 = T(0), a1 = T(0);
+  auto node = [&](int J, int I) {
+    const T2 w = __ldg(reinterpret_cast<const T2*>(g) + J * 9 + I);
+    a0 = fma(w.x, v[J * 2 * GW + I], a0);
+    a1 = fma(w.y, v[4 * GW * GH + J * 2 * GW + I], a1);
+  };
+  const int py = (o >> 1) & 1, px = o & 1;
+  if (o == 8) {
 #pragma unroll
-      for (int I = 0; I < 9; ++I) {
-        if (I < 2 && px) continue;
-        const double2 w = __ldg(gj + I);
-        const double* vi = v + (I & 1) * (GH * GW) + (I >> 1);
-        if (I & 1) {
-          a2 = fma(w.x, vi[0], a2);
-          a3 = fma(w.y, vi[4 * GH * GW], a3);
-        } else {
-          a0 = fma(w.x, vi[0], a0);
-          a1 = fma(w.y, vi[4 * GH * GW], a1);
-        }
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < 9; ++k) {
-      const int dj = k / 3, di = k % 3;
-      if ((dj == 0 && py) || (di == 0 && px)) continue;   // the node's patches only
-      a0 = fma(__ldg(g + 162 + k), P[ly + 1 + dj][lx + 1 + di], a0);
-    }
-    const int I = 2 * i + px, J = 2 * j + py;
-    if (I >= nq || J >= nq) return;
-    const long long k = c * nv + static_cast<long long>(J) * nq + I;
-    const double xv = x != nullptr ? x[k] : 0.0;
-    xo[k] = is_free(I, J, nq) ? fma(su, (a0 + a1) + (a2 + a3), xv) : fma(omega, r[k], xv);
+    for (int e = part; e < 25; e += PARTS) node(2 + e / 5, 2 + e % 5);
+    if (part == 0) a0 = fma(__ldg(g + 162 + 4), P[ly + 2][lx + 2], a0);
   } else {
-#pragma unroll
-    for (int J = 2; J < 7; ++J) {
-      const double* v = &V[0][J & 1][0][ly + (J >> 1)][lx];
-      const double2* gj = reinterpret_cast<const double2*>(g + J * 18);
-#pragma unroll
-      for (int I = 2; I < 7; ++I) {
-        const double2 w = __ldg(gj + I);
-        const double* vi = v + (I & 1) * (GH * GW) + (I >> 1);
-        if (I & 1) {
-          a2 = fma(w.x, vi[0], a2);
-          a3 = fma(w.y, vi[4 * GH * GW], a3);
-        } else {
-          a0 = fma(w.x, vi[0], a0);
-          a1 = fma(w.y, vi[4 * GH * GW], a1);
-        }
-      }
+    const int cnt = (9 - 2 * py) * (9 - 2 * px);   // node columns 2 px .. 8, rows 2 py .. 8
+    if (px) {
+#pragma unroll 8
+      for (int e = part; e < cnt; e += PARTS) node(2 * py + e / 7, 2 + e % 7);
+    } else {
+#pragma unroll 8
+      for (int e = part; e < cnt; e += PARTS) node(2 * py + e / 9, e % 9);
     }
-    a0 = fma(__ldg(g + 162 + 4), P[ly + 2][lx + 2], a0);
+#pragma unroll
+    for (int k = part; k < 9; k += PARTS) {
+      const int dj = k / 3, di = k % 3;
+      if (dj >= py && di >= px) a1 = fma(__ldg(g + 162 + k), P[ly + 1 + dj][lx + 1 + di], a1);
+    }
+  }
+  T d = a0 + a1;
+  d += __shfl_xor_sync(0xffffffffu, d, 8);
+  d += __shfl_xor_sync(0xffffffffu, d, 16);
+  if (part != 0) return;
+  if (o == 8) {
     if (i > n || j > n) return;
     const long long k = 2 * nv + static_cast<long long>(j) * np + i;
-    xo[k] = fma(sp, (a0 + a1) + (a2 + a3), x != nullptr ? x[k] : 0.0);
+    xo[k] = fma(sp, d, x != nullptr ? x[k] : T(0));
+  } else {
+    const int I = 2 * i + px, J = 2 * j + py;
+    if (I >= nq || J >= nq) return;
+    const long long k = (o >> 2) * nv + static_cast<long long>(J) * nq + I;
+    const T xv = x != nullptr ? x[k] : T(0);
+    xo[k] = is_free(I, J, nq) ? fma(su, d, xv) : fma(omega, r[k], xv);
   }
 }
 
@@ -228,16 +224,22 @@ const std::vector<long double>& vanka_stencil() {
   return G;
 }
 
-void launch_vanka_stencil(const LevelDev& L, const double* G, const double* x, const double* b, double* xo,
-                          double omega, double* rscratch, cudaStream_t s) {
-  const double* r = b;
+template <typename T>
+void launch_vanka_stencil(const LevelDev& L, const T* G, const T* x, const T* b, T* xo, double omega, T* rscratch,
+                          cudaStream_t s) {
+  const T* r = b;
   if (x != nullptr) {
-    launch_apply<double>(L, x, b, rscratch, 1, s);
+    launch_apply<T>(L, x, b, rscratch, 1, s);
     r = rscratch;
   }
   count_launches(1);
-  launch_pdl(k_vanka_stencil, dim3((L.np + GX - 1) / GX, (L.np + GY - 1) / GY, 3), dim3(96), 0, s, L, G, x, r, xo,
-             omega / L.cl, omega / L.cb, L.cl / L.cb, omega);
+  launch_pdl(k_vanka_stencil<T>, dim3((L.np + GX - 1) / GX, (L.np + GY - 1) / GY, 3), dim3(96), 0, s, L, G, x, r, xo,
+             T(omega / L.cl), T(omega / L.cb), T(L.cl / L.cb), T(omega));
 }
+
+template void launch_vanka_stencil<double>(const LevelDev&, const double*, const double*, const double*, double*,
+                                           double, double*, cudaStream_t);
+template void launch_vanka_stencil<float>(const LevelDev&, const float*, const float*, const float*, float*, double,
+                                          float*, cudaStream_t);
 
 }  // namespace sv
