@@ -312,7 +312,7 @@ ZERO_GUESS_SHARE = 1.0 / 4.0
 # sweep configurations by stokes_level_tile: fused tiles of TX x TY vertices, or (4, 5; FP64
 # only) the split sweep: 16 x 16 own-patch solves writing the corrections, then the update
 # (5: compiled for two CTAs per SM)
-TILE_NAMES = ["8x8", "16x8", "16x16", "14x14", "split16x16", "split16x16x2", "4x4", "stencil"]
+TILE_NAMES = ["8x8", "16x8", "16x16", "14x14", "split16x16", "split16x16x2", "4x4", "stencil", "stencil-tc"]
 
 
 VC_REPS = 20   # graph replays of the bare V-cycle (median reported)

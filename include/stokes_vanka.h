@@ -76,8 +76,9 @@ typedef struct {
   int maxit;        /* FGMRES iteration cap                            (1000) */
   double rtol;      /* stop when ||b - A x|| <= rtol ||b - A x0||      (1e-8) */
   stokes_precision prec;  /*                                          (FP64) */
-  int tile;         /* Vanka sweep configuration: -1 = chosen per level by
-                       timing at creation; fused tiles of 0 = 8x8, 1 = 16x8,
+  int tile;         /* Vanka sweep configuration: -1 = chosen per level, in
+                       the FP64 form by its size (stokes_level_tile), in the
+                       mixed forms by timing at creation; fused tiles of 0 = 8x8, 1 = 16x8,
                        2 = 16x16, 3 = 14x14 vertices (mixed forms: 3 = the
                        strip sweep of the interior tiles where they fit --
                        BF16 tensor-core patch GEMMs, or FP32 patch solves --
@@ -175,7 +176,11 @@ stokes_status stokes_hierarchy_destroy(stokes_hierarchy* h);
 /* Number of levels L and the grid size n_l of level l (0 = coarsest). */
 stokes_status stokes_level_info(const stokes_hierarchy* h, int* num_levels, int* n_finest);
 stokes_status stokes_level_n(const stokes_hierarchy* h, int level, int* n_level);
-/* Sweep configuration used on a level (see stokes_params.tile).  In the mixed
+/* Sweep configuration used on a level (see stokes_params.tile).  With tile = -1 the
+ * FP64 form takes, on levels with sweeps, 7 (n < 96: the residual, then the sum of all
+ * patch solves as one stencil of FP64 dot products) or 8 (above: the same stencil as an
+ * exact integer contraction on the tensor cores); both are chosen by size only and are
+ * not values of stokes_params.tile.  In the mixed
  * forms, 3 on a level where the interior strips fit means the strip sweep
  * (tensor-core GEMMs in the BF16 form, FP32 patch solves in the FP32 form) with
  * its 14x14 SIMT ring; the autotuner may choose a SIMT shape (0..2, 6) there

@@ -107,7 +107,9 @@ void free_all(stokes_hierarchy* h) {
   h->bt_GL = h->bt_GM = h->bt_buf = nullptr;
   h->lv.clear();
   cudaFree(h->stencil_G);
+  cudaFree(h->stencil_digits);
   h->stencil_G = nullptr;
+  h->stencil_digits = nullptr;
   cudaFree(h->coarse_G);
   cudaFree(h->V);
   cudaFree(h->Z);
@@ -195,6 +197,9 @@ void sweep_f64(stokes_hierarchy* h, sv::Level& L, const double* x, const double*
     sv::launch_bs_sweep<double>(L.d, h->bs, static_cast<double*>(h->bs_buf), L.r, x, b, xo, h->stream);
   else if (h->prm.smoother == STOKES_SMOOTHER_PER_PATCH)
     sv::launch_simple_sweep(L.d, L.pinv, h->delta, L.r, x, b, xo, h->prm.omega, h->stream);
+  else if (L.vk_cfg == sv::VANKA_CFG_TC64)
+    sv::launch_vanka_tc64(L.d, h->stencil_digits, h->stencil_eu, h->stencil_ep, h->stencil_G, x, b, xo, h->prm.omega,
+                          L.r, h->dev_err, h->tc_wait_limit, h->stream);
   else if (L.vk_cfg == sv::VANKA_CFG_STENCIL)
     sv::launch_vanka_stencil<double>(L.d, h->stencil_G, x, b, xo, h->prm.omega, L.r, h->stream);
   else if (sv::vanka_cfg_split(L.vk_cfg))
@@ -792,7 +797,11 @@ cudaError_t tune_level(stokes_hierarchy* h, sv::Level& L, int* cfg) {
   return cudaGetLastError();
 }
 
-constexpr int STENCIL_MAX_N = 160;
+// The FP64 sweep by size: the composite stencil as FP64 dot products below TC64_MIN_N, as
+// the tensor-core contraction from there on.  One zero-guess sweep, FP64 dot products /
+// tensor cores (us): n = 64 17.5 / 33.2, 128 52.2 / 34.1; below, the contraction pays for
+// its prologue (91 KB of coefficients, the first window), above, FP64 for its rate.
+constexpr int TC64_MIN_N = 96;
 cudaError_t choose_tiles(stokes_hierarchy* h) {
   for (sv::Level& L : h->lv) {
     if (h->prm.tile >= 0 || h->prm.smoother != STOKES_SMOOTHER_SHARED || h->prm.precond == 1) {
@@ -806,7 +815,8 @@ cudaError_t choose_tiles(stokes_hierarchy* h) {
     // only the precision the V-cycle runs in is tuned (the FP64 sweep of a
     // mixed hierarchy serves stokes_vanka_sweep alone and keeps 16x8)
     cudaError_t e = cudaSuccess;
-    if (h->prm.prec == STOKES_FP64 && L.d.n >= sv::VS_MIN_N && L.d.n <= STENCIL_MAX_N) L.vk_cfg = sv::VANKA_CFG_STENCIL;
+    if (h->prm.prec == STOKES_FP64 && L.d.n >= sv::VS_MIN_N)
+      L.vk_cfg = (h->stencil_digits && L.d.n >= TC64_MIN_N) ? sv::VANKA_CFG_TC64 : sv::VANKA_CFG_STENCIL;
     else if (h->prm.prec == STOKES_FP64) e = tune_level<double>(h, L, &L.vk_cfg);
     else e = tune_level<float>(h, L, &L.vk_cfg_f);   // strip sweep vs SIMT shapes
     if (e != cudaSuccess) return e;
@@ -1033,6 +1043,17 @@ stokes_status stokes_hierarchy_create(int n, double viscosity, const stokes_para
       free_all(h);
       delete h;
       return cuda_fail(e, "composite stencil upload");
+    }
+    std::vector<unsigned char> dig;
+    if (sv::tc64_pack(dig, &h->stencil_eu, &h->stencil_ep)) {
+      e = dalloc(&h->stencil_digits, dig.size());
+      if (e == cudaSuccess) e = cudaMemcpy(h->stencil_digits, dig.data(), dig.size(), cudaMemcpyHostToDevice);
+      if (e == cudaSuccess) e = sv::vanka_tc64_prepare();
+      if (e != cudaSuccess) {
+        free_all(h);
+        delete h;
+        return cuda_fail(e, "stencil digits upload");
+      }
     }
   }
   const size_t Nf = static_cast<size_t>(h->lv.back().d.N);

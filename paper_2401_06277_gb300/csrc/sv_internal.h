@@ -225,6 +225,8 @@ struct stokes_hierarchy {
   sv::FastDiag fd;               // interior patch factors (level independent)
   sv::FastDiagT<float> fdf;      // the same in FP32
   double* stencil_G = nullptr;   // FP64 form: the composite Vanka stencil (VS_TAB doubles)
+  unsigned char* stencil_digits = nullptr;   // and its interior cell type as tensor-core digits
+  int stencil_eu = 0, stencil_ep = 0;        // exponents of the digits (tc64_pack)
   double* coarse_G = nullptr;    // N0 x N0 dense inverse of the bordered coarse system
   int N0 = 0;
   // FGMRES workspace
@@ -324,6 +326,7 @@ constexpr int VANKA_CFG_SPLIT = 4;   // FP64 only: own-patch solves + separate u
 constexpr int VANKA_CFG_SPLIT2 = 5;  // the same, compiled for two CTAs per SM (at most 128 registers)
 constexpr int VANKA_CFG_4 = 6;       // fused 4x4 tiles: small levels, spread over more SMs
 constexpr int VANKA_CFG_STENCIL = 7; // FP64 only: the residual, then the composite stencil (launch_vanka_stencil)
+constexpr int VANKA_CFG_TC64 = 8;    // FP64 only: the composite stencil on the tensor cores (launch_vanka_tc64)
 inline bool vanka_cfg_split(int cfg) { return cfg == VANKA_CFG_SPLIT || cfg == VANKA_CFG_SPLIT2; }
 template <typename R>
 void launch_vanka(const LevelDev& L, const R* cd, const FastDiagT<R>& fd, const R* x, const R* b, R* xo,
@@ -342,6 +345,17 @@ const std::vector<long double>& vanka_stencil();
 template <typename T>
 void launch_vanka_stencil(const LevelDev& L, const T* G, const T* x, const T* b, T* xo, double omega, T* rscratch,
                           cudaStream_t s);
+
+// The same sweep with the interior cells as an exact digit contraction on the tensor
+// cores (sv_vanka_tc64.cu).  Gp: the packed digits (TC64_BYTES, 16-byte aligned) and the
+// exponents of tc64_pack; Gd: the FP64 table (cells near the boundary); err: set to 1 if
+// a bounded device wait expired (wait_limit polls).
+constexpr int TC64_BYTES = 34 * 168 * 16 + 128;
+bool tc64_pack(std::vector<unsigned char>& out, int* eu, int* ep);
+cudaError_t vanka_tc64_prepare();
+void launch_vanka_tc64(const LevelDev& L, const unsigned char* Gp, int eu, int ep, const double* Gd, const double* x,
+                       const double* b, double* xo, double omega, double* rscratch, int* err, int wait_limit,
+                       cudaStream_t s);
 
 // Persistent coarse-level kernel (sv_vanka.cu): one cooperative launch of `grid`
 // CTAs runs the nops steps; err is set to 1 if a grid barrier gave up.
