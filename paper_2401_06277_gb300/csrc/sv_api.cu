@@ -110,6 +110,8 @@ void free_all(stokes_hierarchy* h) {
   cudaFree(h->stencil_digits);
   h->stencil_G = nullptr;
   h->stencil_digits = nullptr;
+  cudaFree(h->op_digits);
+  h->op_digits = nullptr;
   cudaFree(h->coarse_G);
   cudaFree(h->V);
   cudaFree(h->Z);
@@ -797,6 +799,9 @@ cudaError_t tune_level(stokes_hierarchy* h, sv::Level& L, int* cfg) {
   return cudaGetLastError();
 }
 
+// Levels whose FP64 operator is the tensor-core contraction (smaller ones: FP64, one
+// output per thread).
+constexpr int OP_TC64_MIN_N = 160;
 // The FP64 sweep by size: the composite stencil as FP64 dot products below TC64_MIN_N, as
 // the tensor-core contraction from there on.  One zero-guess sweep, FP64 dot products /
 // tensor cores (us): n = 64 17.5 / 33.2, 128 52.2 / 34.1; below, the contraction pays for
@@ -1068,6 +1073,22 @@ stokes_status stokes_hierarchy_create(int n, double viscosity, const stokes_para
     free_all(h);
     delete h;
     return cuda_fail(e, "Krylov workspace allocation");
+  }
+  if (n >= OP_TC64_MIN_N) {
+    std::vector<unsigned char> dig;
+    sv::apply_tc64_pack(dig);
+    if ((e = dalloc(&h->op_digits, dig.size())) != cudaSuccess ||
+        (e = cudaMemcpy(h->op_digits, dig.data(), dig.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
+        (e = sv::apply_tc64_prepare()) != cudaSuccess) {
+      free_all(h);
+      delete h;
+      return cuda_fail(e, "operator digits upload");
+    }
+    for (sv::Level& L : h->lv)
+      if (L.d.n >= OP_TC64_MIN_N) {
+        L.d.op_digits = h->op_digits;
+        L.d.dev_err = h->dev_err;
+      }
   }
   if ((e = tail_setup(h)) != cudaSuccess) {
     free_all(h);

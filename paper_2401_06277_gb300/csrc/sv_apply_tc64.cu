@@ -1,0 +1,387 @@
+// sv_apply_tc64.cu -- the FP64 operator and residual of the large levels as an exact
+// integer contraction on the tensor cores.
+//
+// The coefficients of the stencils are integers up to 512 (sv_stencil.cuh), exact in
+// FP16.  With x in 6 digits of 10 bits (sv_digits.cuh) a digit's products sum to less
+// than 2^20, so FP32 holds every sum exactly; the six sums of an output are added in
+// 64-bit integers and rounded once, where the FP64 kernel rounds after each of up to 31
+// multiply-adds.  The pressure enters the velocity rows scaled by cb / cl, so that one
+// contraction gives (A x) / cl.  The only loss is that of x, rounded to 58 bits below
+// the largest value of the 4 x 132 cells in reach: 2^-55 of it at most.
+//
+// Columns that the elimination drops (Dirichlet nodes, vertices outside the grid) read
+// as zero and every remaining row is the interior one, so one coefficient set serves
+// the whole grid; Dirichlet rows are the identity.  Cells with values that are not
+// finite in reach are recomputed in FP64, so that they spread as before.
+//
+// One step is two cell rows of a strip of 128: K = 12 cell offsets (dx -1..1, dy -1..2)
+// x 8 + 3 x 4 pressures, 8 MMAs (M = 128 cells, N = 2 rows x 9 outputs padded to 32) per
+// digit.  Bound: the instructions around the contraction (digits of 9 values, 54 sums
+// per cell: about 700 a vertex) and HBM, no longer the FP64 pipe (334 operations a
+// vertex at 2 per clock and SM).
+#include <cuda_fp16.h>
+#include <cuda_runtime.h>
+
+#include <cmath>
+#include <cstdint>
+#include <cstring>
+#include <vector>
+
+#include "sv_digits.cuh"
+#include "sv_internal.h"
+#include "sv_level_ops.cuh"
+#include "sv_stencil.cuh"
+#include "sv_tcgen05.cuh"
+
+namespace sv {
+namespace {
+
+using namespace tc;
+using namespace dig;
+using ops::is_free;
+
+constexpr int NB = 32, KSTEPS = 8;               // operand rows (16 a + o), MMAs per digit
+constexpr int CHUNK = NB * 16;
+constexpr int GBYTES = 2 * KSTEPS * CHUNK;
+constexpr int EDGE_WARPS = 2, EDGE_COLS = 8;     // FP64: columns past the last strip, if few
+constexpr int NT = 32 * (EPI_WARPS + SLICE_WARPS + 1 + EDGE_WARPS);
+
+struct SM {
+  static constexpr int RING = 0;                 // 3 row pairs
+  static constexpr int P = RING + 6 * ROWB;      // pressures of a step, two buffers
+  static constexpr int G = P + 2 * ROWB;
+  static constexpr int BAR = G + GBYTES;         // full[3], done[3], free[2], gload
+  static constexpr int MISC = BAR + 16 * 8;      // tmem slot, fail flag, 8 maxima, 4 exponents
+  static constexpr int BYTES = MISC + 4 * 16;
+  static_assert(G % 128 == 0 && BAR % 8 == 0, "shared memory");
+};
+
+constexpr uint32_t IDESC = (1u << 4) | (static_cast<uint32_t>(NB >> 3) << 17) | ((128u >> 4) << 24);
+
+struct Args {
+  LevelDev L;
+  const unsigned char* G;
+  const double* x;
+  const double* b;       // null: y = A x
+  double* y;
+  double ps;             // cb / cl
+  int strips;
+  int steps_per_seg;
+  int* err;
+  int wait_limit;
+};
+
+// FP64 cell, out of line: the slow path of cells with non-finite values in reach
+__device__ __noinline__ void apply_cell(const Args& A, int i, int j) {
+  ops::apply_vertex<double>(A.L, A.x, A.b, A.y, A.b != nullptr, i, j);
+}
+
+__global__ void __launch_bounds__(NT, 1) k_apply_tc64(const Args A) {
+  pdl_begin();
+  extern __shared__ __align__(1024) unsigned char sm[];
+  const LevelDev& L = A.L;
+  const int n = L.n, nq = L.nq, np = L.np;
+  const long long nv = L.nv;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const uint32_t s0 = su32(sm);
+  const uint32_t bar_full = s0 + SM::BAR, bar_done = bar_full + 24, bar_free = bar_done + 24, bar_g = bar_free + 16;
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(sm + SM::MISC);
+  volatile int* fail = reinterpret_cast<volatile int*>(sm + SM::MISC + 4);
+  int* smax = reinterpret_cast<int*>(sm + SM::MISC + 8);                    // 8 slots
+  volatile int* sexp = reinterpret_cast<volatile int*>(sm + SM::MISC + 40);   // 4 slots
+  const int i0 = COLS * static_cast<int>(blockIdx.x);
+  const int j0 = 2 * A.steps_per_seg * static_cast<int>(blockIdx.y);
+  const int rows = min(2 * A.steps_per_seg, n + 1 - j0);
+  const int S = (rows + 1) / 2;
+
+  if (tid == 0) {
+    for (int k = 0; k < 3; ++k) {
+      mbar_init(bar_full + 8 * k, SLICE_WARPS);
+      mbar_init(bar_done + 8 * k, 1);
+    }
+    mbar_init(bar_free, EPI_WARPS);
+    mbar_init(bar_free + 8, EPI_WARPS);
+    mbar_init(bar_g, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    *fail = 0;
+    for (int k = 0; k < 8; ++k) smax[k] = 0;
+  }
+  for (int k = tid; k < 2 * ROWB / 16; k += NT)   // channels 4..7 of the pressures stay zero
+    reinterpret_cast<uint4*>(sm + SM::P)[k] = make_uint4(0u, 0u, 0u, 0u);
+  fence_proxy();
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tslot)), "r"(512));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  fence_before();
+  __syncthreads();
+  fence_after();
+  const uint32_t tmem = *tslot;
+
+  if (warp < EPI_WARPS) {
+    // ---- accumulators to y: warp -> cell row a, lane quarter of the columns ----
+    const int a = warp >> 2, col = 32 * (warp & 3) + lane, i = i0 + col;
+    const uint32_t tq = tmem + (static_cast<uint32_t>(32 * (warp & 3)) << 16) + 16 * a;
+    for (int s = 0; s < S; ++s) {
+      const int j = j0 + 2 * s + a;
+      const bool own = i <= n && 2 * s + a < rows;
+      const long long ku = static_cast<long long>(2 * j) * nq + 2 * i;
+      const long long kp = 2 * nv + static_cast<long long>(j) * np + i;
+      const bool in1 = i < n, jn1 = j < n;   // the odd nodes exist
+      double bv[9];
+#pragma unroll
+      for (int o = 0; o < 9; ++o) bv[o] = 0.0;
+      if (own && A.b != nullptr) {
+#pragma unroll
+        for (int o = 0; o < 8; ++o)
+          if ((in1 || !(o & 1)) && (jn1 || !(o & 2))) bv[o] = A.b[(o >> 2) * nv + ku + ((o >> 1) & 1) * nq + (o & 1)];
+        bv[8] = A.b[kp];
+      }
+      bool ok = mbar_wait(bar_done + 8 * (s % 3), (s / 3) & 1, A.wait_limit);
+      ok = __all_sync(0xffffffffu, ok) && !*fail;
+      if (!ok) {
+        if (lane == 0) *fail = 1;
+        break;
+      }
+      fence_after();
+      long long hi[9], lo[9];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        uint32_t v[3][9];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) tmem_ld9(tq + 256 * (s & 1) + NB * (3 * h + c), v[c]);
+        wait_ld();
+#pragma unroll
+        for (int o = 0; o < 9; ++o) {
+          const int d0 = __float2int_rn(__uint_as_float(v[0][o])), d1 = __float2int_rn(__uint_as_float(v[1][o])),
+                    d2 = __float2int_rn(__uint_as_float(v[2][o]));
+          // |d| < 2^20: the first two fit 32 bits
+          const long long t = static_cast<long long>(d0 * 1024 + d1) * 1024 + d2;
+          if (h == 0) hi[o] = t;
+          else lo[o] = t;
+        }
+      }
+      fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar_free + 8 * (s & 1));
+      const int eb = sexp[s & 3];
+      if (own) {
+        if (eb == 0x7ff) {
+          apply_cell(A, i, j);
+          continue;
+        }
+        const double sc = exp_scale(eb, -48), su = L.cl * sc, sp = L.cb * sc;
+#pragma unroll
+        for (int o = 0; o < 9; ++o) {
+          const double d = static_cast<double>((hi[o] << 20) + ((lo[o] + 512) >> 10));
+          if (o == 8) {
+            A.y[kp] = A.b != nullptr ? fma(-sp, d, bv[8]) : sp * d;
+          } else if ((in1 || !(o & 1)) && (jn1 || !(o & 2))) {
+            const long long k = (o >> 2) * nv + ku + ((o >> 1) & 1) * nq + (o & 1);
+            if (is_free(2 * i + (o & 1), 2 * j + ((o >> 1) & 1), nq)) A.y[k] = A.b != nullptr ? fma(-su, d, bv[o]) : su * d;
+            else A.y[k] = A.b != nullptr ? bv[o] - A.x[k] : A.x[k];   // Dirichlet row: identity
+          }
+        }
+      }
+    }
+  } else if (warp < EPI_WARPS + SLICE_WARPS) {
+    // ---- values to digits: thread -> cell of the row pair ----
+    const int t = tid - 32 * EPI_WARPS;
+    const bool act = t < 2 * WCOLS;
+    const int a = t >= WCOLS ? 1 : 0, col = act ? t - a * WCOLS : 0, gi = i0 - 2 + col;
+    struct Cell {
+      double v[8];
+      double p[2];
+    };
+    auto load = [&](int q, Cell& c) {   // row pair q: cell rows j0 - 1 + 2 q + a; pressures j0 - 3 + 2 q + 2 a + {0, 1}
+      const int gj = j0 - 1 + 2 * q + a;
+#pragma unroll
+      for (int o = 0; o < 8; ++o) {
+        const int I = 2 * gi + (o & 1), J = 2 * gj + ((o >> 1) & 1);
+        c.v[o] = (act && is_free(I, J, nq)) ? A.x[(o >> 2) * nv + static_cast<long long>(J) * nq + I] : 0.0;
+      }
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const int pj = j0 - 3 + 2 * q + 2 * a + k;
+        c.p[k] = (act && q >= 1 && gi >= 0 && gi <= n && pj >= 0 && pj <= n)
+                     ? A.ps * A.x[2 * nv + static_cast<long long>(pj) * np + gi] : 0.0;
+      }
+    };
+    int eb = 0;
+    auto words = [&](const Cell& c, unsigned long long (&w)[8]) {
+#pragma unroll
+      for (int o = 0; o < 8; ++o) w[o] = static_cast<unsigned long long>(to_fixed(c.v[o], eb)) + digit_bias();
+    };
+    auto put = [&](int q, const unsigned long long (&w)[8]) {
+      if (!act) return;
+#pragma unroll
+      for (int j = 0; j < ND; ++j)
+        *reinterpret_cast<uint4*>(sm + SM::RING + (2 * (q % 3) + a) * ROWB + j * PLANE + col * 16) =
+            make_uint4(digit2(w[0], w[1], j), digit2(w[2], w[3], j), digit2(w[4], w[5], j), digit2(w[6], w[7], j));
+    };
+    Cell cur, nxt;
+    load(0, nxt);
+    bool ok = true;
+    for (int q = 0; q < S + 1 && ok; ++q) {
+      cur = nxt;
+      if (q + 1 < S + 1) load(q + 1, nxt);
+      int m = max(__double2hiint(cur.p[0]) & 0x7fffffff, __double2hiint(cur.p[1]) & 0x7fffffff);
+#pragma unroll
+      for (int o = 0; o < 8; ++o) m = max(m, __double2hiint(cur.v[o]) & 0x7fffffff);
+      m = __reduce_max_sync(0xffffffffu, m);
+      if (lane == 0) atomicMax(smax + (q & 7), m);
+      asm volatile("bar.sync 1, %0;" ::"n"(SLICE_T) : "memory");
+      if (t == 0) smax[(q + 3) & 7] = 0;
+      if (q < 1) continue;
+      const volatile int* vm = smax;
+      const int em = max(vm[q & 7], vm[(q - 1) & 7]) >> 20;   // |x| < 2^(em - 1022)
+      const int s = q - 1;
+      unsigned long long w[8];
+      const bool renew = s == 0 || em > eb || (eb - em > 3 && eb > EB_MIN);
+      if (renew) {   // uniform over the slicer warps: the other row pair again, with the new exponent
+        eb = min(max(em + 1, EB_MIN), 0x7ff);
+        if (s > 0) ok = mbar_wait(bar_done + 8 * ((s - 1) % 3), ((s - 1) / 3) & 1, A.wait_limit);
+        Cell c;
+        load(q - 1, c);
+        words(c, w);
+        put(q - 1, w);
+      } else if (s >= 2) {
+        ok = mbar_wait(bar_done + 8 * ((s - 2) % 3), ((s - 2) / 3) & 1, A.wait_limit);
+      }
+      if (t == 0) sexp[s & 3] = em < 0x7ff ? eb : 0x7ff;
+      words(cur, w);
+      unsigned long long wp[2];
+#pragma unroll
+      for (int k = 0; k < 2; ++k) wp[k] = static_cast<unsigned long long>(to_fixed(cur.p[k], eb)) + digit_bias();
+      if (ok) {
+        put(q, w);
+        if (act) {
+#pragma unroll
+          for (int j = 0; j < ND; ++j)
+            *reinterpret_cast<unsigned*>(sm + SM::P + (s & 1) * ROWB + j * PLANE + col * 16 + 4 * a) = digit2(wp[0], wp[1], j);
+        }
+      } else {
+        *fail = 1;
+      }
+      fence_proxy();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar_full + 8 * (s % 3));
+      // every slicer warp leaves at the same row pair: the named barrier counts them all
+      asm volatile("bar.sync 1, %0;" ::"n"(SLICE_T) : "memory");
+      ok = !*fail;
+    }
+  } else if (warp == EPI_WARPS + SLICE_WARPS) {
+    if (lane == 0) {
+      // ---- coefficients, then the MMAs ----
+      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar_g), "r"(GBYTES) : "memory");
+      asm volatile(
+          "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(s0 + SM::G),
+          "l"(A.G), "r"(GBYTES), "r"(bar_g)
+          : "memory");
+      bool ok = mbar_wait(bar_g, 0, A.wait_limit);
+      int issued = 0;
+      for (int s = 0; s < S && ok; ++s) {
+        ok = mbar_wait(bar_full + 8 * (s % 3), (s / 3) & 1, A.wait_limit);
+        const int use = s >> 1;
+        if (ok && use > 0) ok = mbar_wait(bar_free + 8 * (s & 1), (use - 1) & 1, A.wait_limit);
+        if (!ok || *fail) {
+          ok = false;
+          break;
+        }
+        fence_after();
+        const uint32_t g0 = s0 + SM::G;
+        const uint32_t pair[2] = {s0 + SM::RING + 2 * (s % 3) * ROWB, s0 + SM::RING + 2 * ((s + 1) % 3) * ROWB};
+#pragma unroll 1
+        for (int c = 0; c < ND; ++c) {
+          const uint32_t d = tmem + 256 * (s & 1) + NB * c, off = c * PLANE + 16;   // column of dx = -1
+          int k = 0;
+#pragma unroll
+          for (int b = 0; b < 4; ++b, ++k)   // cell rows dy = -1 .. 2, dx = (-1, 0)
+            mma_f16(d, umma_desc(pair[b >> 1] + (b & 1) * ROWB + off, 16, 128),
+                    umma_desc(g0 + 2 * k * CHUNK, CHUNK, 128), IDESC, k > 0);
+#pragma unroll
+          for (int b = 0; b < 2; ++b, ++k)   // dx = 1 of both rows of a pair
+            mma_f16(d, umma_desc(pair[b] + off + 32, ROWB, 128), umma_desc(g0 + 2 * k * CHUNK, CHUNK, 128), IDESC, 1);
+          const uint32_t pp = s0 + SM::P + (s & 1) * ROWB + off;
+#pragma unroll
+          for (int h = 0; h < 2; ++h, ++k)   // pressures, dx = (-1, 0) and (1, none)
+            mma_f16(d, umma_desc(pp + 32 * h, 16, 128), umma_desc(g0 + 2 * k * CHUNK, CHUNK, 128), IDESC, 1);
+        }
+        mma_commit(bar_done + 8 * (s % 3));
+        ++issued;
+      }
+      if (!ok) *fail = 1;
+      // every chain that was issued has completed before the operands and tensor memory go
+      if (issued > 0 && !mbar_wait(bar_done + 8 * ((issued - 1) % 3), ((issued - 1) / 3) & 1, TC_WAIT_LIMIT)) *fail = 1;
+      mbar_wait(bar_g, 0, TC_WAIT_LIMIT);
+    }
+    __syncwarp();
+  } else {
+    // ---- the columns past the last strip ----
+    const int c0 = COLS * A.strips, w = n + 1 - c0;
+    const int ctas = gridDim.x * gridDim.y, cta = blockIdx.y * gridDim.x + blockIdx.x;
+    const int e0 = ((warp - (EPI_WARPS + SLICE_WARPS + 1)) * ctas + cta) * 32 + lane;
+    for (int e = e0; w > 0 && e < w * (n + 1); e += EDGE_WARPS * ctas * 32) apply_cell(A, c0 + e % w, e / w);
+  }
+  __syncwarp();
+  fence_before();
+  __syncthreads();
+  fence_after();
+  if (tid == 0 && *fail) atomicExch(A.err, 1);
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
+}
+
+}  // namespace
+
+// The integer coefficients in the K order of the kernel's MMAs: row 16 a + o of the
+// operand is output o of cell row j + a.
+void apply_tc64_pack(std::vector<unsigned char>& out) {
+  out.assign(GBYTES, 0);
+  auto place = [&](int a, int o, int chunk, int ch, double v) {
+    const __half h = __float2half_rn(static_cast<float>(v));   // integers up to 512: exact
+    std::memcpy(out.data() + static_cast<size_t>(chunk) * CHUNK + (16 * a + o) * 16 + 2 * ch, &h, 2);
+  };
+  for (int a = 0; a < 2; ++a)
+    for (int o = 0; o < 9; ++o) {
+      const int c = o >> 2, py = (o >> 1) & 1, px = o & 1;
+      for (int dyi = 0; dyi < 4; ++dyi)
+        for (int dx = -1; dx <= 1; ++dx)
+          for (int ch = 0; ch < 8; ++ch) {
+            const int c2 = ch >> 2, I = 2 * dx + (ch & 1), J = 2 * (dyi - 1 - a) + ((ch >> 1) & 1);
+            double v = 0.0;
+            if (o == 8) {
+              v = c2 == 0 ? crow(I) * nrow(J) : nrow(I) * crow(J);
+            } else if (c2 == c) {
+              const int dI = I - px, dJ = J - py;
+              v = k1(px, dI) * m1(py, dJ) + m1(px, dI) * k1(py, dJ);
+            }
+            place(a, o, dx < 1 ? 2 * dyi + dx + 1 : 8 + dyi, ch, v);
+          }
+      if (o == 8) continue;
+      for (int k = 0; k < 4; ++k)        // pressure row j - 1 + k
+        for (int dx = -1; dx <= 1; ++dx) {
+          const int dj = k - 1 - a;
+          place(a, o, 12 + dx + 1, k,
+                c == 0 ? ccol(px, dx) * ncol(py, dj) : ncol(px, dx) * ccol(py, dj));
+        }
+    }
+}
+
+cudaError_t apply_tc64_prepare() {
+  return cudaFuncSetAttribute(k_apply_tc64, cudaFuncAttributeMaxDynamicSharedMemorySize, SM::BYTES);
+}
+
+void launch_apply_tc64(const LevelDev& L, const double* x, const double* b, double* y, cudaStream_t s) {
+  int dev = 0, sms = 152;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  // strips of 128 columns (a remainder of up to EDGE_COLS goes to the FP64 warps: n + 1 is
+  // one more than a multiple of 128 on most grids); each with its segments
+  const int rem = L.np % COLS, strips = L.np / COLS + (rem > EDGE_COLS ? 1 : 0), steps = (L.np + 1) / 2;
+  const int seg = segment_steps(strips, steps, sms, 3);
+  Args A{L, L.op_digits, x, b, y, L.cb / L.cl, strips, seg, L.dev_err, TC_WAIT_LIMIT};
+  count_launches(1);
+  launch_pdl(k_apply_tc64, dim3(strips, (steps + seg - 1) / seg), dim3(NT), SM::BYTES, s, A);
+}
+
+}  // namespace sv

@@ -1,0 +1,81 @@
+// sv_digits.cuh -- FP64 values as small integers for the FP16 tensor cores (the
+// exact contractions of sv_vanka_tc64.cu and sv_apply_tc64.cu).
+//
+// A strip of 128 cell columns (132 held) is walked two cell rows at a time.  The cells
+// in reach of a step share an exponent E: x = 2^(E - 58) q, |x| < 2^E, q an integer
+// written in ND = 6 balanced digits of 10 bits.  In shared memory a digit of a cell row
+// is a plane of 16 bytes per cell (the FP16 digits of its eight velocity values: Q2
+// nodes (2i + PI, 2j + PJ) of component c at 4 c + 2 PJ + PI), so the operand of the
+// cells shifted by (dx, dy) is the same memory at another start address.
+#pragma once
+
+#include <cuda_fp16.h>
+#include <cuda_runtime.h>
+
+#include <cstdint>
+#include <cstring>
+
+namespace sv {
+namespace dig {
+
+constexpr int COLS = 128, WCOLS = COLS + 4;      // owned and held cell columns
+constexpr int ND = 6;                            // digits of a value
+constexpr int PLANE = WCOLS * 16;                // one digit of one cell row
+constexpr int ROWB = ND * PLANE;                 // a cell row
+constexpr int EPI_WARPS = 8, SLICE_WARPS = 9;    // accumulators to results; values to digits
+constexpr int SLICE_T = 32 * SLICE_WARPS;
+static_assert(2 * WCOLS <= SLICE_T, "one thread per cell of a row pair");
+constexpr int EB_MIN = 200;                      // smallest exponent in use (E + 1022): scales stay normal
+
+// q = x 2^(58 - E) rounded to nearest, |x| < 2^E, eb = E + 1022
+__device__ __forceinline__ long long to_fixed(double x, int eb) {
+  const unsigned hi = __double2hiint(x), lo = __double2loint(x);
+  const int e = (hi >> 20) & 0x7ff, d = eb - e, sh = min(max(d, 0), 58);
+  const unsigned long long m = (static_cast<unsigned long long>((hi & 0xfffffu) | 0x100000u) << 32) | lo;
+  unsigned long long v = ((m << 10) + (1ull << (sh + 4))) >> (sh + 5);
+  if (e == 0 || d > 58) v = 0;   // subnormal, or below half a unit
+  return (hi >> 31) ? -static_cast<long long>(v) : static_cast<long long>(v);
+}
+
+constexpr unsigned long long digit_bias() {
+  unsigned long long b = 0;
+  for (int k = 0; k < ND; ++k) b |= 512ull << (10 * k);
+  return b;
+}
+
+// digit j (0 the highest) of two biased words as FP16 integers in [-512, 511]
+__device__ __forceinline__ unsigned digit2(unsigned long long a, unsigned long long b, int j) {
+  const int s = 10 * (ND - 1 - j);
+  const unsigned t = (static_cast<unsigned>(a >> s) & 0x3ffu) | ((static_cast<unsigned>(b >> s) & 0x3ffu) << 16) | 0x64006400u;
+  __half2 h;
+  memcpy(&h, &t, 4);
+  h = __hadd2(h, __half2half2(__ushort_as_half(0xE600)));   // -1536
+  unsigned u;
+  memcpy(&u, &h, 4);
+  return u;
+}
+
+// 2^(E + k) for eb = E + 1022; NaN for eb = 0x7ff (a value that is not finite)
+__device__ __forceinline__ double exp_scale(int eb, int k) {
+  return eb < 0x7ff ? __hiloint2double((eb + 1 + k) << 20, 0) : __hiloint2double(0x7ff80000, 0);
+}
+
+// Steps per segment of a strip.  A segment of k steps costs about k + extra (its first
+// window, its coefficients, its last results), the CTAs run one per SM: the split that
+// minimises waves x (k + extra), fewest CTAs first.
+inline int segment_steps(int strips, int steps, int sms, int extra) {
+  long long best = -1;
+  int seg = steps;
+  for (int nseg = 1; nseg <= steps; ++nseg) {
+    const int k = (steps + nseg - 1) / nseg, used = (steps + k - 1) / k;
+    const long long waves = (static_cast<long long>(strips) * used + sms - 1) / sms, cost = waves * (k + extra);
+    if (best < 0 || cost < best) {
+      best = cost;
+      seg = k;
+    }
+  }
+  return seg;
+}
+
+}  // namespace dig
+}  // namespace sv

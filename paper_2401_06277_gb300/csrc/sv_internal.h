@@ -132,6 +132,10 @@ struct LevelDev {
   // integer stencils (interior_unit_schur), 1 / s = zsinv
   double zs, zsinv;
   float zsf, zsinvf;
+  // levels whose FP64 operator runs on the tensor cores (sv_apply_tc64.cu): the packed
+  // integer coefficients, and the hierarchy's error flag; null elsewhere
+  const unsigned char* op_digits = nullptr;
+  int* dev_err = nullptr;
 };
 
 // cl and cb in the element type
@@ -227,6 +231,7 @@ struct stokes_hierarchy {
   double* stencil_G = nullptr;   // FP64 form: the composite Vanka stencil (VS_TAB doubles)
   unsigned char* stencil_digits = nullptr;   // and its interior cell type as tensor-core digits
   int stencil_eu = 0, stencil_ep = 0;        // exponents of the digits (tc64_pack)
+  unsigned char* op_digits = nullptr;        // integer coefficients of the tensor-core operator
   double* coarse_G = nullptr;    // N0 x N0 dense inverse of the bordered coarse system
   int N0 = 0;
   // FGMRES workspace
@@ -356,6 +361,12 @@ cudaError_t vanka_tc64_prepare();
 void launch_vanka_tc64(const LevelDev& L, const unsigned char* Gp, int eu, int ep, const double* Gd, const double* x,
                        const double* b, double* xo, double omega, double* rscratch, int* err, int wait_limit,
                        cudaStream_t s);
+
+// FP64 operator / residual (b null: y = A x) as an exact digit contraction on the tensor
+// cores (sv_apply_tc64.cu); launch_apply<double> takes it on levels with L.op_digits.
+void apply_tc64_pack(std::vector<unsigned char>& out);
+cudaError_t apply_tc64_prepare();
+void launch_apply_tc64(const LevelDev& L, const double* x, const double* b, double* y, cudaStream_t s);
 
 // Persistent coarse-level kernel (sv_vanka.cu): one cooperative launch of `grid`
 // CTAs runs the nops steps; err is set to 1 if a grid barrier gave up.

@@ -264,6 +264,12 @@ dim3 grid2(int nx, int ny, dim3 blk) {
 
 template <typename T>
 void launch_apply(const LevelDev& L, const T* x, const T* b, T* y, int residual, cudaStream_t s) {
+  if constexpr (sizeof(T) == 8) {
+    if (L.op_digits != nullptr) {
+      launch_apply_tc64(L, x, residual ? b : nullptr, y, s);
+      return;
+    }
+  }
   count_launches(1);
   if (L.np <= OUT_MAX_NP) {
     launch_pdl(k_apply_out<T>, out_grid(L.np, 9), dim3(32), 0, s, L, x, b, y, residual);

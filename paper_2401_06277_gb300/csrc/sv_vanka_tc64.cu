@@ -51,6 +51,7 @@
 #include <cstdint>
 #include <cstring>
 
+#include "sv_digits.cuh"
 #include "sv_internal.h"
 #include "sv_level_ops.cuh"
 #include "sv_stencil.cuh"
@@ -60,22 +61,18 @@ namespace sv {
 namespace {
 
 using namespace tc;
+using namespace dig;
 using ops::is_free;
 
-constexpr int COLS = 128, WCOLS = COLS + 4;      // owned and held cell columns
-constexpr int ND = 6, NG = 7;                    // digits of the residual and of the coefficients
+constexpr int NG = 7;                            // digits of the coefficients
 constexpr int NBLK = 24;                         // N columns per coefficient digit
 constexpr int GROWS = NBLK * NG;                 // 168 rows of the coefficient operand
 constexpr int KSTEPS = 17;
-constexpr int PLANE = WCOLS * 16;                // one digit of one cell row
-constexpr int ROWB = ND * PLANE;
 constexpr int CHUNK = GROWS * 16;                // 8 K-values of all coefficient rows
 constexpr int GBYTES = 2 * KSTEPS * CHUNK + 128; // + the rows a padded N reads past the end
 static_assert(GBYTES == TC64_BYTES, "size of the packed coefficients");
-constexpr int EPI_WARPS = 8, SLICE_WARPS = 9, RING_WARPS = 4;
-constexpr int SLICE_T = 32 * SLICE_WARPS;
+constexpr int RING_WARPS = 4;
 constexpr int NT = 32 * (EPI_WARPS + SLICE_WARPS + 1 + RING_WARPS);
-static_assert(2 * WCOLS <= SLICE_T, "one thread per cell of a row pair");
 
 struct SM {
   static constexpr int RING = 0;                         // 6 cell rows
@@ -91,34 +88,6 @@ __host__ __device__ constexpr int chain_n(int j) { return (NBLK * (NG - j) + 15)
 // instruction descriptor: D FP32, A and B FP16, both K-major, M = 128
 __host__ __device__ constexpr uint32_t idesc(int n) {
   return (1u << 4) | (static_cast<uint32_t>(n >> 3) << 17) | ((128u >> 4) << 24);
-}
-
-// q = x 2^(58 - E) rounded to nearest, |x| < 2^E, eb = E + 1022
-__device__ __forceinline__ long long to_fixed(double x, int eb) {
-  const unsigned hi = __double2hiint(x), lo = __double2loint(x);
-  const int e = (hi >> 20) & 0x7ff, d = eb - e, sh = min(max(d, 0), 58);
-  const unsigned long long m = (static_cast<unsigned long long>((hi & 0xfffffu) | 0x100000u) << 32) | lo;
-  unsigned long long v = ((m << 10) + (1ull << (sh + 4))) >> (sh + 5);
-  if (e == 0 || d > 58) v = 0;   // subnormal, or below half a unit
-  return (hi >> 31) ? -static_cast<long long>(v) : static_cast<long long>(v);
-}
-
-constexpr unsigned long long digit_bias() {
-  unsigned long long b = 0;
-  for (int k = 0; k < ND; ++k) b |= 512ull << (10 * k);
-  return b;
-}
-
-// digit j (0 the highest) of two biased words as FP16 integers in [-512, 511]
-__device__ __forceinline__ unsigned digit2(unsigned long long a, unsigned long long b, int j) {
-  const int s = 10 * (ND - 1 - j);
-  const unsigned t = (static_cast<unsigned>(a >> s) & 0x3ffu) | ((static_cast<unsigned>(b >> s) & 0x3ffu) << 16) | 0x64006400u;
-  __half2 h;
-  memcpy(&h, &t, 4);
-  h = __hadd2(h, __half2half2(__ushort_as_half(0xE600)));   // -1536
-  unsigned u;
-  memcpy(&u, &h, 4);
-  return u;
 }
 
 struct Args {
@@ -309,8 +278,7 @@ __global__ void __launch_bounds__(NT, 1) k_vanka_tc64(const Args A) {
         break;
       }
       const int eb = sexp[s & 3];
-      // 2^(E - 57); NaN where a residual of the window is not finite
-      const double sc = eb < 0x7ff ? __hiloint2double((eb - 56) << 20, 0) : __hiloint2double(0x7ff80000, 0);
+      const double sc = exp_scale(eb, -57);   // NaN where a residual of the window is not finite
       if (own) {
         const double qu = A.qu * sc, qp = A.qp * sc;
 #pragma unroll
@@ -375,9 +343,9 @@ __global__ void __launch_bounds__(NT, 1) k_vanka_tc64(const Args A) {
       const int em = max(vm[q & 7], max(vm[(q - 1) & 7], vm[(q - 2) & 7])) >> 20;   // |x| < 2^(em - 1022)
       const int s = q - 2;
       unsigned long long w[8];
-      const bool renew = s == 0 || em > eb || (eb - em > 3 && eb > 200);
+      const bool renew = s == 0 || em > eb || (eb - em > 3 && eb > EB_MIN);
       if (renew) {   // uniform over the slicer warps
-        eb = min(max(em + 1, 200), 0x7ff);
+        eb = min(max(em + 1, EB_MIN), 0x7ff);
         if (s > 0) ok = mbar_wait(bar_done + 8 * (ND - 1), (s - 1) & 1, A.wait_limit);
         for (int qq = q - 2; qq < q; ++qq) {
           Cell c;
@@ -541,20 +509,8 @@ void launch_vanka_tc64(const LevelDev& L, const unsigned char* Gp, int eu, int e
   int dev = 0, sms = 152;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  // strips of 128 columns; segments of a whole number of row pairs.  A segment of k steps
-  // costs about k + 4 (the first window, the coefficients, the last update), the CTAs run
-  // one per SM: the split that minimises waves x (k + 4), fewest CTAs first.
   const int cells = L.n - 5, strips = (cells + COLS - 1) / COLS, steps = (cells + 1) / 2;
-  long long best = -1;
-  int seg = steps;
-  for (int nseg = 1; nseg <= steps; ++nseg) {
-    const int k = (steps + nseg - 1) / nseg, used = (steps + k - 1) / k;
-    const long long waves = (static_cast<long long>(strips) * used + sms - 1) / sms, cost = waves * (k + 4);
-    if (best < 0 || cost < best) {
-      best = cost;
-      seg = k;
-    }
-  }
+  const int seg = segment_steps(strips, steps, sms, 4);
   Args A{L, Gp, Gd, x, r, xo, omega / L.cl, omega / L.cb, std::ldexp(omega / L.cl, eu), std::ldexp(omega / L.cb, ep),
          L.cl / L.cb, omega, seg, err, wait_limit};
   count_launches(1);
