@@ -108,6 +108,8 @@ void free_all(stokes_hierarchy* h) {
   h->lv.clear();
   cudaFree(h->stencil_G);
   cudaFree(h->stencil_digits);
+  cudaFree(h->stencil_ring);
+  h->stencil_ring = nullptr;
   h->stencil_G = nullptr;
   h->stencil_digits = nullptr;
   cudaFree(h->op_digits);
@@ -200,7 +202,7 @@ void sweep_f64(stokes_hierarchy* h, sv::Level& L, const double* x, const double*
   else if (h->prm.smoother == STOKES_SMOOTHER_PER_PATCH)
     sv::launch_simple_sweep(L.d, L.pinv, h->delta, L.r, x, b, xo, h->prm.omega, h->stream);
   else if (L.vk_cfg == sv::VANKA_CFG_TC64)
-    sv::launch_vanka_tc64(L.d, h->stencil_digits, h->stencil_eu, h->stencil_ep, h->stencil_G, x, b, xo, h->prm.omega,
+    sv::launch_vanka_tc64(L.d, h->stencil_digits, h->stencil_eu, h->stencil_ep, h->stencil_ring, x, b, xo, h->prm.omega,
                           L.r, h->dev_err, h->tc_wait_limit, h->stream);
   else if (L.vk_cfg == sv::VANKA_CFG_STENCIL)
     sv::launch_vanka_stencil<double>(L.d, h->stencil_G, x, b, xo, h->prm.omega, L.r, h->stream);
@@ -1053,6 +1055,10 @@ stokes_status stokes_hierarchy_create(int n, double viscosity, const stokes_para
     if (sv::tc64_pack(dig, &h->stencil_eu, &h->stencil_ep)) {
       e = dalloc(&h->stencil_digits, dig.size());
       if (e == cudaSuccess) e = cudaMemcpy(h->stencil_digits, dig.data(), dig.size(), cudaMemcpyHostToDevice);
+      const std::vector<double> ring = sv::vanka_ring_table();
+      if (e == cudaSuccess) e = dalloc(&h->stencil_ring, ring.size());
+      if (e == cudaSuccess)
+        e = cudaMemcpy(h->stencil_ring, ring.data(), ring.size() * sizeof(double), cudaMemcpyHostToDevice);
       if (e == cudaSuccess) e = sv::vanka_tc64_prepare();
       if (e != cudaSuccess) {
         free_all(h);

@@ -71,9 +71,89 @@ struct Args {
   int wait_limit;
 };
 
-// FP64 cell, out of line: the slow path of cells with non-finite values in reach
-__device__ __noinline__ void apply_cell(const Args& A, int i, int j) {
-  ops::apply_vertex<double>(A.L, A.x, A.b, A.y, A.b != nullptr, i, j);
+// Output o of cell (i, j) in FP64, out of line: the columns past the last strip and the
+// cells with non-finite values in reach
+__device__ __noinline__ void apply_cell(const Args& A, int i, int j, int o) {
+  const int res = A.b != nullptr;
+  switch (o) {
+    case 0: ops::apply_out<double, 0, 0, 0>(A.L, A.x, A.b, A.y, res, i, j); break;
+    case 1: ops::apply_out<double, 0, 0, 1>(A.L, A.x, A.b, A.y, res, i, j); break;
+    case 2: ops::apply_out<double, 0, 1, 0>(A.L, A.x, A.b, A.y, res, i, j); break;
+    case 3: ops::apply_out<double, 0, 1, 1>(A.L, A.x, A.b, A.y, res, i, j); break;
+    case 4: ops::apply_out<double, 1, 0, 0>(A.L, A.x, A.b, A.y, res, i, j); break;
+    case 5: ops::apply_out<double, 1, 0, 1>(A.L, A.x, A.b, A.y, res, i, j); break;
+    case 6: ops::apply_out<double, 1, 1, 0>(A.L, A.x, A.b, A.y, res, i, j); break;
+    case 7: ops::apply_out<double, 1, 1, 1>(A.L, A.x, A.b, A.y, res, i, j); break;
+    default: ops::apply_out<double, 2, 0, 0>(A.L, A.x, A.b, A.y, res, i, j); break;
+  }
+}
+
+struct Shared {   // what the roles of a CTA share
+  uint32_t full, done, free, tmem;
+  volatile int* fail;
+  volatile int* sexp;
+  int i0, j0, rows, S;
+};
+
+// Accumulators to y for the outputs O0 .. O0 + NO - 1: warp -> cell row a and lane
+// quarter of the columns.
+template <int O0, int NO>
+__device__ __forceinline__ void epilogue(const Args& A, const Shared& C, int warp, int lane) {
+  const LevelDev& L = A.L;
+  const int n = L.n, nq = L.nq, np = L.np;
+  const long long nv = L.nv;
+  const int a = (warp >> 2) & 1, i = C.i0 + 32 * (warp & 3) + lane;
+  const uint32_t tq = C.tmem + (static_cast<uint32_t>(32 * (warp & 3)) << 16) + 16 * a + O0;
+  for (int s = 0; s < C.S; ++s) {
+    const int j = C.j0 + 2 * s + a;
+    const bool own = i <= n && 2 * s + a < C.rows;
+    const long long ku = static_cast<long long>(2 * j) * nq + 2 * i;
+    const long long kp = 2 * nv + static_cast<long long>(j) * np + i;
+    auto at = [&](int o) { return o == 8 ? kp : (o >> 2) * nv + ku + ((o >> 1) & 1) * nq + (o & 1); };
+    auto exists = [&](int o) { return own && (o == 8 || ((i < n || !(o & 1)) && (j < n || !(o & 2)))); };
+    double bv[NO];
+#pragma unroll
+    for (int o = 0; o < NO; ++o) bv[o] = exists(O0 + o) && A.b != nullptr ? A.b[at(O0 + o)] : 0.0;
+    const bool ok = mbar_wait_or_fail(C.done + 8 * (s % 3), (s / 3) & 1, A.wait_limit, C.fail);
+    if (!__all_sync(0xffffffffu, ok)) return;
+    fence_after();
+    long long hi[NO], lo[NO];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      uint32_t v[3][NO];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) tmem_ldn<NO>(tq + 256 * (s & 1) + NB * (3 * h + c), v[c]);
+      wait_ld();
+#pragma unroll
+      for (int o = 0; o < NO; ++o) {
+        const int d0 = __float2int_rn(__uint_as_float(v[0][o])), d1 = __float2int_rn(__uint_as_float(v[1][o])),
+                  d2 = __float2int_rn(__uint_as_float(v[2][o]));
+        // |d| < 2^20: the first two fit 32 bits
+        const long long t = static_cast<long long>(d0 * 1024 + d1) * 1024 + d2;
+        if (h == 0) hi[o] = t;
+        else lo[o] = t;
+      }
+    }
+    fence_before();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(C.free + 8 * (s & 1));
+    const int eb = C.sexp[s & 3];
+    if (eb == 0x7ff) {
+      if (own)
+        for (int o = 0; o < NO; ++o) apply_cell(A, i, j, O0 + o);
+      continue;
+    }
+    const double sc = exp_scale(eb, -58), su = L.cl * sc, sp = L.cb * sc;
+#pragma unroll
+    for (int o = 0; o < NO; ++o) {
+      const int oo = O0 + o;
+      if (!exists(oo)) continue;
+      const double d = to_double(hi[o], lo[o]), f = oo == 8 ? sp : su;
+      const long long k = at(oo);
+      if (oo == 8 || is_free(2 * i + (oo & 1), 2 * j + ((oo >> 1) & 1), nq)) A.y[k] = fma(A.b != nullptr ? -f : f, d, bv[o]);
+      else A.y[k] = A.b != nullptr ? bv[o] - A.x[k] : A.x[k];   // Dirichlet row: identity
+    }
+  }
 }
 
 __global__ void __launch_bounds__(NT, 1) k_apply_tc64(const Args A) {
@@ -118,72 +198,11 @@ __global__ void __launch_bounds__(NT, 1) k_apply_tc64(const Args A) {
   fence_after();
   const uint32_t tmem = *tslot;
 
-  if (warp < EPI_WARPS) {
-    // ---- accumulators to y: warp -> cell row a, lane quarter of the columns ----
-    const int a = warp >> 2, col = 32 * (warp & 3) + lane, i = i0 + col;
-    const uint32_t tq = tmem + (static_cast<uint32_t>(32 * (warp & 3)) << 16) + 16 * a;
-    for (int s = 0; s < S; ++s) {
-      const int j = j0 + 2 * s + a;
-      const bool own = i <= n && 2 * s + a < rows;
-      const long long ku = static_cast<long long>(2 * j) * nq + 2 * i;
-      const long long kp = 2 * nv + static_cast<long long>(j) * np + i;
-      const bool in1 = i < n, jn1 = j < n;   // the odd nodes exist
-      double bv[9];
-#pragma unroll
-      for (int o = 0; o < 9; ++o) bv[o] = 0.0;
-      if (own && A.b != nullptr) {
-#pragma unroll
-        for (int o = 0; o < 8; ++o)
-          if ((in1 || !(o & 1)) && (jn1 || !(o & 2))) bv[o] = A.b[(o >> 2) * nv + ku + ((o >> 1) & 1) * nq + (o & 1)];
-        bv[8] = A.b[kp];
-      }
-      bool ok = mbar_wait(bar_done + 8 * (s % 3), (s / 3) & 1, A.wait_limit);
-      ok = __all_sync(0xffffffffu, ok) && !*fail;
-      if (!ok) {
-        if (lane == 0) *fail = 1;
-        break;
-      }
-      fence_after();
-      long long hi[9], lo[9];
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        uint32_t v[3][9];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) tmem_ld9(tq + 256 * (s & 1) + NB * (3 * h + c), v[c]);
-        wait_ld();
-#pragma unroll
-        for (int o = 0; o < 9; ++o) {
-          const int d0 = __float2int_rn(__uint_as_float(v[0][o])), d1 = __float2int_rn(__uint_as_float(v[1][o])),
-                    d2 = __float2int_rn(__uint_as_float(v[2][o]));
-          // |d| < 2^20: the first two fit 32 bits
-          const long long t = static_cast<long long>(d0 * 1024 + d1) * 1024 + d2;
-          if (h == 0) hi[o] = t;
-          else lo[o] = t;
-        }
-      }
-      fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(bar_free + 8 * (s & 1));
-      const int eb = sexp[s & 3];
-      if (own) {
-        if (eb == 0x7ff) {
-          apply_cell(A, i, j);
-          continue;
-        }
-        const double sc = exp_scale(eb, -48), su = L.cl * sc, sp = L.cb * sc;
-#pragma unroll
-        for (int o = 0; o < 9; ++o) {
-          const double d = static_cast<double>((hi[o] << 20) + ((lo[o] + 512) >> 10));
-          if (o == 8) {
-            A.y[kp] = A.b != nullptr ? fma(-sp, d, bv[8]) : sp * d;
-          } else if ((in1 || !(o & 1)) && (jn1 || !(o & 2))) {
-            const long long k = (o >> 2) * nv + ku + ((o >> 1) & 1) * nq + (o & 1);
-            if (is_free(2 * i + (o & 1), 2 * j + ((o >> 1) & 1), nq)) A.y[k] = A.b != nullptr ? fma(-su, d, bv[o]) : su * d;
-            else A.y[k] = A.b != nullptr ? bv[o] - A.x[k] : A.x[k];   // Dirichlet row: identity
-          }
-        }
-      }
-    }
+  const Shared C{bar_full, bar_done, bar_free, tmem, fail, sexp, i0, j0, rows, S};
+  if (warp < EPI_WARPS / 2) {
+    epilogue<0, EPI_SPLIT>(A, C, warp, lane);
+  } else if (warp < EPI_WARPS) {
+    epilogue<EPI_SPLIT, 9 - EPI_SPLIT>(A, C, warp, lane);
   } else if (warp < EPI_WARPS + SLICE_WARPS) {
     // ---- values to digits: thread -> cell of the row pair ----
     const int t = tid - 32 * EPI_WARPS;
@@ -204,7 +223,7 @@ __global__ void __launch_bounds__(NT, 1) k_apply_tc64(const Args A) {
       for (int k = 0; k < 2; ++k) {
         const int pj = j0 - 3 + 2 * q + 2 * a + k;
         c.p[k] = (act && q >= 1 && gi >= 0 && gi <= n && pj >= 0 && pj <= n)
-                     ? A.ps * A.x[2 * nv + static_cast<long long>(pj) * np + gi] : 0.0;
+                     ? A.x[2 * nv + static_cast<long long>(pj) * np + gi] : 0.0;
       }
     };
     int eb = 0;
@@ -219,12 +238,11 @@ __global__ void __launch_bounds__(NT, 1) k_apply_tc64(const Args A) {
         *reinterpret_cast<uint4*>(sm + SM::RING + (2 * (q % 3) + a) * ROWB + j * PLANE + col * 16) =
             make_uint4(digit2(w[0], w[1], j), digit2(w[2], w[3], j), digit2(w[4], w[5], j), digit2(w[6], w[7], j));
     };
-    Cell cur, nxt;
-    load(0, nxt);
-    bool ok = true;
-    for (int q = 0; q < S + 1 && ok; ++q) {
-      cur = nxt;
-      if (q + 1 < S + 1) load(q + 1, nxt);
+    Cell cur;
+    load(0, cur);
+    for (int q = 0; q < S + 1; ++q) {
+      cur.p[0] *= A.ps;
+      cur.p[1] *= A.ps;
       int m = max(__double2hiint(cur.p[0]) & 0x7fffffff, __double2hiint(cur.p[1]) & 0x7fffffff);
 #pragma unroll
       for (int o = 0; o < 8; ++o) m = max(m, __double2hiint(cur.v[o]) & 0x7fffffff);
@@ -232,7 +250,10 @@ __global__ void __launch_bounds__(NT, 1) k_apply_tc64(const Args A) {
       if (lane == 0) atomicMax(smax + (q & 7), m);
       asm volatile("bar.sync 1, %0;" ::"n"(SLICE_T) : "memory");
       if (t == 0) smax[(q + 3) & 7] = 0;
-      if (q < 1) continue;
+      if (q < 1) {
+        load(q + 1, cur);
+        continue;
+      }
       const volatile int* vm = smax;
       const int em = max(vm[q & 7], vm[(q - 1) & 7]) >> 20;   // |x| < 2^(em - 1022)
       const int s = q - 1;
@@ -240,88 +261,86 @@ __global__ void __launch_bounds__(NT, 1) k_apply_tc64(const Args A) {
       const bool renew = s == 0 || em > eb || (eb - em > 3 && eb > EB_MIN);
       if (renew) {   // uniform over the slicer warps: the other row pair again, with the new exponent
         eb = min(max(em + 1, EB_MIN), 0x7ff);
-        if (s > 0) ok = mbar_wait(bar_done + 8 * ((s - 1) % 3), ((s - 1) / 3) & 1, A.wait_limit);
+        if (s > 0) mbar_wait_or_fail(bar_done + 8 * ((s - 1) % 3), ((s - 1) / 3) & 1, A.wait_limit, fail);
         Cell c;
         load(q - 1, c);
         words(c, w);
         put(q - 1, w);
-      } else if (s >= 2) {
-        ok = mbar_wait(bar_done + 8 * ((s - 2) % 3), ((s - 2) / 3) & 1, A.wait_limit);
       }
       if (t == 0) sexp[s & 3] = em < 0x7ff ? eb : 0x7ff;
       words(cur, w);
       unsigned long long wp[2];
 #pragma unroll
       for (int k = 0; k < 2; ++k) wp[k] = static_cast<unsigned long long>(to_fixed(cur.p[k], eb)) + digit_bias();
-      if (ok) {
-        put(q, w);
-        if (act) {
+      if (q + 1 < S + 1) load(q + 1, cur);   // in flight while the planes are written
+      // the row pair's slot and the pressure buffer are free once step s - 2 has read them
+      // (after a failed wait the results are void and only the arrivals matter)
+      if (!renew && s >= 2) mbar_wait_or_fail(bar_done + 8 * ((s - 2) % 3), ((s - 2) / 3) & 1, A.wait_limit, fail);
+      put(q, w);
+      if (act) {
 #pragma unroll
-          for (int j = 0; j < ND; ++j)
-            *reinterpret_cast<unsigned*>(sm + SM::P + (s & 1) * ROWB + j * PLANE + col * 16 + 4 * a) = digit2(wp[0], wp[1], j);
-        }
-      } else {
-        *fail = 1;
+        for (int j = 0; j < ND; ++j)
+          *reinterpret_cast<unsigned*>(sm + SM::P + (s & 1) * ROWB + j * PLANE + col * 16 + 4 * a) = digit2(wp[0], wp[1], j);
       }
       fence_proxy();
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_full + 8 * (s % 3));
-      // every slicer warp leaves at the same row pair: the named barrier counts them all
-      asm volatile("bar.sync 1, %0;" ::"n"(SLICE_T) : "memory");
-      ok = !*fail;
     }
   } else if (warp == EPI_WARPS + SLICE_WARPS) {
-    if (lane == 0) {
-      // ---- coefficients, then the MMAs ----
+    // ---- coefficients, then the MMAs ----
+    const uint32_t on = elect_one();
+    if (on) {
       asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar_g), "r"(GBYTES) : "memory");
       asm volatile(
           "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(s0 + SM::G),
           "l"(A.G), "r"(GBYTES), "r"(bar_g)
           : "memory");
-      bool ok = mbar_wait(bar_g, 0, A.wait_limit);
-      int issued = 0;
-      for (int s = 0; s < S && ok; ++s) {
-        ok = mbar_wait(bar_full + 8 * (s % 3), (s / 3) & 1, A.wait_limit);
-        const int use = s >> 1;
-        if (ok && use > 0) ok = mbar_wait(bar_free + 8 * (s & 1), (use - 1) & 1, A.wait_limit);
-        if (!ok || *fail) {
-          ok = false;
-          break;
-        }
-        fence_after();
-        const uint32_t g0 = s0 + SM::G;
-        const uint32_t pair[2] = {s0 + SM::RING + 2 * (s % 3) * ROWB, s0 + SM::RING + 2 * ((s + 1) % 3) * ROWB};
-#pragma unroll 1
-        for (int c = 0; c < ND; ++c) {
-          const uint32_t d = tmem + 256 * (s & 1) + NB * c, off = c * PLANE + 16;   // column of dx = -1
-          int k = 0;
-#pragma unroll
-          for (int b = 0; b < 4; ++b, ++k)   // cell rows dy = -1 .. 2, dx = (-1, 0)
-            mma_f16(d, umma_desc(pair[b >> 1] + (b & 1) * ROWB + off, 16, 128),
-                    umma_desc(g0 + 2 * k * CHUNK, CHUNK, 128), IDESC, k > 0);
-#pragma unroll
-          for (int b = 0; b < 2; ++b, ++k)   // dx = 1 of both rows of a pair
-            mma_f16(d, umma_desc(pair[b] + off + 32, ROWB, 128), umma_desc(g0 + 2 * k * CHUNK, CHUNK, 128), IDESC, 1);
-          const uint32_t pp = s0 + SM::P + (s & 1) * ROWB + off;
-#pragma unroll
-          for (int h = 0; h < 2; ++h, ++k)   // pressures, dx = (-1, 0) and (1, none)
-            mma_f16(d, umma_desc(pp + 32 * h, 16, 128), umma_desc(g0 + 2 * k * CHUNK, CHUNK, 128), IDESC, 1);
-        }
-        mma_commit(bar_done + 8 * (s % 3));
-        ++issued;
-      }
-      if (!ok) *fail = 1;
-      // every chain that was issued has completed before the operands and tensor memory go
-      if (issued > 0 && !mbar_wait(bar_done + 8 * ((issued - 1) % 3), ((issued - 1) / 3) & 1, TC_WAIT_LIMIT)) *fail = 1;
-      mbar_wait(bar_g, 0, TC_WAIT_LIMIT);
     }
+    __syncwarp();
+    auto wait = [&](uint32_t bar, uint32_t phase) {   // a vote, so that the loop stays uniform
+      return __all_sync(0xffffffffu, mbar_wait_or_fail(bar, phase, A.wait_limit, fail)) != 0;
+    };
+    bool ok = wait(bar_g, 0);
+    int issued = 0;
+    for (int s = 0; s < S && ok; ++s) {
+      ok = wait(bar_full + 8 * (s % 3), (s / 3) & 1);
+      const int use = s >> 1;
+      if (ok && use > 0) ok = wait(bar_free + 8 * (s & 1), (use - 1) & 1);
+      if (!ok) break;
+      fence_after();
+      const uint32_t gl = desc_lo(s0 + SM::G, CHUNK), pl = desc_lo(s0 + SM::P + (s & 1) * ROWB + 16, 16);
+      const uint32_t rl = desc_lo(s0 + SM::RING + 16, 16), r2 = desc_lo(s0 + SM::RING + 48, ROWB);
+      const uint32_t us = s, pair[2] = {us % 3 * (ROWB / 8), (us + 1) % 3 * (ROWB / 8)};   // units of 16 bytes
+#pragma unroll 1
+      for (int c = 0; c < ND; ++c) {
+        const uint32_t d = tmem + 256 * (s & 1) + NB * c, off = c * (PLANE / 16);
+        int k = 0;
+#pragma unroll
+        for (int b = 0; b < 4; ++b, ++k)   // cell rows dy = -1 .. 2, dx = (-1, 0)
+          mma_f16(on, d, rl + off + pair[b >> 1] + (b & 1) * (ROWB / 16), gl + k * (CHUNK / 8), IDESC, k > 0);
+#pragma unroll
+        for (int b = 0; b < 2; ++b, ++k)   // dx = 1 of both rows of a pair
+          mma_f16(on, d, r2 + off + pair[b], gl + k * (CHUNK / 8), IDESC, 1);
+#pragma unroll
+        for (int e = 0; e < 2; ++e, ++k)   // pressures, dx = (-1, 0) and (1, none)
+          mma_f16(on, d, pl + off + 2 * e, gl + k * (CHUNK / 8), IDESC, 1);
+      }
+      mma_commit(on, bar_done + 8 * (s % 3));
+      ++issued;
+    }
+    // every chain that was issued has completed before the operands and tensor memory go
+    if (issued > 0 && !mbar_wait(bar_done + 8 * ((issued - 1) % 3), ((issued - 1) / 3) & 1, TC_WAIT_LIMIT)) *fail = 1;
+    mbar_wait(bar_g, 0, TC_WAIT_LIMIT);
     __syncwarp();
   } else {
     // ---- the columns past the last strip ----
     const int c0 = COLS * A.strips, w = n + 1 - c0;
     const int ctas = gridDim.x * gridDim.y, cta = blockIdx.y * gridDim.x + blockIdx.x;
-    const int e0 = ((warp - (EPI_WARPS + SLICE_WARPS + 1)) * ctas + cta) * 32 + lane;
-    for (int e = e0; w > 0 && e < w * (n + 1); e += EDGE_WARPS * ctas * 32) apply_cell(A, c0 + e % w, e / w);
+    const int units = w > 0 ? 9 * ((w * (n + 1) + 31) / 32) : 0;   // 32 cells and one output
+    for (int u = (warp - (EPI_WARPS + SLICE_WARPS + 1)) * ctas + cta; u < units; u += EDGE_WARPS * ctas) {
+      const int e = (u / 9) * 32 + lane;
+      if (e < w * (n + 1)) apply_cell(A, c0 + e % w, e / w, u % 9);
+    }
   }
   __syncwarp();
   fence_before();

@@ -22,19 +22,22 @@ constexpr int COLS = 128, WCOLS = COLS + 4;      // owned and held cell columns
 constexpr int ND = 6;                            // digits of a value
 constexpr int PLANE = WCOLS * 16;                // one digit of one cell row
 constexpr int ROWB = ND * PLANE;                 // a cell row
-constexpr int EPI_WARPS = 8, SLICE_WARPS = 9;    // accumulators to results; values to digits
+// Warp roles.  Accumulators to results: two groups of eight warps (cell row, lane
+// quarter), the first the outputs 0..4 of a cell, the second 5..8; values to digits: nine.
+constexpr int EPI_WARPS = 16, EPI_SPLIT = 5, SLICE_WARPS = 9;
 constexpr int SLICE_T = 32 * SLICE_WARPS;
 static_assert(2 * WCOLS <= SLICE_T, "one thread per cell of a row pair");
 constexpr int EB_MIN = 200;                      // smallest exponent in use (E + 1022): scales stay normal
 
-// q = x 2^(58 - E) rounded to nearest, |x| < 2^E, eb = E + 1022
+// q = x 2^(58 - E) rounded toward zero, |x| < 2^E, eb = E + 1022.  Exact for |x| >=
+// 2^(E - 6): the mantissa's 53 bits then lie above the last place.
 __device__ __forceinline__ long long to_fixed(double x, int eb) {
   const unsigned hi = __double2hiint(x), lo = __double2loint(x);
-  const int e = (hi >> 20) & 0x7ff, d = eb - e, sh = min(max(d, 0), 58);
+  const int e = (hi >> 20) & 0x7ff, d = eb - e;
   const unsigned long long m = (static_cast<unsigned long long>((hi & 0xfffffu) | 0x100000u) << 32) | lo;
-  unsigned long long v = ((m << 10) + (1ull << (sh + 4))) >> (sh + 5);
-  if (e == 0 || d > 58) v = 0;   // subnormal, or below half a unit
-  return (hi >> 31) ? -static_cast<long long>(v) : static_cast<long long>(v);
+  unsigned long long v = (m << 5) >> min(d, 63);    // 0 for d > 58
+  if (e == 0) v = 0;                                // zero, or subnormal
+  return static_cast<int>(hi) < 0 ? -static_cast<long long>(v) : static_cast<long long>(v);
 }
 
 constexpr unsigned long long digit_bias() {
@@ -53,6 +56,21 @@ __device__ __forceinline__ unsigned digit2(unsigned long long a, unsigned long l
   unsigned u;
   memcpy(&u, &h, 4);
   return u;
+}
+
+// hi 2^30 + lo rounded to nearest, |hi| < 2^61, |lo| < 2^60, by integer arithmetic: a
+// conversion instruction costs three of the FP64 unit's 64-clock slots, these about
+// thirty single issue slots
+__device__ __forceinline__ double to_double(long long hi, long long lo) {
+  const int sh = min(30, __clzll(hi ^ (hi >> 63)) - 2);               // a small sum keeps its low bits
+  const long long t = (hi << sh) + (lo >> (30 - sh));                 // in units of 2^(30 - sh)
+  const unsigned long long u = t < 0 ? -static_cast<unsigned long long>(t) : static_cast<unsigned long long>(t);
+  const int lz = __clzll(u);
+  const unsigned long long m = u << (lz & 63);                        // bit 63 set
+  const unsigned long long r = (m >> 11) + ((m >> 10) & 1ull);        // 53 bits, possibly carrying
+  unsigned long long bits = (static_cast<unsigned long long>(1115 - sh - lz) << 52) + r;
+  bits |= static_cast<unsigned long long>(t) & 0x8000000000000000ull;
+  return u != 0 ? __longlong_as_double(static_cast<long long>(bits)) : 0.0;
 }
 
 // 2^(E + k) for eb = E + 1022; NaN for eb = 0x7ff (a value that is not finite)

@@ -230,6 +230,7 @@ struct stokes_hierarchy {
   sv::FastDiagT<float> fdf;      // the same in FP32
   double* stencil_G = nullptr;   // FP64 form: the composite Vanka stencil (VS_TAB doubles)
   unsigned char* stencil_digits = nullptr;   // and its interior cell type as tensor-core digits
+  double* stencil_ring = nullptr;            // and the table of the cells near the boundary
   int stencil_eu = 0, stencil_ep = 0;        // exponents of the digits (tc64_pack)
   unsigned char* op_digits = nullptr;        // integer coefficients of the tensor-core operator
   double* coarse_G = nullptr;    // N0 x N0 dense inverse of the bordered coarse system
@@ -353,9 +354,13 @@ void launch_vanka_stencil(const LevelDev& L, const T* G, const T* x, const T* b,
 
 // The same sweep with the interior cells as an exact digit contraction on the tensor
 // cores (sv_vanka_tc64.cu).  Gp: the packed digits (TC64_BYTES, 16-byte aligned) and the
-// exponents of tc64_pack; Gd: the FP64 table (cells near the boundary); err: set to 1 if
+// exponents of tc64_pack; Gd: vanka_ring_table (cells near the boundary); err: set to 1 if
 // a bounded device wait expired (wait_limit polls).
-constexpr int TC64_BYTES = 34 * 168 * 16 + 128;
+constexpr int TC64_BYTES = 34 * 126 * 16 + 32;
+// The FP64 table of the cells near the boundary, by cell type: [171 residuals][8 velocity
+// outputs], then the 51 coefficients of the pressure output (25 nodes x 2, p).
+constexpr int RT_TYPE = 171 * 8 + 52, RT_TAB = VS_POS * VS_POS * RT_TYPE;
+std::vector<double> vanka_ring_table();
 bool tc64_pack(std::vector<unsigned char>& out, int* eu, int* ep);
 cudaError_t vanka_tc64_prepare();
 void launch_vanka_tc64(const LevelDev& L, const unsigned char* Gp, int eu, int ep, const double* Gd, const double* x,

@@ -27,6 +27,17 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t phase, int limi
   return false;
 }
 
+// the same for several warp roles that share a fail flag: a wait that runs out sets it,
+// and every other wait then returns at once
+__device__ __forceinline__ bool mbar_wait_or_fail(uint32_t bar, uint32_t phase, int limit, volatile int* fail) {
+  for (int it = 0; it < limit; ++it) {
+    if (mbar_wait(bar, phase, 1)) return true;
+    if (*fail) return false;
+  }
+  *fail = 1;
+  return false;
+}
+
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count));
 }
@@ -38,30 +49,48 @@ __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::aft
 __device__ __forceinline__ void fence_proxy() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
-// UMMA shared-memory descriptor: K-major, no swizzle (layout type 0), version 1.
-// lbo: bytes to the next core matrix along K, sbo: to the next 8-row group along M/N.
-__device__ __forceinline__ uint64_t umma_desc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
-  const uint32_t lo = ((saddr >> 4) & 0x3FFFu) | (((lbo >> 4) & 0x3FFFu) << 16);
-  const uint32_t hi = ((sbo >> 4) & 0x3FFFu) | (1u << 14);
-  return (static_cast<uint64_t>(hi) << 32) | lo;
-}
+// UMMA shared-memory descriptor: K-major, no swizzle (layout type 0), version 1.  Low
+// word: start address and lbo (bytes to the next core matrix along K), both / 16; a
+// start further by `bytes` is the word + bytes / 16.  High word: sbo (bytes to the next
+// 8-row group along M or N) / 16.
+__device__ __forceinline__ uint32_t desc_lo(uint32_t saddr, uint32_t lbo) { return (saddr >> 4) | ((lbo >> 4) << 16); }
+constexpr uint32_t desc_hi(uint32_t sbo) { return (sbo >> 4) | (1u << 14); }
 
-__device__ __forceinline__ void mma_f16(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accum) {
+// One MMA / commit by the lane with `on` set, executed by a whole warp with uniform
+// operands: inside a branch of one lane the compiler moves every descriptor from vector
+// to uniform registers, which took 75 clocks per MMA.
+// The operands' 8-row groups follow each other (sbo = 128).
+__device__ __forceinline__ void mma_f16(uint32_t on, uint32_t d, uint32_t a, uint32_t b, uint32_t idesc,
+                                        uint32_t accum) {
   asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
-      "l"(a), "l"(b), "r"(idesc), "r"(accum));
+      "{\n .reg .pred p, q;\n .reg .b64 a, b;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
+      " mov.b64 a, {%1, %6};\n mov.b64 b, {%2, %6};\n"
+      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p;\n}\n" ::"r"(d),
+      "r"(a), "r"(b), "r"(idesc), "r"(accum), "r"(on), "n"(desc_hi(128)));
 }
-__device__ __forceinline__ void mma_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+__device__ __forceinline__ void mma_commit(uint32_t on, uint32_t bar) {
+  asm volatile(
+      "{\n .reg .pred q;\n setp.ne.b32 q, %1, 0;\n"
+      " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(bar),
+      "r"(on)
+      : "memory");
+}
+// 1 in one lane of a converged warp
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t on;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(on));
+  return on;
 }
 
-// nine consecutive accumulator columns of this lane
-__device__ __forceinline__ void tmem_ld9(uint32_t taddr, uint32_t (&r)[9]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+// N consecutive accumulator columns of this lane (N = 4 or 5)
+template <int N>
+__device__ __forceinline__ void tmem_ldn(uint32_t taddr, uint32_t (&r)[N]) {
+  static_assert(N == 4 || N == 5, "columns of one load");
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                : "r"(taddr));
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r[8]) : "r"(taddr + 8));
+  if constexpr (N == 5)
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r[4]) : "r"(taddr + 4));
 }
 
 }  // namespace tc

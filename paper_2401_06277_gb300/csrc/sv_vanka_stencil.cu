@@ -224,6 +224,24 @@ const std::vector<long double>& vanka_stencil() {
   return G;
 }
 
+std::vector<double> vanka_ring_table() {
+  const std::vector<long double>& G = vanka_stencil();
+  std::vector<double> R(RT_TAB, 0.0);
+  for (int t = 0; t < VS_POS * VS_POS; ++t) {
+    const long double* g = G.data() + static_cast<size_t>(t) * VS_TYPE;
+    double* r = R.data() + static_cast<size_t>(t) * RT_TYPE;
+    for (int k = 0; k < 171; ++k)
+      for (int o = 0; o < 8; ++o) r[k * 8 + o] = static_cast<double>(g[o * VS_OUT + k]);
+    const long double* gp = g + 8 * VS_OUT;
+    for (int J = 2; J < 7; ++J)
+      for (int I = 2; I < 7; ++I)
+        for (int c = 0; c < 2; ++c)
+          r[171 * 8 + ((J - 2) * 5 + I - 2) * 2 + c] = static_cast<double>(gp[(J * 9 + I) * 2 + c]);
+    r[171 * 8 + 50] = static_cast<double>(gp[162 + 4]);
+  }
+  return R;
+}
+
 template <typename T>
 void launch_vanka_stencil(const LevelDev& L, const T* G, const T* x, const T* b, T* xo, double omega, T* rscratch,
                           cudaStream_t s) {

@@ -25,13 +25,14 @@
 // [cell column] of 16 bytes (the 8 velocity residuals of a cell): the operand of the
 // cells shifted by (dx, dy) is the same memory at another start address, so nothing is
 // gathered (an implicit im2col with M = 128 consecutive cells).  One step computes two
-// cell rows: K = 30 cell offsets x 8 + 3 x 4 pressures (17 MMAs of K = 16), N = 24
-// columns per coefficient digit (9 outputs of each row, padded to 12).  Digit j of the
-// residual is one chain of 17 MMAs with N = 24 (7 - j) into an accumulator of its own
-// (two alternate); the coefficients (91 KB) stay in shared memory for the whole walk.
+// cell rows: K = 30 cell offsets x 8 + 3 x 4 pressures (17 MMAs of K = 16), N = 18
+// columns per coefficient digit (9 outputs of each row).  Digit j of the residual is one
+// chain of 17 MMAs with N = 18 (7 - j) into an accumulator of its own
+// (chains j and j + 3 take turns); the coefficients (69 KB) stay in shared memory for the whole walk.
 //
-// Warps: 8 read the accumulators and update x (one cell per thread and row), 9 load
-// residuals and write digits, 1 issues the MMAs, and 4 compute the cells near the
+// Warps: 16 read the accumulators and update x (half the outputs of a cell each), 9 load
+// residuals and write digits, 3 issue the MMAs (an MMA takes a warp about as long to
+// issue as the tensor cores to execute), and 4 compute the cells near the
 // boundary, where the stencil differs, as FP64 dot products on the otherwise idle FP64
 // units.  They meet only in mbarriers, per digit: plane j is overwritten for the next
 // rows as soon as chain j has read it.
@@ -65,26 +66,33 @@ using namespace dig;
 using ops::is_free;
 
 constexpr int NG = 7;                            // digits of the coefficients
-constexpr int NBLK = 24;                         // N columns per coefficient digit
-constexpr int GROWS = NBLK * NG;                 // 168 rows of the coefficient operand
+constexpr int NBLK = 18;                         // N columns per coefficient digit: 9 outputs of each cell row
+constexpr int GROWS = NBLK * NG;                 // 126 rows of the coefficient operand
 constexpr int KSTEPS = 17;
 constexpr int CHUNK = GROWS * 16;                // 8 K-values of all coefficient rows
-constexpr int GBYTES = 2 * KSTEPS * CHUNK + 128; // + the rows a padded N reads past the end
+constexpr int GBYTES = 2 * KSTEPS * CHUNK + 32;  // + the two rows that N = 128 reads past the end
 static_assert(GBYTES == TC64_BYTES, "size of the packed coefficients");
-constexpr int RING_WARPS = 4;
-constexpr int NT = 32 * (EPI_WARPS + SLICE_WARPS + 1 + RING_WARPS);
+constexpr int MMA_WARPS = 3, RING_WARPS = 4;   // MMA warp w: chains w and w + 3, one accumulator
+constexpr int NT = 32 * (EPI_WARPS + SLICE_WARPS + MMA_WARPS + RING_WARPS);
 
 struct SM {
   static constexpr int RING = 0;                         // 6 cell rows
   static constexpr int P = RING + 6 * ROWB;              // pressures of the step: [digit][column] 16 B
   static constexpr int G = P + ROWB;
-  static constexpr int BAR = G + GBYTES;                 // full[6], done[6], free[2], gload
+  static constexpr int BAR = (G + GBYTES + 7) / 8 * 8;                 // full[6], done[6], free[3], gload
   static constexpr int MISC = BAR + 16 * 8;              // tmem slot, fail flag, 8 maxima, 4 exponents
   static constexpr int BYTES = MISC + 4 * 16;
-  static_assert(G % 128 == 0 && BAR % 8 == 0 && BYTES <= 227 * 1024, "shared memory");
+  static_assert(G % 16 == 0 && BAR % 8 == 0 && BYTES <= 227 * 1024, "shared memory");
 };
 
 __host__ __device__ constexpr int chain_n(int j) { return (NBLK * (NG - j) + 15) / 16 * 16; }
+// accumulator of the chains c and c + 3: its first tensor-memory column
+__host__ __device__ constexpr int acc_col(int c) {
+  int k = 0;
+  for (int i = 0; i < c % MMA_WARPS; ++i) k += chain_n(i);
+  return k;
+}
+static_assert(acc_col(2) + chain_n(2) <= 512, "tensor memory");
 // instruction descriptor: D FP32, A and B FP16, both K-major, M = 128
 __host__ __device__ constexpr uint32_t idesc(int n) {
   return (1u << 4) | (static_cast<uint32_t>(n >> 3) << 17) | ((128u >> 4) << 24);
@@ -107,79 +115,176 @@ struct Args {
 };
 
 // FP64 dot products of the cells outside [3, n - 3]^2: three cell rows below and above,
-// three columns left and right between them, in units of 8 cells and one output (a
-// warp; four lanes per output).
-__device__ __forceinline__ int ring_units(int n) {
-  return 6 * ((n + 8) / 8) + 6 * ((n - 5 + 7) / 8);
-}
-
-__device__ void ring_unit(const Args& A, int unit, int o) {
-  const LevelDev& L = A.L;
-  const int n = L.n, nq = L.nq, np = L.np, lane = threadIdx.x & 31, part = lane >> 3, c8 = lane & 7;
-  const long long nv = L.nv;
-  const int w = (n + 8) / 8, h = (n - 5 + 7) / 8;
-  int i, j;
+// three columns left and right between them.  The MMAs take nearly all of the shared
+// memory and L1 bandwidth, so a unit is laid out for few load wavefronts: four cells along
+// the band x the eight velocity outputs, whose coefficients are adjacent in the table
+// (a load of the residual serves eight lanes, one of the coefficients four); the pressure
+// outputs take 32 cells.  Node rows and columns off the grid are left out.
+struct Band {
+  int i, j;          // this lane's cell
   bool in;
+  int J0, J1, I0, I1;   // node rows and columns of the 9 x 9 window in use, uniform in the warp
+};
+__host__ __device__ constexpr int ring_units(int n, int cells) {
+  return 6 * ((n + cells) / cells) + 6 * ((n - 5 + cells - 1) / cells);
+}
+__device__ __forceinline__ Band band_of(int n, int unit, int cells, int k) {
+  const int w = (n + cells) / cells, h = (n - 5 + cells - 1) / cells;
+  Band b;
+  b.J0 = b.I0 = 0;
+  b.J1 = b.I1 = 8;
   if (unit < 6 * w) {          // rows 0, 1, 2, n - 2, n - 1, n
     const int row = unit / w;
-    j = row < 3 ? row : n - 2 + row - 3;
-    i = 8 * (unit - row * w) + c8;
-    in = i <= n && j <= n;
+    b.j = row < 3 ? row : n - 2 + row - 3;
+    b.i = cells * (unit - row * w) + k;
+    b.in = b.i <= n;
+    b.J0 = max(0, 5 - 2 * b.j);
+    b.J1 = min(8, 2 * (n - b.j) + 3);
   } else {                     // columns, rows 3 .. n - 3
     const int v = unit - 6 * w, col = v / h;
-    i = col < 3 ? col : n - 2 + col - 3;
-    j = 3 + 8 * (v - col * h) + c8;
-    in = i <= n && j <= n - 3;
+    b.i = col < 3 ? col : n - 2 + col - 3;
+    b.j = 3 + cells * (v - col * h) + k;
+    b.in = b.j <= n - 3;
+    b.I0 = max(0, 5 - 2 * b.i);
+    b.I1 = min(8, 2 * (n - b.i) + 3);
   }
+  return b;
+}
+__device__ __forceinline__ int cell_type(int n, const Band& b) {
   auto pos = [n](int a) { return a < 3 ? a : a <= n - 3 ? 3 : a >= n ? 6 : a - (n - 2) + 4; };
-  const double* g = A.Gd + static_cast<size_t>(pos(in ? j : 0) * VS_POS + pos(in ? i : 0)) * VS_TYPE + o * VS_OUT;
+  return b.in ? pos(b.j) * VS_POS + pos(b.i) : 0;
+}
+
+__device__ __forceinline__ void ring_velocity(const Args& A, int unit, int lane) {
+  const LevelDev& L = A.L;
+  const int n = L.n, nq = L.nq, np = L.np, o = lane & 7;
+  const long long nv = L.nv;
+  const Band b = band_of(n, unit, 4, lane >> 3);
+  const double* g = A.Gd + static_cast<size_t>(cell_type(n, b)) * RT_TYPE + o;
   double a0 = 0.0, a1 = 0.0;
-  auto node = [&](int rJ, int rI) {
-    const int I = 2 * i - 4 + rI, J = 2 * j - 4 + rJ;
-    if (!in || !is_free(I, J, nq)) return;
-    const double2 wgt = __ldg(reinterpret_cast<const double2*>(g) + rJ * 9 + rI);
-    const double* p = A.r + static_cast<long long>(J) * nq + I;
-    a0 = fma(wgt.x, __ldg(p), a0);
-    a1 = fma(wgt.y, __ldg(p + nv), a1);
-  };
-  const int py = o == 8 ? 0 : (o >> 1) & 1, px = o == 8 ? 0 : o & 1;
-  if (o == 8) {
-#pragma unroll
-    for (int e = part; e < 25; e += 4) node(2 + e / 5, 2 + e % 5);
-  } else if (px) {
-    const int cnt = (9 - 2 * py) * 7;
-#pragma unroll 4
-    for (int e = part; e < cnt; e += 4) node(2 * py + e / 7, 2 + e % 7);
-  } else {
-    const int cnt = (9 - 2 * py) * 9;
-#pragma unroll 4
-    for (int e = part; e < cnt; e += 4) node(2 * py + e / 9, e % 9);
+  for (int rJ = b.J0; rJ <= b.J1; ++rJ) {
+    const int J = 2 * b.j - 4 + rJ;
+    const double* rr = A.r + static_cast<long long>(J) * nq + 2 * b.i - 4;
+    const double* gr = g + rJ * 144;
+#pragma unroll 3
+    for (int rI = b.I0; rI <= b.I1; ++rI) {
+      const bool ok = b.in && is_free(2 * b.i - 4 + rI, J, nq);
+      const double r0 = ok ? __ldg(rr + rI) : 0.0, r1 = ok ? __ldg(rr + nv + rI) : 0.0;
+      a0 = fma(__ldg(gr + rI * 16), r0, a0);
+      a1 = fma(__ldg(gr + rI * 16 + 8), r1, a1);
+    }
   }
   double ap = 0.0;
-  for (int k = part; k < 9; k += 4) {
-    const int dj = k / 3 - 1, di = k % 3 - 1, pi = i + di, pj = j + dj;
-    if (!in || pi < 0 || pj < 0 || pi > n || pj > n) continue;
-    ap = fma(__ldg(g + 162 + k), A.rps * __ldg(A.r + 2 * nv + static_cast<long long>(pj) * np + pi), ap);
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    const int pi = b.i + k % 3 - 1, pj = b.j + k / 3 - 1;
+    const bool ok = b.in && pi >= 0 && pj >= 0 && pi <= n && pj <= n;
+    const double r0 = ok ? __ldg(A.r + 2 * nv + static_cast<long long>(pj) * np + pi) : 0.0;
+    ap = fma(__ldg(g + 162 * 8 + k * 8), r0, ap);
   }
-  double d = (a0 + a1) + ap;
-  d += __shfl_xor_sync(0xffffffffu, d, 8);
-  d += __shfl_xor_sync(0xffffffffu, d, 16);
-  if (part != 0 || !in) return;
-  if (o == 8) {
-    const long long k = 2 * nv + static_cast<long long>(j) * np + i;
-    A.xo[k] = fma(A.sp, d, A.x != nullptr ? A.x[k] : 0.0);
-  } else {
-    const int I = 2 * i + px, J = 2 * j + py;
-    if (I >= nq || J >= nq) return;
-    const long long k = (o >> 2) * nv + static_cast<long long>(J) * nq + I;
-    const double xv = A.x != nullptr ? A.x[k] : 0.0;
-    A.xo[k] = is_free(I, J, nq) ? fma(A.su, d, xv) : fma(A.omega, A.r[k], xv);
+  const int I = 2 * b.i + (o & 1), J = 2 * b.j + ((o >> 1) & 1);
+  if (!b.in || I >= nq || J >= nq) return;
+  const long long k = (o >> 2) * nv + static_cast<long long>(J) * nq + I;
+  const double xv = A.x != nullptr ? A.x[k] : 0.0;
+  A.xo[k] = is_free(I, J, nq) ? fma(A.su, fma(A.rps, ap, a0 + a1), xv) : fma(A.omega, A.r[k], xv);
+}
+
+__device__ __forceinline__ void ring_pressure(const Args& A, int unit, int lane) {
+  const LevelDev& L = A.L;
+  const int n = L.n, nq = L.nq;
+  const long long nv = L.nv;
+  const Band b = band_of(n, unit, 32, lane);
+  const double* g = A.Gd + static_cast<size_t>(cell_type(n, b)) * RT_TYPE + 171 * 8;
+  double a0 = 0.0, a1 = 0.0;
+  for (int rJ = max(2, b.J0); rJ <= min(6, b.J1); ++rJ) {
+    const int J = 2 * b.j - 4 + rJ;
+#pragma unroll
+    for (int rI = 2; rI < 7; ++rI) {
+      const int I = 2 * b.i - 4 + rI;
+      const bool ok = b.in && is_free(I, J, nq);
+      const double* rr = A.r + static_cast<long long>(J) * nq + I;
+      const double* gr = g + ((rJ - 2) * 5 + rI - 2) * 2;
+      a0 = fma(__ldg(gr), ok ? __ldg(rr) : 0.0, a0);
+      a1 = fma(__ldg(gr + 1), ok ? __ldg(rr + nv) : 0.0, a1);
+    }
   }
+  if (!b.in) return;
+  const long long k = 2 * nv + static_cast<long long>(b.j) * L.np + b.i;
+  const double d = fma(A.rps * __ldg(g + 50), A.r[k], a0 + a1);
+  A.xo[k] = fma(A.sp, d, A.x != nullptr ? A.x[k] : 0.0);
 }
 
 // T += D 2^k for the weights of the digit pairs; the compiler makes it one IMAD.WIDE
 __device__ __forceinline__ void madw(long long& t, uint32_t f, int k) {
   t += static_cast<long long>(__float2int_rn(__uint_as_float(f))) * (1ll << k);
+}
+
+constexpr int BATCH = 4;   // coefficient digits read from tensor memory at a time
+
+struct Shared {   // what the roles of a CTA share
+  uint32_t full, done, free, tmem;
+  volatile int* fail;
+  volatile int* sexp;
+  int i0, j0, rows, S;
+};
+
+// Accumulators to x for the outputs O0 .. O0 + NO - 1: warp -> cell row a and lane
+// quarter of the columns.
+template <int O0, int NO>
+__device__ __forceinline__ void epilogue(const Args& A, const Shared& C, int warp, int lane) {
+  const LevelDev& L = A.L;
+  const int n = L.n, nq = L.nq, np = L.np;
+  const long long nv = L.nv;
+  const int a = (warp >> 2) & 1, i = C.i0 + 32 * (warp & 3) + lane;
+  const uint32_t tq = C.tmem + (static_cast<uint32_t>(32 * (warp & 3)) << 16) + 9 * a + O0;
+  for (int s = 0; s < C.S; ++s) {
+    const int j = C.j0 + 2 * s + a;
+    const bool own = i <= n - 3 && 2 * s + a < C.rows;
+    const long long ku = static_cast<long long>(2 * j) * nq + 2 * i;
+    const long long kp = 2 * nv + static_cast<long long>(j) * np + i;
+    auto at = [&](int o) { return o == 8 ? kp : (o >> 2) * nv + ku + ((o >> 1) & 1) * nq + (o & 1); };
+    double xv[NO];
+#pragma unroll
+    for (int o = 0; o < NO; ++o) xv[o] = own && A.x != nullptr ? A.x[at(O0 + o)] : 0.0;
+    long long hi[NO], lo[NO];
+#pragma unroll
+    for (int o = 0; o < NO; ++o) hi[o] = lo[o] = 0;
+    bool ok = true;
+#pragma unroll
+    for (int c = 0; c < ND; ++c) {
+      ok = mbar_wait_or_fail(C.done + 8 * c, s & 1, A.wait_limit, C.fail);
+      if (!__all_sync(0xffffffffu, ok)) return;
+      fence_after();
+#pragma unroll
+      for (int i2 = 0; i2 < NG - c; i2 += BATCH) {
+        uint32_t v[BATCH][NO];
+#pragma unroll
+        for (int u = 0; u < BATCH; ++u)
+          if (i2 + u < NG - c) tmem_ldn<NO>(tq + acc_col(c) + NBLK * (i2 + u), v[u]);
+        wait_ld();
+#pragma unroll
+        for (int u = 0; u < BATCH; ++u) {
+          const int gi = i2 + u, k = 59 - 9 * gi - 10 * c;
+          if (gi >= NG - c) continue;
+#pragma unroll
+          for (int o = 0; o < NO; ++o) {
+            if (k >= 30) madw(hi[o], v[u][o], k - 30);
+            else madw(lo[o], v[u][o], k);
+          }
+        }
+      }
+      fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(C.free + 8 * (c % MMA_WARPS));
+    }
+    const double sc = exp_scale(C.sexp[s & 3], -75);   // NaN where a residual of the window is not finite
+    if (own) {
+      const double qu = A.qu * sc, qp = A.qp * sc;
+#pragma unroll
+      for (int o = 0; o < NO; ++o)
+        A.xo[at(O0 + o)] = fma(O0 + o == 8 ? qp : qu, to_double(hi[o], lo[o]), xv[o]);
+    }
+  }
 }
 
 __global__ void __launch_bounds__(NT, 1) k_vanka_tc64(const Args A) {
@@ -191,7 +296,7 @@ __global__ void __launch_bounds__(NT, 1) k_vanka_tc64(const Args A) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t s0 = su32(sm);
   const uint32_t bar_full = s0 + SM::BAR, bar_done = bar_full + 8 * ND, bar_free = bar_done + 8 * ND,
-                 bar_g = bar_free + 16;
+                 bar_g = bar_free + 8 * MMA_WARPS;
   uint32_t* tslot = reinterpret_cast<uint32_t*>(sm + SM::MISC);
   volatile int* fail = reinterpret_cast<volatile int*>(sm + SM::MISC + 4);
   int* smax = reinterpret_cast<int*>(sm + SM::MISC + 8);                    // 8 slots
@@ -206,8 +311,7 @@ __global__ void __launch_bounds__(NT, 1) k_vanka_tc64(const Args A) {
       mbar_init(bar_full + 8 * k, SLICE_WARPS);
       mbar_init(bar_done + 8 * k, 1);
     }
-    mbar_init(bar_free, EPI_WARPS);
-    mbar_init(bar_free + 8, EPI_WARPS);
+    for (int k = 0; k < MMA_WARPS; ++k) mbar_init(bar_free + 8 * k, EPI_WARPS);
     mbar_init(bar_g, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     *fail = 0;
@@ -225,71 +329,11 @@ __global__ void __launch_bounds__(NT, 1) k_vanka_tc64(const Args A) {
   fence_after();
   const uint32_t tmem = *tslot;
 
-  if (warp < EPI_WARPS) {
-    // ---- accumulators to x: warp -> cell row a, lane quarter of the columns ----
-    const int a = warp >> 2, col = 32 * (warp & 3) + lane, i = i0 + col;
-    const uint32_t tq = tmem + (static_cast<uint32_t>(32 * (warp & 3)) << 16) + 12 * a;
-    for (int s = 0; s < S; ++s) {
-      const int j = j0 + 2 * s + a;
-      const bool own = i <= n - 3 && 2 * s + a < rows;
-      const long long ku = static_cast<long long>(2 * j) * nq + 2 * i;
-      const long long kp = 2 * nv + static_cast<long long>(j) * np + i;
-      double xv[9];
-#pragma unroll
-      for (int o = 0; o < 9; ++o) xv[o] = 0.0;
-      if (own && A.x != nullptr) {
-#pragma unroll
-        for (int o = 0; o < 8; ++o) xv[o] = A.x[(o >> 2) * nv + ku + ((o >> 1) & 1) * nq + (o & 1)];
-        xv[8] = A.x[kp];
-      }
-      long long hi[9], lo[9];
-#pragma unroll
-      for (int o = 0; o < 9; ++o) hi[o] = lo[o] = 0;
-      bool ok = true;
-#pragma unroll
-      for (int c = 0; c < ND; ++c) {
-        ok = ok && mbar_wait(bar_done + 8 * c, s & 1, A.wait_limit);
-        ok = __all_sync(0xffffffffu, ok) && !*fail;
-        if (!ok) break;
-        fence_after();
-#pragma unroll
-        for (int i2 = 0; i2 < NG - c; i2 += 2) {
-          uint32_t v[2][9];
-          tmem_ld9(tq + 256 * (c & 1) + NBLK * i2, v[0]);
-          if (i2 + 1 < NG - c) tmem_ld9(tq + 256 * (c & 1) + NBLK * (i2 + 1), v[1]);
-          wait_ld();
-#pragma unroll
-          for (int u = 0; u < 2; ++u) {
-            const int gi = i2 + u, k = 59 - 9 * gi - 10 * c;
-            if (gi >= NG - c) continue;
-#pragma unroll
-            for (int o = 0; o < 9; ++o) {
-              if (k >= 30) madw(hi[o], v[u][o], k - 30);
-              else madw(lo[o], v[u][o], k);
-            }
-          }
-        }
-        fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar_free + 8 * (c & 1));
-      }
-      if (!ok) {
-        if (lane == 0) *fail = 1;
-        break;
-      }
-      const int eb = sexp[s & 3];
-      const double sc = exp_scale(eb, -57);   // NaN where a residual of the window is not finite
-      if (own) {
-        const double qu = A.qu * sc, qp = A.qp * sc;
-#pragma unroll
-        for (int o = 0; o < 9; ++o) {
-          const long long t = (hi[o] << 12) + ((lo[o] + (1ll << 17)) >> 18);
-          const double d = static_cast<double>(t);
-          if (o < 8) A.xo[(o >> 2) * nv + ku + ((o >> 1) & 1) * nq + (o & 1)] = fma(qu, d, xv[o]);
-          else A.xo[kp] = fma(qp, d, xv[8]);
-        }
-      }
-    }
+  const Shared C{bar_full, bar_done, bar_free, tmem, fail, sexp, i0, j0, rows, S};
+  if (warp < EPI_WARPS / 2) {
+    epilogue<0, EPI_SPLIT>(A, C, warp, lane);
+  } else if (warp < EPI_WARPS) {
+    epilogue<EPI_SPLIT, 9 - EPI_SPLIT>(A, C, warp, lane);
   } else if (warp < EPI_WARPS + SLICE_WARPS) {
     // ---- residuals to digits: thread -> cell of the row pair ----
     const int t = tid - 32 * EPI_WARPS;
@@ -311,7 +355,7 @@ __global__ void __launch_bounds__(NT, 1) k_vanka_tc64(const Args A) {
       for (int k = 0; k < 2; ++k) {
         const int pj = j0 - 5 + 2 * q + 2 * a + k;
         c.p[k] = (act && q >= 2 && gi <= n && pj <= n)
-                     ? A.rps * A.r[2 * nv + static_cast<long long>(pj) * np + gi] : 0.0;
+                     ? A.r[2 * nv + static_cast<long long>(pj) * np + gi] : 0.0;
       }
     };
     int eb = 0;
@@ -324,12 +368,11 @@ __global__ void __launch_bounds__(NT, 1) k_vanka_tc64(const Args A) {
       const uint4 d = make_uint4(digit2(w[0], w[1], j), digit2(w[2], w[3], j), digit2(w[4], w[5], j), digit2(w[6], w[7], j));
       *reinterpret_cast<uint4*>(sm + SM::RING + (2 * (q % 3) + a) * ROWB + j * PLANE + col * 16) = d;
     };
-    Cell cur, nxt;
-    load(0, nxt);
-    bool ok = true;
-    for (int q = 0; q < S + 2 && ok; ++q) {
-      cur = nxt;
-      if (q + 1 < S + 2) load(q + 1, nxt);
+    Cell cur;
+    load(0, cur);
+    for (int q = 0; q < S + 2; ++q) {
+      cur.p[0] *= A.rps;
+      cur.p[1] *= A.rps;
       int m = 0;
 #pragma unroll
       for (int o = 0; o < 8; ++o) m = max(m, __double2hiint(cur.v[o]) & 0x7fffffff);
@@ -338,7 +381,10 @@ __global__ void __launch_bounds__(NT, 1) k_vanka_tc64(const Args A) {
       if (lane == 0) atomicMax(smax + (q & 7), m);
       asm volatile("bar.sync 1, %0;" ::"n"(SLICE_T) : "memory");
       if (t == 0) smax[(q + 3) & 7] = 0;
-      if (q < 2) continue;
+      if (q < 2) {
+        load(q + 1, cur);
+        continue;
+      }
       const volatile int* vm = smax;
       const int em = max(vm[q & 7], max(vm[(q - 1) & 7], vm[(q - 2) & 7])) >> 20;   // |x| < 2^(em - 1022)
       const int s = q - 2;
@@ -346,7 +392,7 @@ __global__ void __launch_bounds__(NT, 1) k_vanka_tc64(const Args A) {
       const bool renew = s == 0 || em > eb || (eb - em > 3 && eb > EB_MIN);
       if (renew) {   // uniform over the slicer warps
         eb = min(max(em + 1, EB_MIN), 0x7ff);
-        if (s > 0) ok = mbar_wait(bar_done + 8 * (ND - 1), (s - 1) & 1, A.wait_limit);
+        if (s > 0) mbar_wait_or_fail(bar_done + 8 * (ND - 1), (s - 1) & 1, A.wait_limit, fail);
         for (int qq = q - 2; qq < q; ++qq) {
           Cell c;
           load(qq, c);
@@ -360,80 +406,78 @@ __global__ void __launch_bounds__(NT, 1) k_vanka_tc64(const Args A) {
       unsigned long long wp[2];
 #pragma unroll
       for (int k = 0; k < 2; ++k) wp[k] = static_cast<unsigned long long>(to_fixed(cur.p[k], eb)) + digit_bias();
+      if (q + 1 < S + 2) load(q + 1, cur);   // in flight while the planes are written
 #pragma unroll
       for (int j = 0; j < ND; ++j) {
-        if (!renew && ok) ok = mbar_wait(bar_done + 8 * j, (s - 1) & 1, A.wait_limit);
-        if (ok) {
-          put(q, j, w);
-          if (act) *reinterpret_cast<unsigned*>(sm + SM::P + j * PLANE + col * 16 + 4 * a) = digit2(wp[0], wp[1], j);
-        }
+        // plane j of the row pair is free once chain j of the step before has read it (after
+        // a failed wait the results are void and only the arrivals matter)
+        if (!renew) mbar_wait_or_fail(bar_done + 8 * j, (s - 1) & 1, A.wait_limit, fail);
+        put(q, j, w);
+        if (act) *reinterpret_cast<unsigned*>(sm + SM::P + j * PLANE + col * 16 + 4 * a) = digit2(wp[0], wp[1], j);
         fence_proxy();
         __syncwarp();
         if (lane == 0) mbar_arrive(bar_full + 8 * j);
       }
-      if (!ok) *fail = 1;
-      ok = !*fail;
-      // every slicer warp leaves at the same row pair: the named barrier above counts them all
-      asm volatile("bar.sync 1, %0;" ::"n"(SLICE_T) : "memory");
-      ok = !*fail;
     }
-  } else if (warp == EPI_WARPS + SLICE_WARPS) {
-    if (lane == 0) {
-      // ---- coefficients, then the MMAs ----
+  } else if (warp < EPI_WARPS + SLICE_WARPS + MMA_WARPS) {
+    // ---- coefficients, then the MMAs ----
+    const uint32_t on = elect_one();
+    if (on && warp == EPI_WARPS + SLICE_WARPS) {
       asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar_g), "r"(GBYTES) : "memory");
       asm volatile(
           "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(s0 + SM::G),
           "l"(A.G), "r"(GBYTES), "r"(bar_g)
           : "memory");
-      bool ok = mbar_wait(bar_g, 0, A.wait_limit);
-      int issued = 0;   // chains committed
-      for (int s = 0; s < S && ok; ++s) {
-#pragma unroll 1
-        for (int c = 0; c < ND && ok; ++c) {
-          ok = mbar_wait(bar_full + 8 * c, s & 1, A.wait_limit);
-          const int use = 3 * s + (c >> 1);   // earlier chains of this accumulator
-          if (ok && use > 0) ok = mbar_wait(bar_free + 8 * (c & 1), (use - 1) & 1, A.wait_limit);
-          if (!ok || *fail) {
-            ok = false;
-            break;
-          }
-          fence_after();
-          const uint32_t d = tmem + 256 * (c & 1), id = idesc(chain_n(c));
-          const uint32_t g0 = s0 + SM::G, pl = s0 + SM::RING + c * PLANE;
-          const uint32_t row[3] = {pl + 2 * (s % 3) * ROWB, pl + 2 * ((s + 1) % 3) * ROWB, pl + 2 * ((s + 2) % 3) * ROWB};
-          int k = 0;
-#pragma unroll
-          for (int b = 0; b < 6; ++b)   // cell rows dy = -2 .. 3, offsets dx = (-2, -1) and (0, 1)
-#pragma unroll
-            for (int h = 0; h < 2; ++h, ++k)
-              mma_f16(d, umma_desc(row[b >> 1] + (b & 1) * ROWB + 32 * h, 16, 128),
-                      umma_desc(g0 + 2 * k * CHUNK, CHUNK, 128), id, k > 0);
-#pragma unroll
-          for (int b = 0; b < 3; ++b, ++k)   // dx = 2 of both rows of a pair
-            mma_f16(d, umma_desc(row[b] + 64, ROWB, 128), umma_desc(g0 + 2 * k * CHUNK, CHUNK, 128), id, 1);
-          const uint32_t pp = s0 + SM::P + c * PLANE + 16;
-#pragma unroll
-          for (int h = 0; h < 2; ++h, ++k)   // pressures, dx = (-1, 0) and (1, none)
-            mma_f16(d, umma_desc(pp + 32 * h, 16, 128), umma_desc(g0 + 2 * k * CHUNK, CHUNK, 128), id, 1);
-          mma_commit(bar_done + 8 * c);
-          ++issued;
-        }
-      }
-      if (!ok) *fail = 1;
-      // every chain that was issued has completed before the operands and tensor memory go
-      if (issued > 0) {
-        const int last = issued - 1;
-        if (!mbar_wait(bar_done + 8 * (last % ND), (last / ND) & 1, TC_WAIT_LIMIT)) *fail = 1;
-      }
-      mbar_wait(bar_g, 0, TC_WAIT_LIMIT);
     }
+    __syncwarp();
+    auto wait = [&](uint32_t bar, uint32_t phase) {   // a vote, so that the loop stays uniform
+      return __all_sync(0xffffffffu, mbar_wait_or_fail(bar, phase, A.wait_limit, fail)) != 0;
+    };
+    bool ok = wait(bar_g, 0);
+    const int w = warp - (EPI_WARPS + SLICE_WARPS);
+    int last = -1;   // the last chain committed, as s ND + c
+    const uint32_t gl = desc_lo(s0 + SM::G, CHUNK), pl = desc_lo(s0 + SM::P + 16, 16);
+    const uint32_t rl = desc_lo(s0 + SM::RING, 16), r2 = desc_lo(s0 + SM::RING + 64, ROWB);
+    for (int s = 0; s < S && ok; ++s) {
+      // the row pairs dy = (-2, -1), (0, 1), (2, 3) in units of 16 bytes
+      const uint32_t us = s, row[3] = {us % 3 * (ROWB / 8), (us + 1) % 3 * (ROWB / 8), (us + 2) % 3 * (ROWB / 8)};
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int c = w + MMA_WARPS * h;
+        if (ok) ok = wait(bar_full + 8 * c, s & 1);
+        const int use = 2 * s + h;   // earlier chains of this accumulator
+        if (ok && use > 0) ok = wait(bar_free + 8 * w, (use - 1) & 1);
+        if (!ok) break;
+        fence_after();
+        const uint32_t d = tmem + acc_col(w), id = idesc(chain_n(c)), off = c * (PLANE / 16);
+        int k = 0;
+#pragma unroll
+        for (int b = 0; b < 6; ++b)   // cell rows dy = -2 .. 3, offsets dx = (-2, -1) and (0, 1)
+#pragma unroll
+          for (int e = 0; e < 2; ++e, ++k)
+            mma_f16(on, d, rl + off + row[b >> 1] + (b & 1) * (ROWB / 16) + 2 * e, gl + k * (CHUNK / 8), id, k > 0);
+#pragma unroll
+        for (int b = 0; b < 3; ++b, ++k)   // dx = 2 of both rows of a pair
+          mma_f16(on, d, r2 + off + row[b], gl + k * (CHUNK / 8), id, 1);
+#pragma unroll
+        for (int e = 0; e < 2; ++e, ++k)   // pressures, dx = (-1, 0) and (1, none)
+          mma_f16(on, d, pl + off + 2 * e, gl + k * (CHUNK / 8), id, 1);
+        mma_commit(on, bar_done + 8 * c);
+        last = s * ND + c;
+      }
+    }
+    // every chain that was issued has completed before the operands and tensor memory go
+    if (last >= 0 && !mbar_wait(bar_done + 8 * (last % ND), (last / ND) & 1, TC_WAIT_LIMIT)) *fail = 1;
+    mbar_wait(bar_g, 0, TC_WAIT_LIMIT);
     __syncwarp();
   } else {
     // ---- cells near the boundary: units dealt to the ring warps of all CTAs ----
     const int ctas = gridDim.x * gridDim.y, cta = blockIdx.y * gridDim.x + blockIdx.x;
-    const int units = 9 * ring_units(n);
-    for (int u = (warp - (EPI_WARPS + SLICE_WARPS + 1)) * ctas + cta; u < units; u += RING_WARPS * ctas)
-      ring_unit(A, u / 9, u % 9);
+    const int uv = ring_units(n, 4), up = ring_units(n, 32);
+    for (int u = (warp - (EPI_WARPS + SLICE_WARPS + MMA_WARPS)) * ctas + cta; u < uv + up; u += RING_WARPS * ctas) {
+      if (u < uv) ring_velocity(A, u, lane);
+      else ring_pressure(A, u - uv, lane);
+    }
   }
   __syncwarp();
   fence_before();
@@ -445,7 +489,7 @@ __global__ void __launch_bounds__(NT, 1) k_vanka_tc64(const Args A) {
 
 }  // namespace
 
-// Digits of the interior cell type in the K order of the kernel's MMAs.  Row 24 i + 12 a
+// Digits of the interior cell type in the K order of the kernel's MMAs.  Row 18 i + 9 a
 // + o of the operand is digit i of output o of cell row j + a.  Returns the exponents of
 // the velocity and pressure outputs and whether every digit pair sums below 2^24.
 bool tc64_pack(std::vector<unsigned char>& out, int* eu, int* ep) {
@@ -468,7 +512,7 @@ bool tc64_pack(std::vector<unsigned char>& out, int* eu, int* ep) {
       X = (X - d) >> 9;
       sum[i][9 * a + o] += std::fabs(static_cast<double>(d));
       const __half h = __float2half_rn(static_cast<float>(d));   // exact
-      std::memcpy(out.data() + static_cast<size_t>(chunk) * CHUNK + (NBLK * i + 12 * a + o) * 16 + 2 * ch, &h, 2);
+      std::memcpy(out.data() + static_cast<size_t>(chunk) * CHUNK + (NBLK * i + 9 * a + o) * 16 + 2 * ch, &h, 2);
     }
   };
   for (int a = 0; a < 2; ++a)
