@@ -107,6 +107,8 @@ void free_all(stokes_hierarchy* h) {
   h->bt_GL = h->bt_GM = h->bt_buf = nullptr;
   h->lv.clear();
   cudaFree(h->stencil_G);
+  cudaFree(h->stencil_Gf);
+  h->stencil_Gf = nullptr;
   cudaFree(h->stencil_digits);
   cudaFree(h->stencil_ring);
   h->stencil_ring = nullptr;
@@ -247,6 +249,8 @@ void timed_sweep<float>(stokes_hierarchy* h, bool finest, sv::Level& L, const fl
   if (ev) cudaEventRecord(ev[0], h->stream);
   if (h->prm.smoother == STOKES_SMOOTHER_BRAESS_SARAZIN || h->prm.smoother == STOKES_SMOOTHER_SCHUR_UZAWA) {
     sv::launch_bs_sweep<float>(L.d, h->bs, static_cast<float*>(h->bs_buf), L.rf, x, b, xo, h->stream);
+  } else if (L.vk_cfg_f == sv::VANKA_CFG_STENCIL) {
+    sv::launch_vanka_stencil<float>(L.d, h->stencil_Gf, x, b, xo, h->prm.omega, L.rf, h->stream);
   } else if (L.strip && L.tc_on) {
     tc_sweep(h, L, x, b, xo, h->stream);
   } else if (sv::vanka_cfg_split(L.vk_cfg_f)) {
@@ -801,6 +805,10 @@ cudaError_t tune_level(stokes_hierarchy* h, sv::Level& L, int* cfg) {
   return cudaGetLastError();
 }
 
+// The FP32 sweep of the mixed forms is the composite stencil up to this size.  V-cycle
+// of a 128^2 grid with it up to n = 0 / 32 / 64 / 128: 260 / 216 / 200 / 223 us; beyond
+// n = 64 its 1125 multiply-adds per vertex exceed those of the tiled patch solves.
+constexpr int STENCIL_F32_MAX_N = 64;
 // Levels whose FP64 operator is the tensor-core contraction (smaller ones: FP64, one
 // output per thread).
 constexpr int OP_TC64_MIN_N = 160;
@@ -825,6 +833,7 @@ cudaError_t choose_tiles(stokes_hierarchy* h) {
     if (h->prm.prec == STOKES_FP64 && L.d.n >= sv::VS_MIN_N)
       L.vk_cfg = (h->stencil_digits && L.d.n >= TC64_MIN_N) ? sv::VANKA_CFG_TC64 : sv::VANKA_CFG_STENCIL;
     else if (h->prm.prec == STOKES_FP64) e = tune_level<double>(h, L, &L.vk_cfg);
+    else if (h->stencil_Gf && L.d.n >= sv::VS_MIN_N && L.d.n <= STENCIL_F32_MAX_N) L.vk_cfg_f = sv::VANKA_CFG_STENCIL;
     else e = tune_level<float>(h, L, &L.vk_cfg_f);   // strip sweep vs SIMT shapes
     if (e != cudaSuccess) return e;
   }
@@ -1039,6 +1048,16 @@ stokes_status stokes_hierarchy_create(int n, double viscosity, const stokes_para
       free_all(h);
       delete h;
       return cuda_fail(e, "block-triangular set-up");
+    }
+  }
+  if (mixed && prm.smoother == STOKES_SMOOTHER_SHARED) {
+    const std::vector<long double>& G = sv::vanka_stencil();
+    const std::vector<float> Gf(G.begin(), G.end());
+    if ((e = dalloc(&h->stencil_Gf, Gf.size())) != cudaSuccess ||
+        (e = cudaMemcpy(h->stencil_Gf, Gf.data(), Gf.size() * sizeof(float), cudaMemcpyHostToDevice)) != cudaSuccess) {
+      free_all(h);
+      delete h;
+      return cuda_fail(e, "composite stencil upload");
     }
   }
   if (prm.prec == STOKES_FP64 && prm.smoother == STOKES_SMOOTHER_SHARED) {

@@ -229,6 +229,7 @@ struct stokes_hierarchy {
   sv::FastDiag fd;               // interior patch factors (level independent)
   sv::FastDiagT<float> fdf;      // the same in FP32
   double* stencil_G = nullptr;   // FP64 form: the composite Vanka stencil (VS_TAB doubles)
+  float* stencil_Gf = nullptr;               // mixed forms: the table in FP32
   unsigned char* stencil_digits = nullptr;   // and its interior cell type as tensor-core digits
   double* stencil_ring = nullptr;            // and the table of the cells near the boundary
   int stencil_eu = 0, stencil_ep = 0;        // exponents of the digits (tc64_pack)
