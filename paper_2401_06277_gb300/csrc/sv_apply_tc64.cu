@@ -88,6 +88,9 @@ __device__ __noinline__ void apply_cell(const Args& A, int i, int j, int o) {
   }
 }
 
+// phase of full[s % 3] for step s >= 1 (step 0 needs no arrival)
+__device__ __forceinline__ uint32_t full_phase(int s) { return (s % 3 == 0 ? s / 3 - 1 : s / 3) & 1; }
+
 struct Shared {   // what the roles of a CTA share
   uint32_t full, done, free, tmem;
   volatile int* fail;
@@ -188,7 +191,6 @@ __global__ void __launch_bounds__(NT, 1) k_apply_tc64(const Args A) {
   }
   for (int k = tid; k < 2 * ROWB / 16; k += NT)   // channels 4..7 of the pressures stay zero
     reinterpret_cast<uint4*>(sm + SM::P)[k] = make_uint4(0u, 0u, 0u, 0u);
-  fence_proxy();
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tslot)), "r"(512));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
@@ -197,6 +199,86 @@ __global__ void __launch_bounds__(NT, 1) k_apply_tc64(const Args A) {
   __syncthreads();
   fence_after();
   const uint32_t tmem = *tslot;
+  if (tid == 0) {   // the coefficients, while the first window is loaded
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar_g), "r"(GBYTES) : "memory");
+    asm volatile(
+        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(s0 + SM::G),
+        "l"(A.G), "r"(GBYTES), "r"(bar_g)
+        : "memory");
+  }
+
+  // ---- values to digits: a thread takes a cell (a, col) of a row pair q ----
+  struct Cell {
+    double v[8];
+    double p[2];
+  };
+  auto load = [&](int q, int a, int col, bool act, Cell& c) {   // cell row j0 - 1 + 2 q + a; pressures j0 - 3 + 2 q + 2 a + {0, 1}
+    const int gi = i0 - 2 + col, gj = j0 - 1 + 2 * q + a;
+#pragma unroll
+    for (int o = 0; o < 8; ++o) {
+      const int I = 2 * gi + (o & 1), J = 2 * gj + ((o >> 1) & 1);
+      c.v[o] = (act && is_free(I, J, nq)) ? A.x[(o >> 2) * nv + static_cast<long long>(J) * nq + I] : 0.0;
+    }
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int pj = j0 - 3 + 2 * q + 2 * a + k;
+      c.p[k] = (act && q >= 1 && gi >= 0 && gi <= n && pj >= 0 && pj <= n)
+                   ? A.x[2 * nv + static_cast<long long>(pj) * np + gi] : 0.0;
+    }
+  };
+  auto note_max = [&](int q, Cell& c) {   // pressures to their units; the pair's largest exponent
+    c.p[0] *= A.ps;
+    c.p[1] *= A.ps;
+    int m = max(__double2hiint(c.p[0]) & 0x7fffffff, __double2hiint(c.p[1]) & 0x7fffffff);
+#pragma unroll
+    for (int o = 0; o < 8; ++o) m = max(m, __double2hiint(c.v[o]) & 0x7fffffff);
+    m = __reduce_max_sync(0xffffffffu, m);
+    if (lane == 0) atomicMax(smax + (q & 7), m);
+  };
+  auto put = [&](int q, int a, int col, int eb, const Cell& c) {
+    unsigned long long w[8];
+#pragma unroll
+    for (int o = 0; o < 8; ++o) w[o] = static_cast<unsigned long long>(to_fixed(c.v[o], eb)) + digit_bias();
+#pragma unroll
+    for (int j = 0; j < ND; ++j)
+      *reinterpret_cast<uint4*>(sm + SM::RING + (2 * (q % 3) + a) * ROWB + j * PLANE + col * 16) =
+          make_uint4(digit2(w[0], w[1], j), digit2(w[2], w[3], j), digit2(w[4], w[5], j), digit2(w[6], w[7], j));
+  };
+  auto put_p = [&](int s, int a, int col, int eb, const Cell& c) {
+    unsigned long long w[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) w[k] = static_cast<unsigned long long>(to_fixed(c.p[k], eb)) + digit_bias();
+#pragma unroll
+    for (int j = 0; j < ND; ++j)
+      *reinterpret_cast<unsigned*>(sm + SM::P + (s & 1) * ROWB + j * PLANE + col * 16 + 4 * a) = digit2(w[0], w[1], j);
+  };
+  auto largest = [&](int q) {   // |x| < 2^(e - 1022) over the pairs q - 1, q
+    const volatile int* vm = smax;
+    return max(vm[q & 7], vm[(q - 1) & 7]) >> 20;
+  };
+
+  // the first window (row pairs 0 and 1) by 18 warps at once
+  int eb;
+  {
+    const int q = warp / SLICE_WARPS, t = tid - q * SLICE_T;
+    const bool act = q < 2 && t < 2 * WCOLS;
+    const int a = t >= WCOLS ? 1 : 0, col = t - a * WCOLS;
+    Cell c;
+    if (q < 2) {
+      load(q, a, col, act, c);
+      note_max(q, c);
+    }
+    __syncthreads();
+    const int em = largest(1);
+    eb = min(max(em + 1, EB_MIN), 0x7ff);
+    if (act) {
+      put(q, a, col, eb, c);
+      if (q == 1) put_p(0, a, col, eb, c);
+    }
+    if (tid == 0) sexp[0] = em < 0x7ff ? eb : 0x7ff;
+    fence_proxy();
+    __syncthreads();
+  }
 
   const Shared C{bar_full, bar_done, bar_free, tmem, fail, sexp, i0, j0, rows, S};
   if (warp < EPI_WARPS / 2) {
@@ -204,106 +286,49 @@ __global__ void __launch_bounds__(NT, 1) k_apply_tc64(const Args A) {
   } else if (warp < EPI_WARPS) {
     epilogue<EPI_SPLIT, 9 - EPI_SPLIT>(A, C, warp, lane);
   } else if (warp < EPI_WARPS + SLICE_WARPS) {
-    // ---- values to digits: thread -> cell of the row pair ----
+    // ---- the row pairs after the first window ----
     const int t = tid - 32 * EPI_WARPS;
     const bool act = t < 2 * WCOLS;
-    const int a = t >= WCOLS ? 1 : 0, col = act ? t - a * WCOLS : 0, gi = i0 - 2 + col;
-    struct Cell {
-      double v[8];
-      double p[2];
-    };
-    auto load = [&](int q, Cell& c) {   // row pair q: cell rows j0 - 1 + 2 q + a; pressures j0 - 3 + 2 q + 2 a + {0, 1}
-      const int gj = j0 - 1 + 2 * q + a;
-#pragma unroll
-      for (int o = 0; o < 8; ++o) {
-        const int I = 2 * gi + (o & 1), J = 2 * gj + ((o >> 1) & 1);
-        c.v[o] = (act && is_free(I, J, nq)) ? A.x[(o >> 2) * nv + static_cast<long long>(J) * nq + I] : 0.0;
-      }
-#pragma unroll
-      for (int k = 0; k < 2; ++k) {
-        const int pj = j0 - 3 + 2 * q + 2 * a + k;
-        c.p[k] = (act && q >= 1 && gi >= 0 && gi <= n && pj >= 0 && pj <= n)
-                     ? A.x[2 * nv + static_cast<long long>(pj) * np + gi] : 0.0;
-      }
-    };
-    int eb = 0;
-    auto words = [&](const Cell& c, unsigned long long (&w)[8]) {
-#pragma unroll
-      for (int o = 0; o < 8; ++o) w[o] = static_cast<unsigned long long>(to_fixed(c.v[o], eb)) + digit_bias();
-    };
-    auto put = [&](int q, const unsigned long long (&w)[8]) {
-      if (!act) return;
-#pragma unroll
-      for (int j = 0; j < ND; ++j)
-        *reinterpret_cast<uint4*>(sm + SM::RING + (2 * (q % 3) + a) * ROWB + j * PLANE + col * 16) =
-            make_uint4(digit2(w[0], w[1], j), digit2(w[2], w[3], j), digit2(w[4], w[5], j), digit2(w[6], w[7], j));
-    };
+    const int a = t >= WCOLS ? 1 : 0, col = t - a * WCOLS;
     Cell cur;
-    load(0, cur);
-    for (int q = 0; q < S + 1; ++q) {
-      cur.p[0] *= A.ps;
-      cur.p[1] *= A.ps;
-      int m = max(__double2hiint(cur.p[0]) & 0x7fffffff, __double2hiint(cur.p[1]) & 0x7fffffff);
-#pragma unroll
-      for (int o = 0; o < 8; ++o) m = max(m, __double2hiint(cur.v[o]) & 0x7fffffff);
-      m = __reduce_max_sync(0xffffffffu, m);
-      if (lane == 0) atomicMax(smax + (q & 7), m);
+    if (S > 1) load(2, a, col, act, cur);
+    for (int q = 2; q < S + 1; ++q) {
+      note_max(q, cur);
       asm volatile("bar.sync 1, %0;" ::"n"(SLICE_T) : "memory");
       if (t == 0) smax[(q + 3) & 7] = 0;
-      if (q < 1) {
-        load(q + 1, cur);
-        continue;
-      }
-      const volatile int* vm = smax;
-      const int em = max(vm[q & 7], vm[(q - 1) & 7]) >> 20;   // |x| < 2^(em - 1022)
-      const int s = q - 1;
-      unsigned long long w[8];
-      const bool renew = s == 0 || em > eb || (eb - em > 3 && eb > EB_MIN);
+      const int em = largest(q), s = q - 1;
+      const bool renew = em > eb || (eb - em > 3 && eb > EB_MIN);
       if (renew) {   // uniform over the slicer warps: the other row pair again, with the new exponent
         eb = min(max(em + 1, EB_MIN), 0x7ff);
-        if (s > 0) mbar_wait_or_fail(bar_done + 8 * ((s - 1) % 3), ((s - 1) / 3) & 1, A.wait_limit, fail);
+        mbar_wait_or_fail(bar_done + 8 * ((s - 1) % 3), ((s - 1) / 3) & 1, A.wait_limit, fail);
         Cell c;
-        load(q - 1, c);
-        words(c, w);
-        put(q - 1, w);
+        load(q - 1, a, col, act, c);
+        if (act) put(q - 1, a, col, eb, c);
+      } else if (s >= 2) {
+        // the row pair's slot and the pressure buffer are free once step s - 2 has read them
+        // (after a failed wait the results are void and only the arrivals matter)
+        mbar_wait_or_fail(bar_done + 8 * ((s - 2) % 3), ((s - 2) / 3) & 1, A.wait_limit, fail);
       }
       if (t == 0) sexp[s & 3] = em < 0x7ff ? eb : 0x7ff;
-      words(cur, w);
-      unsigned long long wp[2];
-#pragma unroll
-      for (int k = 0; k < 2; ++k) wp[k] = static_cast<unsigned long long>(to_fixed(cur.p[k], eb)) + digit_bias();
-      if (q + 1 < S + 1) load(q + 1, cur);   // in flight while the planes are written
-      // the row pair's slot and the pressure buffer are free once step s - 2 has read them
-      // (after a failed wait the results are void and only the arrivals matter)
-      if (!renew && s >= 2) mbar_wait_or_fail(bar_done + 8 * ((s - 2) % 3), ((s - 2) / 3) & 1, A.wait_limit, fail);
-      put(q, w);
       if (act) {
-#pragma unroll
-        for (int j = 0; j < ND; ++j)
-          *reinterpret_cast<unsigned*>(sm + SM::P + (s & 1) * ROWB + j * PLANE + col * 16 + 4 * a) = digit2(wp[0], wp[1], j);
+        put(q, a, col, eb, cur);
+        put_p(s, a, col, eb, cur);
       }
+      if (q + 1 < S + 1) load(q + 1, a, col, act, cur);   // in flight over the fence and the next barrier
       fence_proxy();
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_full + 8 * (s % 3));
     }
   } else if (warp == EPI_WARPS + SLICE_WARPS) {
-    // ---- coefficients, then the MMAs ----
+    // ---- the MMAs ----
     const uint32_t on = elect_one();
-    if (on) {
-      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar_g), "r"(GBYTES) : "memory");
-      asm volatile(
-          "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(s0 + SM::G),
-          "l"(A.G), "r"(GBYTES), "r"(bar_g)
-          : "memory");
-    }
-    __syncwarp();
     auto wait = [&](uint32_t bar, uint32_t phase) {   // a vote, so that the loop stays uniform
       return __all_sync(0xffffffffu, mbar_wait_or_fail(bar, phase, A.wait_limit, fail)) != 0;
     };
     bool ok = wait(bar_g, 0);
     int issued = 0;
     for (int s = 0; s < S && ok; ++s) {
-      ok = wait(bar_full + 8 * (s % 3), (s / 3) & 1);
+      if (s > 0) ok = wait(bar_full + 8 * (s % 3), full_phase(s));   // step 0: the first window
       const int use = s >> 1;
       if (ok && use > 0) ok = wait(bar_free + 8 * (s & 1), (use - 1) & 1);
       if (!ok) break;

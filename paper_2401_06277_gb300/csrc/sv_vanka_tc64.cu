@@ -72,6 +72,7 @@ constexpr int KSTEPS = 17;
 constexpr int CHUNK = GROWS * 16;                // 8 K-values of all coefficient rows
 constexpr int GBYTES = 2 * KSTEPS * CHUNK + 32;  // + the two rows that N = 128 reads past the end
 static_assert(GBYTES == TC64_BYTES, "size of the packed coefficients");
+constexpr int RING_CTA_WARPS = 16, RING_PARTS_MAX_N = 512;
 constexpr int MMA_WARPS = 3, RING_WARPS = 4;   // MMA warp w: chains w and w + 3, one accumulator
 constexpr int NT = 32 * (EPI_WARPS + SLICE_WARPS + MMA_WARPS + RING_WARPS);
 
@@ -109,6 +110,7 @@ struct Args {
   double qu, qp;              // the same with the units of the digit sums
   double rps;                 // cl / cb
   double omega;
+  int strips, ctas;           // CTAs past `ctas` compute cells near the boundary only
   int steps_per_seg;
   int* err;
   int wait_limit;
@@ -155,14 +157,19 @@ __device__ __forceinline__ int cell_type(int n, const Band& b) {
   return b.in ? pos(b.j) * VS_POS + pos(b.i) : 0;
 }
 
+// PARTS = 1: a unit is four cells, a lane one output of one of them (162 multiply-adds
+// each: 10,000 clocks of a sub-partition's FP64 unit).  PARTS = 4: one cell, four lanes per
+// output, for the grids on which the longest unit, not the work, sets the time.
+template <int PARTS>
 __device__ __forceinline__ void ring_velocity(const Args& A, int unit, int lane) {
+  static_assert(PARTS == 1 || PARTS == 4, "lanes: 8 outputs x 4 cells or 4 parts");
   const LevelDev& L = A.L;
-  const int n = L.n, nq = L.nq, np = L.np, o = lane & 7;
+  const int n = L.n, nq = L.nq, np = L.np, o = lane & 7, part = PARTS == 4 ? lane >> 3 : 0;
   const long long nv = L.nv;
-  const Band b = band_of(n, unit, 4, lane >> 3);
+  const Band b = band_of(n, unit, 4 / PARTS, PARTS == 4 ? 0 : lane >> 3);
   const double* g = A.Gd + static_cast<size_t>(cell_type(n, b)) * RT_TYPE + o;
   double a0 = 0.0, a1 = 0.0;
-  for (int rJ = b.J0; rJ <= b.J1; ++rJ) {
+  for (int rJ = b.J0 + part; rJ <= b.J1; rJ += PARTS) {
     const int J = 2 * b.j - 4 + rJ;
     const double* rr = A.r + static_cast<long long>(J) * nq + 2 * b.i - 4;
     const double* gr = g + rJ * 144;
@@ -176,17 +183,22 @@ __device__ __forceinline__ void ring_velocity(const Args& A, int unit, int lane)
   }
   double ap = 0.0;
 #pragma unroll
-  for (int k = 0; k < 9; ++k) {
+  for (int k = part; k < 9; k += PARTS) {
     const int pi = b.i + k % 3 - 1, pj = b.j + k / 3 - 1;
     const bool ok = b.in && pi >= 0 && pj >= 0 && pi <= n && pj <= n;
     const double r0 = ok ? __ldg(A.r + 2 * nv + static_cast<long long>(pj) * np + pi) : 0.0;
     ap = fma(__ldg(g + 162 * 8 + k * 8), r0, ap);
   }
+  double d = fma(A.rps, ap, a0 + a1);
+  if (PARTS == 4) {
+    d += __shfl_xor_sync(0xffffffffu, d, 8);
+    d += __shfl_xor_sync(0xffffffffu, d, 16);
+  }
   const int I = 2 * b.i + (o & 1), J = 2 * b.j + ((o >> 1) & 1);
-  if (!b.in || I >= nq || J >= nq) return;
+  if (part != 0 || !b.in || I >= nq || J >= nq) return;
   const long long k = (o >> 2) * nv + static_cast<long long>(J) * nq + I;
   const double xv = A.x != nullptr ? A.x[k] : 0.0;
-  A.xo[k] = is_free(I, J, nq) ? fma(A.su, fma(A.rps, ap, a0 + a1), xv) : fma(A.omega, A.r[k], xv);
+  A.xo[k] = is_free(I, J, nq) ? fma(A.su, d, xv) : fma(A.omega, A.r[k], xv);
 }
 
 __device__ __forceinline__ void ring_pressure(const Args& A, int unit, int lane) {
@@ -212,6 +224,17 @@ __device__ __forceinline__ void ring_pressure(const Args& A, int unit, int lane)
   const long long k = 2 * nv + static_cast<long long>(b.j) * L.np + b.i;
   const double d = fma(A.rps * __ldg(g + 50), A.r[k], a0 + a1);
   A.xo[k] = fma(A.sp, d, A.x != nullptr ? A.x[k] : 0.0);
+}
+
+// All units, dealt to `slots` warps.
+__device__ __forceinline__ void ring(const Args& A, int slot, int slots, int lane) {
+  const int n = A.L.n, wide = n > RING_PARTS_MAX_N;
+  const int uv = ring_units(n, wide ? 4 : 1), up = ring_units(n, 32);
+  for (int u = slot; u < uv + up; u += slots) {
+    if (u >= uv) ring_pressure(A, u - uv, lane);
+    else if (wide) ring_velocity<1>(A, u, lane);
+    else ring_velocity<4>(A, u, lane);
+  }
 }
 
 // T += D 2^k for the weights of the digit pairs; the compiler makes it one IMAD.WIDE
@@ -301,8 +324,14 @@ __global__ void __launch_bounds__(NT, 1) k_vanka_tc64(const Args A) {
   volatile int* fail = reinterpret_cast<volatile int*>(sm + SM::MISC + 4);
   int* smax = reinterpret_cast<int*>(sm + SM::MISC + 8);                    // 8 slots
   volatile int* sexp = reinterpret_cast<volatile int*>(sm + SM::MISC + 40);   // 4 slots
-  const int i0 = 3 + COLS * static_cast<int>(blockIdx.x);
-  const int j0 = 3 + 2 * A.steps_per_seg * static_cast<int>(blockIdx.y);
+  if (static_cast<int>(blockIdx.x) >= A.ctas) {
+    if (warp < RING_CTA_WARPS)
+      ring(A, RING_WARPS * A.ctas + (blockIdx.x - A.ctas) * RING_CTA_WARPS + warp,
+           RING_WARPS * A.ctas + (gridDim.x - A.ctas) * RING_CTA_WARPS, lane);
+    return;
+  }
+  const int i0 = 3 + COLS * (static_cast<int>(blockIdx.x) % A.strips);
+  const int j0 = 3 + 2 * A.steps_per_seg * (static_cast<int>(blockIdx.x) / A.strips);
   const int rows = min(2 * A.steps_per_seg, n - 2 - j0);   // owned cell rows, up to n - 3
   const int S = (rows + 1) / 2;
 
@@ -319,7 +348,6 @@ __global__ void __launch_bounds__(NT, 1) k_vanka_tc64(const Args A) {
   }
   for (int k = tid; k < ROWB / 16; k += NT)   // channels 4..7 of the pressures stay zero
     reinterpret_cast<uint4*>(sm + SM::P)[k] = make_uint4(0u, 0u, 0u, 0u);
-  fence_proxy();
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tslot)), "r"(512));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
@@ -328,6 +356,90 @@ __global__ void __launch_bounds__(NT, 1) k_vanka_tc64(const Args A) {
   __syncthreads();
   fence_after();
   const uint32_t tmem = *tslot;
+  if (tid == 0) {   // the coefficients, while the first window is loaded
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar_g), "r"(GBYTES) : "memory");
+    asm volatile(
+        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(s0 + SM::G),
+        "l"(A.G), "r"(GBYTES), "r"(bar_g)
+        : "memory");
+  }
+
+  // ---- residuals to digits: a thread takes a cell (a, col) of a row pair q ----
+  struct Cell {
+    double v[8];
+    double p[2];
+  };
+  auto load = [&](int q, int a, int col, bool act, Cell& c) {   // cell row j0 - 2 + 2 q + a; pressures j0 - 5 + 2 q + 2 a + {0, 1}
+    const int gi = i0 - 2 + col, gj = j0 - 2 + 2 * q + a;
+    const bool in = act && gi <= n && gj <= n;
+#pragma unroll
+    for (int o = 0; o < 8; ++o) {
+      const int I = 2 * gi + (o & 1), J = 2 * gj + ((o >> 1) & 1);
+      c.v[o] = (in && I < nq - 1 && J < nq - 1) ? A.r[(o >> 2) * nv + static_cast<long long>(J) * nq + I] : 0.0;
+    }
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int pj = j0 - 5 + 2 * q + 2 * a + k;
+      c.p[k] = (act && q >= 2 && gi <= n && pj <= n) ? A.r[2 * nv + static_cast<long long>(pj) * np + gi] : 0.0;
+    }
+  };
+  auto note_max = [&](int q, Cell& c) {   // pressures to their units; the pair's largest exponent
+    c.p[0] *= A.rps;
+    c.p[1] *= A.rps;
+    int m = max(__double2hiint(c.p[0]) & 0x7fffffff, __double2hiint(c.p[1]) & 0x7fffffff);
+#pragma unroll
+    for (int o = 0; o < 8; ++o) m = max(m, __double2hiint(c.v[o]) & 0x7fffffff);
+    m = __reduce_max_sync(0xffffffffu, m);
+    if (lane == 0) atomicMax(smax + (q & 7), m);
+  };
+  auto words = [&](const Cell& c, int eb, unsigned long long (&w)[8]) {
+#pragma unroll
+    for (int o = 0; o < 8; ++o) w[o] = static_cast<unsigned long long>(to_fixed(c.v[o], eb)) + digit_bias();
+  };
+  auto words_p = [&](const Cell& c, int eb, unsigned long long (&w)[2]) {
+#pragma unroll
+    for (int k = 0; k < 2; ++k) w[k] = static_cast<unsigned long long>(to_fixed(c.p[k], eb)) + digit_bias();
+  };
+  auto put = [&](int q, int a, int col, int j, const unsigned long long (&w)[8]) {
+    *reinterpret_cast<uint4*>(sm + SM::RING + (2 * (q % 3) + a) * ROWB + j * PLANE + col * 16) =
+        make_uint4(digit2(w[0], w[1], j), digit2(w[2], w[3], j), digit2(w[4], w[5], j), digit2(w[6], w[7], j));
+  };
+  auto put_p = [&](int a, int col, int j, const unsigned long long (&w)[2]) {
+    *reinterpret_cast<unsigned*>(sm + SM::P + j * PLANE + col * 16 + 4 * a) = digit2(w[0], w[1], j);
+  };
+  auto largest = [&](int q) {   // |x| < 2^(e - 1022) over the pairs q - 2 .. q
+    const volatile int* vm = smax;
+    return max(vm[q & 7], max(vm[(q - 1) & 7], vm[(q - 2) & 7])) >> 20;
+  };
+
+  // the first window (row pairs 0, 1, 2) by 27 warps at once
+  int eb;
+  {
+    const int q = warp / SLICE_WARPS, t = tid - q * SLICE_T;
+    const bool act = q < 3 && t < 2 * WCOLS;
+    const int a = t >= WCOLS ? 1 : 0, col = t - a * WCOLS;
+    Cell c;
+    if (q < 3) {
+      load(q, a, col, act, c);
+      note_max(q, c);
+    }
+    __syncthreads();
+    const int em = largest(2);
+    eb = min(max(em + 1, EB_MIN), 0x7ff);
+    if (act) {
+      unsigned long long w[8], wp[2];
+      words(c, eb, w);
+      words_p(c, eb, wp);
+#pragma unroll
+      for (int j = 0; j < ND; ++j) {
+        put(q, a, col, j, w);
+        if (q == 2) put_p(a, col, j, wp);
+      }
+    }
+    if (tid == 0) sexp[0] = em < 0x7ff ? eb : 0x7ff;
+    fence_proxy();
+    __syncthreads();
+  }
 
   const Shared C{bar_full, bar_done, bar_free, tmem, fail, sexp, i0, j0, rows, S};
   if (warp < EPI_WARPS / 2) {
@@ -335,101 +447,53 @@ __global__ void __launch_bounds__(NT, 1) k_vanka_tc64(const Args A) {
   } else if (warp < EPI_WARPS) {
     epilogue<EPI_SPLIT, 9 - EPI_SPLIT>(A, C, warp, lane);
   } else if (warp < EPI_WARPS + SLICE_WARPS) {
-    // ---- residuals to digits: thread -> cell of the row pair ----
+    // ---- the row pairs after the first window ----
     const int t = tid - 32 * EPI_WARPS;
     const bool act = t < 2 * WCOLS;
-    const int a = t >= WCOLS ? 1 : 0, col = act ? t - a * WCOLS : 0, gi = i0 - 2 + col;
-    struct Cell {
-      double v[8];
-      double p[2];
-    };
-    auto load = [&](int q, Cell& c) {   // row pair q: cell rows j0 - 2 + 2 q + a; pressures j0 - 5 + 2 q + 2 a + {0, 1}
-      const int gj = j0 - 2 + 2 * q + a;
-      const bool in = act && gi <= n && gj <= n;
-#pragma unroll
-      for (int o = 0; o < 8; ++o) {
-        const int I = 2 * gi + (o & 1), J = 2 * gj + ((o >> 1) & 1);
-        c.v[o] = (in && I < nq - 1 && J < nq - 1) ? A.r[(o >> 2) * nv + static_cast<long long>(J) * nq + I] : 0.0;
-      }
-#pragma unroll
-      for (int k = 0; k < 2; ++k) {
-        const int pj = j0 - 5 + 2 * q + 2 * a + k;
-        c.p[k] = (act && q >= 2 && gi <= n && pj <= n)
-                     ? A.r[2 * nv + static_cast<long long>(pj) * np + gi] : 0.0;
-      }
-    };
-    int eb = 0;
-    auto words = [&](const Cell& c, unsigned long long (&w)[8]) {
-#pragma unroll
-      for (int o = 0; o < 8; ++o) w[o] = static_cast<unsigned long long>(to_fixed(c.v[o], eb)) + digit_bias();
-    };
-    auto put = [&](int q, int j, const unsigned long long (&w)[8]) {
-      if (!act) return;
-      const uint4 d = make_uint4(digit2(w[0], w[1], j), digit2(w[2], w[3], j), digit2(w[4], w[5], j), digit2(w[6], w[7], j));
-      *reinterpret_cast<uint4*>(sm + SM::RING + (2 * (q % 3) + a) * ROWB + j * PLANE + col * 16) = d;
-    };
+    const int a = t >= WCOLS ? 1 : 0, col = t - a * WCOLS;
     Cell cur;
-    load(0, cur);
-    for (int q = 0; q < S + 2; ++q) {
-      cur.p[0] *= A.rps;
-      cur.p[1] *= A.rps;
-      int m = 0;
-#pragma unroll
-      for (int o = 0; o < 8; ++o) m = max(m, __double2hiint(cur.v[o]) & 0x7fffffff);
-      m = max(m, max(__double2hiint(cur.p[0]) & 0x7fffffff, __double2hiint(cur.p[1]) & 0x7fffffff));
-      m = __reduce_max_sync(0xffffffffu, m);
-      if (lane == 0) atomicMax(smax + (q & 7), m);
+    if (S > 1) load(3, a, col, act, cur);
+    for (int q = 3; q < S + 2; ++q) {
+      note_max(q, cur);
       asm volatile("bar.sync 1, %0;" ::"n"(SLICE_T) : "memory");
       if (t == 0) smax[(q + 3) & 7] = 0;
-      if (q < 2) {
-        load(q + 1, cur);
-        continue;
-      }
-      const volatile int* vm = smax;
-      const int em = max(vm[q & 7], max(vm[(q - 1) & 7], vm[(q - 2) & 7])) >> 20;   // |x| < 2^(em - 1022)
-      const int s = q - 2;
-      unsigned long long w[8];
-      const bool renew = s == 0 || em > eb || (eb - em > 3 && eb > EB_MIN);
-      if (renew) {   // uniform over the slicer warps
+      const int em = largest(q), s = q - 2;
+      unsigned long long w[8], wp[2];
+      const bool renew = em > eb || (eb - em > 3 && eb > EB_MIN);
+      if (renew) {   // uniform over the slicer warps: the window again, once the step before has read it
         eb = min(max(em + 1, EB_MIN), 0x7ff);
-        if (s > 0) mbar_wait_or_fail(bar_done + 8 * (ND - 1), (s - 1) & 1, A.wait_limit, fail);
+        mbar_wait_or_fail(bar_done + 8 * (ND - 1), (s - 1) & 1, A.wait_limit, fail);
         for (int qq = q - 2; qq < q; ++qq) {
           Cell c;
-          load(qq, c);
-          words(c, w);
+          load(qq, a, col, act, c);
+          words(c, eb, w);
+          if (act) {
 #pragma unroll
-          for (int j = 0; j < ND; ++j) put(qq, j, w);
+            for (int j = 0; j < ND; ++j) put(qq, a, col, j, w);
+          }
         }
       }
       if (t == 0) sexp[s & 3] = em < 0x7ff ? eb : 0x7ff;
-      words(cur, w);
-      unsigned long long wp[2];
-#pragma unroll
-      for (int k = 0; k < 2; ++k) wp[k] = static_cast<unsigned long long>(to_fixed(cur.p[k], eb)) + digit_bias();
-      if (q + 1 < S + 2) load(q + 1, cur);   // in flight while the planes are written
+      words(cur, eb, w);
+      words_p(cur, eb, wp);
+      if (q + 1 < S + 2) load(q + 1, a, col, act, cur);   // in flight while the planes are written
 #pragma unroll
       for (int j = 0; j < ND; ++j) {
         // plane j of the row pair is free once chain j of the step before has read it (after
         // a failed wait the results are void and only the arrivals matter)
         if (!renew) mbar_wait_or_fail(bar_done + 8 * j, (s - 1) & 1, A.wait_limit, fail);
-        put(q, j, w);
-        if (act) *reinterpret_cast<unsigned*>(sm + SM::P + j * PLANE + col * 16 + 4 * a) = digit2(wp[0], wp[1], j);
+        if (act) {
+          put(q, a, col, j, w);
+          put_p(a, col, j, wp);
+        }
         fence_proxy();
         __syncwarp();
         if (lane == 0) mbar_arrive(bar_full + 8 * j);
       }
     }
   } else if (warp < EPI_WARPS + SLICE_WARPS + MMA_WARPS) {
-    // ---- coefficients, then the MMAs ----
+    // ---- the MMAs ----
     const uint32_t on = elect_one();
-    if (on && warp == EPI_WARPS + SLICE_WARPS) {
-      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar_g), "r"(GBYTES) : "memory");
-      asm volatile(
-          "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(s0 + SM::G),
-          "l"(A.G), "r"(GBYTES), "r"(bar_g)
-          : "memory");
-    }
-    __syncwarp();
     auto wait = [&](uint32_t bar, uint32_t phase) {   // a vote, so that the loop stays uniform
       return __all_sync(0xffffffffu, mbar_wait_or_fail(bar, phase, A.wait_limit, fail)) != 0;
     };
@@ -444,7 +508,7 @@ __global__ void __launch_bounds__(NT, 1) k_vanka_tc64(const Args A) {
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const int c = w + MMA_WARPS * h;
-        if (ok) ok = wait(bar_full + 8 * c, s & 1);
+        if (ok && s > 0) ok = wait(bar_full + 8 * c, (s - 1) & 1);   // step 0: the first window
         const int use = 2 * s + h;   // earlier chains of this accumulator
         if (ok && use > 0) ok = wait(bar_free + 8 * w, (use - 1) & 1);
         if (!ok) break;
@@ -471,13 +535,9 @@ __global__ void __launch_bounds__(NT, 1) k_vanka_tc64(const Args A) {
     mbar_wait(bar_g, 0, TC_WAIT_LIMIT);
     __syncwarp();
   } else {
-    // ---- cells near the boundary: units dealt to the ring warps of all CTAs ----
-    const int ctas = gridDim.x * gridDim.y, cta = blockIdx.y * gridDim.x + blockIdx.x;
-    const int uv = ring_units(n, 4), up = ring_units(n, 32);
-    for (int u = (warp - (EPI_WARPS + SLICE_WARPS + MMA_WARPS)) * ctas + cta; u < uv + up; u += RING_WARPS * ctas) {
-      if (u < uv) ring_velocity(A, u, lane);
-      else ring_pressure(A, u - uv, lane);
-    }
+    // ---- cells near the boundary ----
+    ring(A, (warp - (EPI_WARPS + SLICE_WARPS + MMA_WARPS)) * A.ctas + blockIdx.x,
+         RING_WARPS * A.ctas + (gridDim.x - A.ctas) * RING_CTA_WARPS, lane);
   }
   __syncwarp();
   fence_before();
@@ -555,11 +615,13 @@ void launch_vanka_tc64(const LevelDev& L, const unsigned char* Gp, int eu, int e
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int cells = L.n - 5, strips = (cells + COLS - 1) / COLS, steps = (cells + 1) / 2;
   const int seg = segment_steps(strips, steps, sms, 4);
+  // SMs left over compute cells near the boundary
+  const int ctas = strips * ((steps + seg - 1) / seg), extra = ctas < sms ? sms - ctas : 0;
   Args A{L, Gp, Gd, x, r, xo, omega / L.cl, omega / L.cb, std::ldexp(omega / L.cl, eu), std::ldexp(omega / L.cb, ep),
-         L.cl / L.cb, omega, seg, err, wait_limit};
+         L.cl / L.cb, omega, strips, ctas, seg, err, wait_limit};
   count_launches(1);
   g_tc_launches.fetch_add(1, std::memory_order_relaxed);
-  launch_pdl(k_vanka_tc64, dim3(strips, (steps + seg - 1) / seg), dim3(NT), SM::BYTES, s, A);
+  launch_pdl(k_vanka_tc64, dim3(ctas + extra), dim3(NT), SM::BYTES, s, A);
 }
 
 }  // namespace sv
