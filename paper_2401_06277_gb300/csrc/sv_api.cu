@@ -99,6 +99,10 @@ void free_all(stokes_hierarchy* h) {
   h->delta = nullptr;
   cudaFree(h->deltaf);
   h->deltaf = nullptr;
+  cudaFree(const_cast<double*>(h->bs.tab));
+  cudaFree(const_cast<float*>(h->bs.tabf));
+  h->bs.tab = nullptr;
+  h->bs.tabf = nullptr;
   cudaFree(h->bs_buf);
   h->bs_buf = nullptr;
   cudaFree(h->bt_GL);
@@ -1001,6 +1005,16 @@ stokes_status stokes_hierarchy_create(int n, double viscosity, const stokes_para
                              prm.smoother == STOKES_SMOOTHER_SCHUR_UZAWA) && k + 1 == sizes.size()) {
       const size_t el = sv::bs_scratch_elems(L.d) * (prm.prec == STOKES_FP64 ? sizeof(double) : sizeof(float));
       e = dalloc_bytes(&h->bs_buf, el);
+      const std::vector<double> tab = sv::bs_schur_table();
+      const std::vector<float> tabf(tab.begin(), tab.end());
+      double* td = nullptr;
+      float* tf = nullptr;
+      if (e == cudaSuccess) e = dalloc(&td, tab.size());
+      h->bs.tab = td;
+      if (e == cudaSuccess) e = dalloc(&tf, tabf.size());
+      h->bs.tabf = tf;
+      if (e == cudaSuccess) e = cudaMemcpy(td, tab.data(), tab.size() * sizeof(double), cudaMemcpyHostToDevice);
+      if (e == cudaSuccess) e = cudaMemcpy(tf, tabf.data(), tabf.size() * sizeof(float), cudaMemcpyHostToDevice);
     }
     if (e == cudaSuccess && prm.prec != STOKES_FP64) {
       std::vector<float> cdf(L.cd_host.begin(), L.cd_host.end());

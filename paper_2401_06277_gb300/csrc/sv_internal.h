@@ -110,7 +110,14 @@ constexpr int TC_WAIT_LIMIT = 1 << 22;   // polls of an mbarrier before a tensor
 constexpr int TAIL_SPIN_LIMIT = 1 << 22;   // polls (about 64 ns apart) of a grid barrier before it gives up
 
 
+// Schur complement stencils of the vertices near the boundary (sv_bs.cu): by axis class of
+// the vertex, 25 coefficients and the reciprocal of the diagonal, integer units
+constexpr int BS_TYPE = 26, BS_TAB = NCLASS * BS_TYPE;
+std::vector<double> bs_schur_table();
+
 struct BSParams {
+  const double* tab = nullptr;    // bs_schur_table on the device, in FP64
+  const float* tabf = nullptr;    // and in FP32
   double t = 1.0, omega = 1.0, jacobi_weight = 1.0;
   int jacobi_iters = 2;
   bool uzawa = false;   // Schur-Uzawa (Algorithm 4): no B^T dp in the velocity update
@@ -414,7 +421,7 @@ void launch_coarse(const double* G, int N0, const double* r, double* e, cudaStre
 cudaError_t vanka_prepare();
 
 // ---- Braess-Sarazin relaxation (sv_bs.cu) ----
-size_t bs_scratch_elems(const LevelDev& L);   // 2 nv + 3 np^2
+size_t bs_scratch_elems(const LevelDev& L);   // 3 np^2
 // x_out = x + omega (du, dp) (Algorithm 2); x may be nullptr (zero guess);
 // rbuf (level size) receives b - A x; scratch holds bs_scratch_elems(L)
 template <typename T>

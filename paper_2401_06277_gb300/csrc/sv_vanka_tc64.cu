@@ -72,7 +72,7 @@ constexpr int KSTEPS = 17;
 constexpr int CHUNK = GROWS * 16;                // 8 K-values of all coefficient rows
 constexpr int GBYTES = 2 * KSTEPS * CHUNK + 32;  // + the two rows that N = 128 reads past the end
 static_assert(GBYTES == TC64_BYTES, "size of the packed coefficients");
-constexpr int RING_CTA_WARPS = 16, RING_PARTS_MAX_N = 512;
+constexpr int RING_CTA_WARPS = 16, RING_PARTS_MAX_N = 256;
 constexpr int MMA_WARPS = 3, RING_WARPS = 4;   // MMA warp w: chains w and w + 3, one accumulator
 constexpr int NT = 32 * (EPI_WARPS + SLICE_WARPS + MMA_WARPS + RING_WARPS);
 
