@@ -50,7 +50,7 @@ struct SM {
   static constexpr int RING = 0;                 // 3 row pairs
   static constexpr int P = RING + 6 * ROWB;      // pressures of a step, two buffers
   static constexpr int G = P + 2 * ROWB;
-  static constexpr int BAR = G + GBYTES;         // full[3], done[3], free[2], gload
+  static constexpr int BAR = G + GBYTES;         // full[3], done[2], free[2], gload
   static constexpr int MISC = BAR + 16 * 8;      // tmem slot, fail flag, 8 maxima, 4 exponents
   static constexpr int BYTES = MISC + 4 * 16;
   static_assert(G % 128 == 0 && BAR % 8 == 0, "shared memory");
@@ -98,63 +98,83 @@ struct Shared {   // what the roles of a CTA share
   int i0, j0, rows, S;
 };
 
-// Accumulators to y for the outputs O0 .. O0 + NO - 1: warp -> cell row a and lane
-// quarter of the columns.
-template <int O0, int NO>
-__device__ __forceinline__ void epilogue(const Args& A, const Shared& C, int warp, int lane) {
+// Accumulators to y, steps g, g + 2, ...: warp -> cell row a and lane quarter of the
+// columns.  The digit sums have weights 2^(50 - 10 c), taken in units of 2^7 (velocity
+// rows: the coefficients sum to 1300 at most, |T| < 2^62) and 2^2 (pressure rows: 60).
+__device__ __forceinline__ void epilogue(const Args& A, const Shared& C, int g, int warp, int lane) {
   const LevelDev& L = A.L;
   const int n = L.n, nq = L.nq, np = L.np;
   const long long nv = L.nv;
   const int a = (warp >> 2) & 1, i = C.i0 + 32 * (warp & 3) + lane;
-  const uint32_t tq = C.tmem + (static_cast<uint32_t>(32 * (warp & 3)) << 16) + 16 * a + O0;
-  for (int s = 0; s < C.S; ++s) {
-    const int j = C.j0 + 2 * s + a;
-    const bool own = i <= n && 2 * s + a < C.rows;
-    const long long ku = static_cast<long long>(2 * j) * nq + 2 * i;
-    const long long kp = 2 * nv + static_cast<long long>(j) * np + i;
-    auto at = [&](int o) { return o == 8 ? kp : (o >> 2) * nv + ku + ((o >> 1) & 1) * nq + (o & 1); };
-    auto exists = [&](int o) { return own && (o == 8 || ((i < n || !(o & 1)) && (j < n || !(o & 2)))); };
-    double bv[NO];
-#pragma unroll
-    for (int o = 0; o < NO; ++o) bv[o] = exists(O0 + o) && A.b != nullptr ? A.b[at(O0 + o)] : 0.0;
-    const bool ok = mbar_wait_or_fail(C.done + 8 * (s % 3), (s / 3) & 1, A.wait_limit, C.fail);
+  const uint32_t tq = C.tmem + (static_cast<uint32_t>(32 * (warp & 3)) << 16) + 16 * a + 256 * g;
+  for (int s = g; s < C.S; s += 2) {
+    const bool ok = mbar_wait_or_fail(C.done + 8 * g, (s >> 1) & 1, A.wait_limit, C.fail);
     if (!__all_sync(0xffffffffu, ok)) return;
     fence_after();
-    long long hi[NO], lo[NO];
+    long long T[9];
+    {
+      uint32_t v[3][9];
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      uint32_t v[3][NO];
-#pragma unroll
-      for (int c = 0; c < 3; ++c) tmem_ldn<NO>(tq + 256 * (s & 1) + NB * (3 * h + c), v[c]);
+      for (int c = 0; c < 3; ++c) tmem_ld9(tq + NB * c, v[c]);
       wait_ld();
 #pragma unroll
-      for (int o = 0; o < NO; ++o) {
-        const int d0 = __float2int_rn(__uint_as_float(v[0][o])), d1 = __float2int_rn(__uint_as_float(v[1][o])),
-                  d2 = __float2int_rn(__uint_as_float(v[2][o]));
-        // |d| < 2^20: the first two fit 32 bits
-        const long long t = static_cast<long long>(d0 * 1024 + d1) * 1024 + d2;
-        if (h == 0) hi[o] = t;
-        else lo[o] = t;
+      for (int o = 0; o < 9; ++o) T[o] = 0;
+#pragma unroll
+      for (int o = 0; o < 8; ++o) {
+        add_digit<43>(T[o], v[0][o]);
+        add_digit<33>(T[o], v[1][o]);
+        add_digit<23>(T[o], v[2][o]);
       }
+      add_digit<48>(T[8], v[0][8]);
+      add_digit<38>(T[8], v[1][8]);
+      add_digit<28>(T[8], v[2][8]);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) tmem_ld9(tq + NB * (3 + c), v[c]);
+      wait_ld();
+#pragma unroll
+      for (int o = 0; o < 8; ++o) {
+        add_digit<13>(T[o], v[0][o]);
+        add_digit<3>(T[o], v[1][o]);
+        add_digit<-7>(T[o], v[2][o]);
+      }
+      add_digit<18>(T[8], v[0][8]);
+      add_digit<8>(T[8], v[1][8]);
+      add_digit<-2>(T[8], v[2][8]);
     }
     fence_before();
     __syncwarp();
-    if (lane == 0) mbar_arrive(C.free + 8 * (s & 1));
+    if (lane == 0) mbar_arrive(C.free + 8 * g);
+    const int j = C.j0 + 2 * s + a;
+    if (i > n || 2 * s + a >= C.rows) continue;
     const int eb = C.sexp[s & 3];
     if (eb == 0x7ff) {
-      if (own)
-        for (int o = 0; o < NO; ++o) apply_cell(A, i, j, O0 + o);
+      for (int o = 0; o < 9; ++o) apply_cell(A, i, j, o);
       continue;
     }
-    const double sc = exp_scale(eb, -58), su = L.cl * sc, sp = L.cb * sc;
+    const long long ku = static_cast<long long>(2 * j) * nq + 2 * i;
+    const long long kp = 2 * nv + static_cast<long long>(j) * np + i;
+    auto at = [&](int o) { return (o >> 2) * nv + ku + ((o >> 1) & 1) * nq + (o & 1); };
+    const bool res = A.b != nullptr;
+    const double su = (res ? -L.cl : L.cl) * exp_scale(eb, -51), sp = (res ? -L.cb : L.cb) * exp_scale(eb, -56);
+    if (i >= 1 && j >= 1 && i <= n - 1 && j <= n - 1) {   // all four nodes exist and are free
+      double bv[9];
 #pragma unroll
-    for (int o = 0; o < NO; ++o) {
-      const int oo = O0 + o;
-      if (!exists(oo)) continue;
-      const double d = to_double(hi[o], lo[o]), f = oo == 8 ? sp : su;
-      const long long k = at(oo);
-      if (oo == 8 || is_free(2 * i + (oo & 1), 2 * j + ((oo >> 1) & 1), nq)) A.y[k] = fma(A.b != nullptr ? -f : f, d, bv[o]);
-      else A.y[k] = A.b != nullptr ? bv[o] - A.x[k] : A.x[k];   // Dirichlet row: identity
+      for (int o = 0; o < 8; ++o) bv[o] = res ? A.b[at(o)] : 0.0;
+      bv[8] = res ? A.b[kp] : 0.0;
+#pragma unroll
+      for (int o = 0; o < 8; ++o) A.y[at(o)] = fma(su, to_double(T[o]), bv[o]);
+      A.y[kp] = fma(sp, to_double(T[8]), bv[8]);
+    } else {
+#pragma unroll
+      for (int o = 0; o < 8; ++o) {
+        const int I = 2 * i + (o & 1), J = 2 * j + ((o >> 1) & 1);
+        if (I >= nq || J >= nq) continue;
+        const long long k = at(o);
+        const double b0 = res ? A.b[k] : 0.0;
+        if (is_free(I, J, nq)) A.y[k] = fma(su, to_double(T[o]), b0);
+        else A.y[k] = res ? b0 - A.x[k] : A.x[k];   // Dirichlet row: identity
+      }
+      A.y[kp] = fma(sp, to_double(T[8]), res ? A.b[kp] : 0.0);
     }
   }
 }
@@ -182,8 +202,8 @@ __global__ void __launch_bounds__(NT, 1) k_apply_tc64(const Args A) {
       mbar_init(bar_full + 8 * k, SLICE_WARPS);
       mbar_init(bar_done + 8 * k, 1);
     }
-    mbar_init(bar_free, EPI_WARPS);
-    mbar_init(bar_free + 8, EPI_WARPS);
+    mbar_init(bar_free, EPI_GROUP);
+    mbar_init(bar_free + 8, EPI_GROUP);
     mbar_init(bar_g, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     *fail = 0;
@@ -281,10 +301,8 @@ __global__ void __launch_bounds__(NT, 1) k_apply_tc64(const Args A) {
   }
 
   const Shared C{bar_full, bar_done, bar_free, tmem, fail, sexp, i0, j0, rows, S};
-  if (warp < EPI_WARPS / 2) {
-    epilogue<0, EPI_SPLIT>(A, C, warp, lane);
-  } else if (warp < EPI_WARPS) {
-    epilogue<EPI_SPLIT, 9 - EPI_SPLIT>(A, C, warp, lane);
+  if (warp < EPI_WARPS) {
+    epilogue(A, C, warp / EPI_GROUP, warp, lane);
   } else if (warp < EPI_WARPS + SLICE_WARPS) {
     // ---- the row pairs after the first window ----
     const int t = tid - 32 * EPI_WARPS;
@@ -300,14 +318,14 @@ __global__ void __launch_bounds__(NT, 1) k_apply_tc64(const Args A) {
       const bool renew = em > eb || (eb - em > 3 && eb > EB_MIN);
       if (renew) {   // uniform over the slicer warps: the other row pair again, with the new exponent
         eb = min(max(em + 1, EB_MIN), 0x7ff);
-        mbar_wait_or_fail(bar_done + 8 * ((s - 1) % 3), ((s - 1) / 3) & 1, A.wait_limit, fail);
+        mbar_wait_or_fail(bar_done + 8 * ((s - 1) & 1), ((s - 1) >> 1) & 1, A.wait_limit, fail);
         Cell c;
         load(q - 1, a, col, act, c);
         if (act) put(q - 1, a, col, eb, c);
       } else if (s >= 2) {
         // the row pair's slot and the pressure buffer are free once step s - 2 has read them
         // (after a failed wait the results are void and only the arrivals matter)
-        mbar_wait_or_fail(bar_done + 8 * ((s - 2) % 3), ((s - 2) / 3) & 1, A.wait_limit, fail);
+        mbar_wait_or_fail(bar_done + 8 * (s & 1), ((s - 2) >> 1) & 1, A.wait_limit, fail);
       }
       if (t == 0) sexp[s & 3] = em < 0x7ff ? eb : 0x7ff;
       if (act) {
@@ -350,11 +368,11 @@ __global__ void __launch_bounds__(NT, 1) k_apply_tc64(const Args A) {
         for (int e = 0; e < 2; ++e, ++k)   // pressures, dx = (-1, 0) and (1, none)
           mma_f16(on, d, pl + off + 2 * e, gl + k * (CHUNK / 8), IDESC, 1);
       }
-      mma_commit(on, bar_done + 8 * (s % 3));
+      mma_commit(on, bar_done + 8 * (s & 1));
       ++issued;
     }
     // every chain that was issued has completed before the operands and tensor memory go
-    if (issued > 0 && !mbar_wait(bar_done + 8 * ((issued - 1) % 3), ((issued - 1) / 3) & 1, TC_WAIT_LIMIT)) *fail = 1;
+    if (issued > 0 && !mbar_wait(bar_done + 8 * ((issued - 1) & 1), ((issued - 1) >> 1) & 1, TC_WAIT_LIMIT)) *fail = 1;
     mbar_wait(bar_g, 0, TC_WAIT_LIMIT);
     __syncwarp();
   } else {

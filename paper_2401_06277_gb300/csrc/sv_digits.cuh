@@ -23,8 +23,9 @@ constexpr int ND = 6;                            // digits of a value
 constexpr int PLANE = WCOLS * 16;                // one digit of one cell row
 constexpr int ROWB = ND * PLANE;                 // a cell row
 // Warp roles.  Accumulators to results: two groups of eight warps (cell row, lane
-// quarter), the first the outputs 0..4 of a cell, the second 5..8; values to digits: nine.
-constexpr int EPI_WARPS = 16, EPI_SPLIT = 5, SLICE_WARPS = 9;
+// quarter) that take the steps in turn, so that one group's arithmetic runs while the
+// other reads the next step's accumulators; values to digits: nine warps.
+constexpr int EPI_WARPS = 16, EPI_GROUP = 8, SLICE_WARPS = 9;
 constexpr int SLICE_T = 32 * SLICE_WARPS;
 static_assert(2 * WCOLS <= SLICE_T, "one thread per cell of a row pair");
 constexpr int EB_MIN = 200;                      // smallest exponent in use (E + 1022): scales stay normal
@@ -58,17 +59,31 @@ __device__ __forceinline__ unsigned digit2(unsigned long long a, unsigned long l
   return u;
 }
 
-// hi 2^30 + lo rounded to nearest, |hi| < 2^61, |lo| < 2^60, by integer arithmetic: a
-// conversion instruction costs three of the FP64 unit's 64-clock slots, these about
-// thirty single issue slots
-__device__ __forceinline__ double to_double(long long hi, long long lo) {
-  const int sh = min(30, __clzll(hi ^ (hi >> 63)) - 2);               // a small sum keeps its low bits
-  const long long t = (hi << sh) + (lo >> (30 - sh));                 // in units of 2^(30 - sh)
+// T += 2^K times a digit sum (an integer in FP32; below 2^(63 - K)), rounded to an integer
+// for K < 0
+template <int K>
+__device__ __forceinline__ void add_digit(long long& t, uint32_t f) {
+  static_assert(K <= 48, "weight of a digit sum");
+  const float v = __uint_as_float(f);
+  if constexpr (K < 0) {
+    t += static_cast<long long>(__float2int_rn(v * (1.0f / (1 << -K))));
+  } else if constexpr (K <= 30) {
+    t += static_cast<long long>(__float2int_rn(v)) * (1 << K);            // one IMAD.WIDE
+  } else if constexpr (K == 31) {
+    t += static_cast<long long>(__float2int_rn(v) * 2) * (1 << 30);
+  } else {
+    t += static_cast<long long>(__float2int_rn(v) * (1 << (K - 32))) << 32;
+  }
+}
+
+// t rounded to nearest, |t| < 2^62, by integer arithmetic: a conversion instruction
+// costs three of the FP64 unit's 64-clock slots, these about twenty-five single issue slots
+__device__ __forceinline__ double to_double(long long t) {
   const unsigned long long u = t < 0 ? -static_cast<unsigned long long>(t) : static_cast<unsigned long long>(t);
   const int lz = __clzll(u);
   const unsigned long long m = u << (lz & 63);                        // bit 63 set
   const unsigned long long r = (m >> 11) + ((m >> 10) & 1ull);        // 53 bits, possibly carrying
-  unsigned long long bits = (static_cast<unsigned long long>(1115 - sh - lz) << 52) + r;
+  unsigned long long bits = (static_cast<unsigned long long>(1085 - lz) << 52) + r;
   bits |= static_cast<unsigned long long>(t) & 0x8000000000000000ull;
   return u != 0 ? __longlong_as_double(static_cast<long long>(bits)) : 0.0;
 }

@@ -30,7 +30,7 @@
 // chain of 17 MMAs with N = 18 (7 - j) into an accumulator of its own
 // (chains j and j + 3 take turns); the coefficients (69 KB) stay in shared memory for the whole walk.
 //
-// Warps: 16 read the accumulators and update x (half the outputs of a cell each), 9 load
+// Warps: 16 read the accumulators and update x (two groups, alternating steps), 9 load
 // residuals and write digits, 3 issue the MMAs (an MMA takes a warp about as long to
 // issue as the tensor cores to execute), and 4 compute the cells near the
 // boundary, where the stencil differs, as FP64 dot products on the otherwise idle FP64
@@ -51,6 +51,7 @@
 #include <cmath>
 #include <cstdint>
 #include <cstring>
+#include <type_traits>
 
 #include "sv_digits.cuh"
 #include "sv_internal.h"
@@ -80,8 +81,8 @@ struct SM {
   static constexpr int RING = 0;                         // 6 cell rows
   static constexpr int P = RING + 6 * ROWB;              // pressures of the step: [digit][column] 16 B
   static constexpr int G = P + ROWB;
-  static constexpr int BAR = (G + GBYTES + 7) / 8 * 8;                 // full[6], done[6], free[3], gload
-  static constexpr int MISC = BAR + 16 * 8;              // tmem slot, fail flag, 8 maxima, 4 exponents
+  static constexpr int BAR = (G + GBYTES + 7) / 8 * 8;                 // full[6], done[2][6] (by step parity), free[3], gload
+  static constexpr int MISC = BAR + 22 * 8;              // tmem slot, fail flag, 8 maxima, 4 exponents
   static constexpr int BYTES = MISC + 4 * 16;
   static_assert(G % 16 == 0 && BAR % 8 == 0 && BYTES <= 227 * 1024, "shared memory");
 };
@@ -237,13 +238,6 @@ __device__ __forceinline__ void ring(const Args& A, int slot, int slots, int lan
   }
 }
 
-// T += D 2^k for the weights of the digit pairs; the compiler makes it one IMAD.WIDE
-__device__ __forceinline__ void madw(long long& t, uint32_t f, int k) {
-  t += static_cast<long long>(__float2int_rn(__uint_as_float(f))) * (1ll << k);
-}
-
-constexpr int BATCH = 4;   // coefficient digits read from tensor memory at a time
-
 struct Shared {   // what the roles of a CTA share
   uint32_t full, done, free, tmem;
   volatile int* fail;
@@ -251,62 +245,68 @@ struct Shared {   // what the roles of a CTA share
   int i0, j0, rows, S;
 };
 
-// Accumulators to x for the outputs O0 .. O0 + NO - 1: warp -> cell row a and lane
-// quarter of the columns.
-template <int O0, int NO>
-__device__ __forceinline__ void epilogue(const Args& A, const Shared& C, int warp, int lane) {
+// One chain's accumulators: T[o] += the digit sums (gi, c) with weight 2^(59 - 9 gi - 10 c),
+// in units of 2^16 (velocities) and 2^14 (pressure): the sums of |G| / 2^e_o are below 5
+// and 1.4, so |T| < 2^62.  Weights below the unit are rounded one by one (about a dozen).
+constexpr int UNIT_U = 16, UNIT_P = 14;
+template <int C, int GI>
+__device__ __forceinline__ void add_chain(uint32_t taddr, long long (&T)[9]) {
+  if constexpr (GI < NG - C) {
+    constexpr int K = 59 - 9 * GI - 10 * C;
+    constexpr bool two = GI + 1 < NG - C;
+    uint32_t v[2][9];
+    tmem_ld9(taddr + NBLK * GI, v[0]);
+    if constexpr (two) tmem_ld9(taddr + NBLK * (GI + 1), v[1]);
+    wait_ld();
+#pragma unroll
+    for (int o = 0; o < 8; ++o) {
+      add_digit<K - UNIT_U>(T[o], v[0][o]);
+      if constexpr (two) add_digit<K - 9 - UNIT_U>(T[o], v[1][o]);
+    }
+    add_digit<K - UNIT_P>(T[8], v[0][8]);
+    if constexpr (two) add_digit<K - 9 - UNIT_P>(T[8], v[1][8]);
+    add_chain<C, GI + 2>(taddr, T);
+  }
+}
+
+// Accumulators to x, steps g, g + 2, ...: warp -> cell row a and lane quarter of the columns.
+__device__ __forceinline__ void epilogue(const Args& A, const Shared& C, int g, int warp, int lane) {
   const LevelDev& L = A.L;
   const int n = L.n, nq = L.nq, np = L.np;
   const long long nv = L.nv;
   const int a = (warp >> 2) & 1, i = C.i0 + 32 * (warp & 3) + lane;
-  const uint32_t tq = C.tmem + (static_cast<uint32_t>(32 * (warp & 3)) << 16) + 9 * a + O0;
-  for (int s = 0; s < C.S; ++s) {
-    const int j = C.j0 + 2 * s + a;
-    const bool own = i <= n - 3 && 2 * s + a < C.rows;
-    const long long ku = static_cast<long long>(2 * j) * nq + 2 * i;
-    const long long kp = 2 * nv + static_cast<long long>(j) * np + i;
-    auto at = [&](int o) { return o == 8 ? kp : (o >> 2) * nv + ku + ((o >> 1) & 1) * nq + (o & 1); };
-    double xv[NO];
+  const uint32_t tq = C.tmem + (static_cast<uint32_t>(32 * (warp & 3)) << 16) + 9 * a;
+  for (int s = g; s < C.S; s += 2) {
+    long long T[9];
 #pragma unroll
-    for (int o = 0; o < NO; ++o) xv[o] = own && A.x != nullptr ? A.x[at(O0 + o)] : 0.0;
-    long long hi[NO], lo[NO];
-#pragma unroll
-    for (int o = 0; o < NO; ++o) hi[o] = lo[o] = 0;
-    bool ok = true;
-#pragma unroll
-    for (int c = 0; c < ND; ++c) {
-      ok = mbar_wait_or_fail(C.done + 8 * c, s & 1, A.wait_limit, C.fail);
-      if (!__all_sync(0xffffffffu, ok)) return;
+    for (int o = 0; o < 9; ++o) T[o] = 0;
+    auto chain = [&](auto c_) {
+      constexpr int c = decltype(c_)::value;
+      const bool ok = mbar_wait_or_fail(C.done + 8 * (ND * g + c), (s >> 1) & 1, A.wait_limit, C.fail);
+      if (!__all_sync(0xffffffffu, ok)) return false;
       fence_after();
-#pragma unroll
-      for (int i2 = 0; i2 < NG - c; i2 += BATCH) {
-        uint32_t v[BATCH][NO];
-#pragma unroll
-        for (int u = 0; u < BATCH; ++u)
-          if (i2 + u < NG - c) tmem_ldn<NO>(tq + acc_col(c) + NBLK * (i2 + u), v[u]);
-        wait_ld();
-#pragma unroll
-        for (int u = 0; u < BATCH; ++u) {
-          const int gi = i2 + u, k = 59 - 9 * gi - 10 * c;
-          if (gi >= NG - c) continue;
-#pragma unroll
-          for (int o = 0; o < NO; ++o) {
-            if (k >= 30) madw(hi[o], v[u][o], k - 30);
-            else madw(lo[o], v[u][o], k);
-          }
-        }
-      }
+      add_chain<c, 0>(tq + acc_col(c), T);
       fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(C.free + 8 * (c % MMA_WARPS));
-    }
-    const double sc = exp_scale(C.sexp[s & 3], -75);   // NaN where a residual of the window is not finite
-    if (own) {
-      const double qu = A.qu * sc, qp = A.qp * sc;
+      return true;
+    };
+    if (!(chain(std::integral_constant<int, 0>{}) && chain(std::integral_constant<int, 1>{}) &&
+          chain(std::integral_constant<int, 2>{}) && chain(std::integral_constant<int, 3>{}) &&
+          chain(std::integral_constant<int, 4>{}) && chain(std::integral_constant<int, 5>{})))
+      return;
+    const int j = C.j0 + 2 * s + a;
+    if (i > n - 3 || 2 * s + a >= C.rows) continue;
+    const long long ku = static_cast<long long>(2 * j) * nq + 2 * i;
+    const long long kp = 2 * nv + static_cast<long long>(j) * np + i;
+    auto at = [&](int o) { return o == 8 ? kp : (o >> 2) * nv + ku + ((o >> 1) & 1) * nq + (o & 1); };
+    double xv[9];
 #pragma unroll
-      for (int o = 0; o < NO; ++o)
-        A.xo[at(O0 + o)] = fma(O0 + o == 8 ? qp : qu, to_double(hi[o], lo[o]), xv[o]);
-    }
+    for (int o = 0; o < 9; ++o) xv[o] = A.x != nullptr ? A.x[at(o)] : 0.0;
+    const int eb = C.sexp[s & 3];   // NaN where a residual of the window is not finite
+    const double qu = A.qu * exp_scale(eb, UNIT_U - 75), qp = A.qp * exp_scale(eb, UNIT_P - 75);
+#pragma unroll
+    for (int o = 0; o < 9; ++o) A.xo[at(o)] = fma(o == 8 ? qp : qu, to_double(T[o]), xv[o]);
   }
 }
 
@@ -318,7 +318,7 @@ __global__ void __launch_bounds__(NT, 1) k_vanka_tc64(const Args A) {
   const long long nv = L.nv;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t s0 = su32(sm);
-  const uint32_t bar_full = s0 + SM::BAR, bar_done = bar_full + 8 * ND, bar_free = bar_done + 8 * ND,
+  const uint32_t bar_full = s0 + SM::BAR, bar_done = bar_full + 8 * ND, bar_free = bar_done + 16 * ND,
                  bar_g = bar_free + 8 * MMA_WARPS;
   uint32_t* tslot = reinterpret_cast<uint32_t*>(sm + SM::MISC);
   volatile int* fail = reinterpret_cast<volatile int*>(sm + SM::MISC + 4);
@@ -339,8 +339,9 @@ __global__ void __launch_bounds__(NT, 1) k_vanka_tc64(const Args A) {
     for (int k = 0; k < ND; ++k) {
       mbar_init(bar_full + 8 * k, SLICE_WARPS);
       mbar_init(bar_done + 8 * k, 1);
+      mbar_init(bar_done + 8 * (ND + k), 1);
     }
-    for (int k = 0; k < MMA_WARPS; ++k) mbar_init(bar_free + 8 * k, EPI_WARPS);
+    for (int k = 0; k < MMA_WARPS; ++k) mbar_init(bar_free + 8 * k, EPI_GROUP);
     mbar_init(bar_g, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     *fail = 0;
@@ -442,10 +443,8 @@ __global__ void __launch_bounds__(NT, 1) k_vanka_tc64(const Args A) {
   }
 
   const Shared C{bar_full, bar_done, bar_free, tmem, fail, sexp, i0, j0, rows, S};
-  if (warp < EPI_WARPS / 2) {
-    epilogue<0, EPI_SPLIT>(A, C, warp, lane);
-  } else if (warp < EPI_WARPS) {
-    epilogue<EPI_SPLIT, 9 - EPI_SPLIT>(A, C, warp, lane);
+  if (warp < EPI_WARPS) {
+    epilogue(A, C, warp / EPI_GROUP, warp, lane);
   } else if (warp < EPI_WARPS + SLICE_WARPS) {
     // ---- the row pairs after the first window ----
     const int t = tid - 32 * EPI_WARPS;
@@ -462,7 +461,8 @@ __global__ void __launch_bounds__(NT, 1) k_vanka_tc64(const Args A) {
       const bool renew = em > eb || (eb - em > 3 && eb > EB_MIN);
       if (renew) {   // uniform over the slicer warps: the window again, once the step before has read it
         eb = min(max(em + 1, EB_MIN), 0x7ff);
-        mbar_wait_or_fail(bar_done + 8 * (ND - 1), (s - 1) & 1, A.wait_limit, fail);
+        for (int j = 0; j < ND; ++j)
+          mbar_wait_or_fail(bar_done + 8 * (ND * ((s - 1) & 1) + j), ((s - 1) >> 1) & 1, A.wait_limit, fail);
         for (int qq = q - 2; qq < q; ++qq) {
           Cell c;
           load(qq, a, col, act, c);
@@ -481,7 +481,7 @@ __global__ void __launch_bounds__(NT, 1) k_vanka_tc64(const Args A) {
       for (int j = 0; j < ND; ++j) {
         // plane j of the row pair is free once chain j of the step before has read it (after
         // a failed wait the results are void and only the arrivals matter)
-        if (!renew) mbar_wait_or_fail(bar_done + 8 * j, (s - 1) & 1, A.wait_limit, fail);
+        if (!renew) mbar_wait_or_fail(bar_done + 8 * (ND * ((s - 1) & 1) + j), ((s - 1) >> 1) & 1, A.wait_limit, fail);
         if (act) {
           put(q, a, col, j, w);
           put_p(a, col, j, wp);
@@ -526,12 +526,12 @@ __global__ void __launch_bounds__(NT, 1) k_vanka_tc64(const Args A) {
 #pragma unroll
         for (int e = 0; e < 2; ++e, ++k)   // pressures, dx = (-1, 0) and (1, none)
           mma_f16(on, d, pl + off + 2 * e, gl + k * (CHUNK / 8), id, 1);
-        mma_commit(on, bar_done + 8 * c);
+        mma_commit(on, bar_done + 8 * (ND * (s & 1) + c));
         last = s * ND + c;
       }
     }
     // every chain that was issued has completed before the operands and tensor memory go
-    if (last >= 0 && !mbar_wait(bar_done + 8 * (last % ND), (last / ND) & 1, TC_WAIT_LIMIT)) *fail = 1;
+    if (last >= 0 && !mbar_wait(bar_done + 8 * (last % (2 * ND)), (last / (2 * ND)) & 1, TC_WAIT_LIMIT)) *fail = 1;
     mbar_wait(bar_g, 0, TC_WAIT_LIMIT);
     __syncwarp();
   } else {
