@@ -34,8 +34,8 @@
 // residuals and write digits, 3 issue the MMAs (an MMA takes a warp about as long to
 // issue as the tensor cores to execute), and 4 compute the cells near the
 // boundary, where the stencil differs, as FP64 dot products on the otherwise idle FP64
-// units.  They meet only in mbarriers, per digit: plane j is overwritten for the next
-// rows as soon as chain j has read it.
+// units.  They meet only in mbarriers, per digit or pair of digits: a plane is overwritten
+// for the next rows as soon as its chain has read it.
 //
 // The exponent E is shared by the cells in reach of a step.  It follows the residual:
 // when the largest of the window leaves [2^(E-4), 2^E), the digits of the window are
@@ -81,14 +81,17 @@ struct SM {
   static constexpr int RING = 0;                         // 6 cell rows
   static constexpr int P = RING + 6 * ROWB;              // pressures of the step: [digit][column] 16 B
   static constexpr int G = P + ROWB;
-  static constexpr int BAR = (G + GBYTES + 7) / 8 * 8;                 // full[6], done[2][6] (by step parity), free[3], gload
+  static constexpr int BAR = (G + GBYTES + 7) / 8 * 8;                 // full[3] (plane pairs), done[2][6] (by step parity), free[3], gload
   static constexpr int MISC = BAR + 22 * 8;              // tmem slot, fail flag, 8 maxima, 4 exponents
   static constexpr int BYTES = MISC + 4 * 16;
   static_assert(G % 16 == 0 && BAR % 8 == 0 && BYTES <= 227 * 1024, "shared memory");
 };
 
 __host__ __device__ constexpr int chain_n(int j) { return (NBLK * (NG - j) + 15) / 16 * 16; }
-// accumulator of the chains c and c + 3: its first tensor-memory column
+// accumulator of the chains c and c + 3: its first tensor-memory column.  One more for
+// each chain (five fit) let the MMAs run a step ahead and was slower (544 against 493 us
+// at 2048^2): MMAs of N <= 128 read shared memory at 97% of its rate, and the other warps'
+// accesses need the pauses.
 __host__ __device__ constexpr int acc_col(int c) {
   int k = 0;
   for (int i = 0; i < c % MMA_WARPS; ++i) k += chain_n(i);
@@ -337,7 +340,7 @@ __global__ void __launch_bounds__(NT, 1) k_vanka_tc64(const Args A) {
 
   if (tid == 0) {
     for (int k = 0; k < ND; ++k) {
-      mbar_init(bar_full + 8 * k, SLICE_WARPS);
+      if (k < ND / 2) mbar_init(bar_full + 8 * k, SLICE_WARPS);
       mbar_init(bar_done + 8 * k, 1);
       mbar_init(bar_done + 8 * (ND + k), 1);
     }
@@ -478,17 +481,23 @@ __global__ void __launch_bounds__(NT, 1) k_vanka_tc64(const Args A) {
       words_p(cur, eb, wp);
       if (q + 1 < S + 2) load(q + 1, a, col, act, cur);   // in flight while the planes are written
 #pragma unroll
-      for (int j = 0; j < ND; ++j) {
-        // plane j of the row pair is free once chain j of the step before has read it (after
-        // a failed wait the results are void and only the arrivals matter)
-        if (!renew) mbar_wait_or_fail(bar_done + 8 * (ND * ((s - 1) & 1) + j), ((s - 1) >> 1) & 1, A.wait_limit, fail);
+      for (int h = 0; h < ND / 2; ++h) {
+        // two planes of the row pair are free once their chains of the step before have read
+        // them (after a failed wait the results are void and only the arrivals matter)
+        if (!renew) {
+          mbar_wait_or_fail(bar_done + 8 * (ND * ((s - 1) & 1) + 2 * h), ((s - 1) >> 1) & 1, A.wait_limit, fail);
+          mbar_wait_or_fail(bar_done + 8 * (ND * ((s - 1) & 1) + 2 * h + 1), ((s - 1) >> 1) & 1, A.wait_limit, fail);
+        }
         if (act) {
-          put(q, a, col, j, w);
-          put_p(a, col, j, wp);
+#pragma unroll
+          for (int j = 2 * h; j < 2 * h + 2; ++j) {
+            put(q, a, col, j, w);
+            put_p(a, col, j, wp);
+          }
         }
         fence_proxy();
         __syncwarp();
-        if (lane == 0) mbar_arrive(bar_full + 8 * j);
+        if (lane == 0) mbar_arrive(bar_full + 8 * h);
       }
     }
   } else if (warp < EPI_WARPS + SLICE_WARPS + MMA_WARPS) {
@@ -508,7 +517,7 @@ __global__ void __launch_bounds__(NT, 1) k_vanka_tc64(const Args A) {
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const int c = w + MMA_WARPS * h;
-        if (ok && s > 0) ok = wait(bar_full + 8 * c, (s - 1) & 1);   // step 0: the first window
+        if (ok && s > 0) ok = wait(bar_full + 8 * (c >> 1), (s - 1) & 1);   // step 0: the first window
         const int use = 2 * s + h;   // earlier chains of this accumulator
         if (ok && use > 0) ok = wait(bar_free + 8 * w, (use - 1) & 1);
         if (!ok) break;
