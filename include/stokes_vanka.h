@@ -177,7 +177,7 @@ stokes_status stokes_hierarchy_destroy(stokes_hierarchy* h);
 stokes_status stokes_level_info(const stokes_hierarchy* h, int* num_levels, int* n_finest);
 stokes_status stokes_level_n(const stokes_hierarchy* h, int level, int* n_level);
 /* Sweep configuration used on a level (see stokes_params.tile).  With tile = -1 the
- * FP64 form takes, on levels with sweeps, 7 (n < 96: the residual, then the sum of all
+ * FP64 form takes, on levels with sweeps, 7 (n < 56: the residual, then the sum of all
  * patch solves as one stencil of FP64 dot products) or 8 (above: the same stencil as an
  * exact integer contraction on the tensor cores); both are chosen by size only and are
  * not values of stokes_params.tile.  In the mixed

@@ -814,13 +814,15 @@ cudaError_t tune_level(stokes_hierarchy* h, sv::Level& L, int* cfg) {
 // n = 64 its 1125 multiply-adds per vertex exceed those of the tiled patch solves.
 constexpr int STENCIL_F32_MAX_N = 64;
 // Levels whose FP64 operator is the tensor-core contraction (smaller ones: FP64, one
-// output per thread).
+// output per thread): 8.4 us at n = 128 in FP64, 11.4 us at n = 256 by the contraction
+// (57 us in FP64 before it).
 constexpr int OP_TC64_MIN_N = 160;
 // The FP64 sweep by size: the composite stencil as FP64 dot products below TC64_MIN_N, as
 // the tensor-core contraction from there on.  One zero-guess sweep, FP64 dot products /
-// tensor cores (us): n = 64 17.5 / 33.2, 128 52.2 / 34.1; below, the contraction pays for
-// its prologue (91 KB of coefficients, the first window), above, FP64 for its rate.
-constexpr int TC64_MIN_N = 96;
+// tensor cores (us): n = 48 10.9 / 13.0, 56 14.3 / 12.9, 64 17.6 / 12.9, 128 52.4 / 13.9.
+// Below, the contraction pays for its prologue (69 KB of coefficients, the first window),
+// above, the dot products for the FP64 rate.
+constexpr int TC64_MIN_N = 56;
 cudaError_t choose_tiles(stokes_hierarchy* h) {
   for (sv::Level& L : h->lv) {
     if (h->prm.tile >= 0 || h->prm.smoother != STOKES_SMOOTHER_SHARED || h->prm.precond == 1) {

@@ -16,7 +16,7 @@ from oracle import stokes_oracle as O
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n,coarse_n", [(8, 4), (10, 5), (12, 6), (14, 7), (16, 4), (28, 7), (40, 5), (64, 4)])
+@pytest.mark.parametrize("n,coarse_n", [(8, 4), (10, 5), (12, 6), (14, 7), (16, 4), (28, 7), (40, 5), (48, 6)])
 def test_stencil_sweep_matches_patch_sweep(n, coarse_n):
     import paper_2401_06277_gb300 as pkg
     from paper_2401_06277_gb300 import stokes
