@@ -252,10 +252,9 @@ def job_throughput(ws, units_local: float, ms_local: float) -> tuple[float, floa
 # kernel at 1024 x 1024 (ncu --set full, summaries in profiles/); at other sizes the
 # bench scales them by the number of dofs (the traffic of a sweep is proportional)
 TRAFFIC_1024 = {
-    "fp64": {"bytes": 151244032 + 45977088 + 84809216 + 172724736 + 269548032 + 56484864, "tile": "split16x16x2",
-             "source": "profiles/k_vanka_own_f64_n1024.md (k_apply<double> residual + k_vanka_own<double,16,16,256,2> "
-                       "+ k_colsum_update, a sweep from a non-zero iterate; "
-                       "writes still in L2 at kernel end are not counted)"},
+    "fp64": {"bytes": 154744064 + 45769472 + 157928448 + 45379072, "tile": "stencil-tc",
+             "source": "profiles/tc64_kernels_f64_n1024.md (k_apply_tc64 residual + k_vanka_tc64, a sweep from a "
+                       "non-zero iterate; writes still in L2 at kernel end are not counted)"},
     "mixed": {"bytes": 77614592 + 7096320, "tile": "14x14",
               "source": "profiles/k_vanka_strip_f32_n1024.md (k_vanka_strip<false> interior strips; the ring "
                         "launch is not included; writes still in L2 at kernel end are not counted)"},
@@ -311,7 +310,8 @@ PRECS = {"fp64": 0, "mixed": 1, "bf16": 2}
 ZERO_GUESS_SHARE = 1.0 / 4.0
 # sweep configurations by stokes_level_tile: fused tiles of TX x TY vertices, or (4, 5; FP64
 # only) the split sweep: 16 x 16 own-patch solves writing the corrections, then the update
-# (5: compiled for two CTAs per SM)
+# (5: compiled for two CTAs per SM), or (7, 8) the composite stencil of all patch solves, as
+# dot products or as the tensor-core digit contraction
 TILE_NAMES = ["8x8", "16x8", "16x16", "14x14", "split16x16", "split16x16x2", "4x4", "stencil", "stencil-tc"]
 
 
@@ -443,13 +443,33 @@ def _time_form(args, prec_name, ws, rank, f_host, ud_host, with_e2e, smoother, h
                     "algorithmic_flops_per_launch": fl, "algorithmic_bytes_per_launch": by,
                     "hbm_gbs_achieved": round(by / (sweep_ms * 1e-3) / 1e9, 1),
                     "hbm_frac": round(by / (sweep_ms * 1e-3) / 1e9 / peaks.get("hbm_gbs", 6780.0), 4)}
+    elif prec_name == "fp64" and tile == "stencil-tc":
+        # issued FP16 operations of the digit contractions per vertex: sweep 17 MMAs of K = 16
+        # and N = 18 x 27 digit pairs for two cell rows, operator 8 of K = 16, N = 32 x 6
+        # digits; the zero-guess sweeps form no residual
+        nv = (n + 1) ** 2
+        fl = 2.0 * nv * (17 * 16 * 18 * 27 / 2 + (1.0 - ZERO_GUESS_SHARE) * 8 * 16 * 32 * 6 / 2)
+        by = sweep_bytes(n) * (3.0 - ZERO_GUESS_SHARE) / 3.0
+        peak = peaks.get("bf16_tflops", 1900.0)
+        achieved = fl / (sweep_ms * 1e-3) / 1e12
+        hbm = by / (sweep_ms * 1e-3) / 1e9
+        roofline = {"bound": "tensor", "kernel": "k_apply_tc64 (residual) + k_vanka_tc64 (finest level): FP64 as exact "
+                                                 "sums of FP16 digit products",
+                    "achieved": round(achieved, 1), "peak": peak, "unit": "TFLOP/s",
+                    "frac": round(achieved / peak, 4), "traffic": args.traffic,
+                    "peak_source": "measured dense 16-bit rate (MEASURED_PEAKS.json)" if "bf16_tflops" in peaks
+                                   else "fallback: an earlier measurement of the dense 16-bit rate",
+                    "issued_fp16_flops_per_launch": fl,
+                    "algorithmic_flops_per_launch": sweep_flops(n) - ZERO_GUESS_SHARE * 361.0 * nv,
+                    "algorithmic_bytes_per_launch": by,
+                    "hbm_gbs_achieved": round(hbm, 1), "hbm_frac": round(hbm / peaks.get("hbm_gbs", 6780.0), 4)}
     elif prec_name == "fp64":
         # the first pre-smoothing sweep of each cycle starts from zero (no residual: 361 flops
         # per vertex fewer); the timed launches average over all nu1 + nu2 sweeps
         fl = sweep_flops(n) - ZERO_GUESS_SHARE * 361.0 * (n + 1) ** 2
         peak = FP64_PEAK["peak"]
         achieved = fl / (sweep_ms * 1e-3) / 1e9
-        kname = ("k_apply<double> + k_vanka_own<double,16,16> + k_colsum_update (split sweep, finest level)"
+        kname = ("k_apply_tc64 + k_vanka_own<double,16,16> + k_colsum_update (split sweep, finest level)"
                  if tile.startswith("split")
                  else "k_vanka<double> (finest level)")
         roofline = {"bound": "alu", "kernel": kname, "achieved": round(achieved, 2),
@@ -459,10 +479,9 @@ def _time_form(args, prec_name, ws, rank, f_host, ud_host, with_e2e, smoother, h
                     "fp64_peaks": {k: FP64_PEAK[k] for k in ("fma_probe_gflops", "dgemm_gflops")},
                     "nominal_gflops": round(SM_COUNT * 4 * sm_max * 1e6 / 1e9, 1),
                     "algorithmic_flops_per_launch": fl,
-                    "executed_flops_note": "the kernels execute fewer FP64 flops than the algorithmic count (about "
-                                           "1071 against 1681 per vertex at 1024^2, ncu: shared row transforms, the fused "
-                                           "column pass and the shared last pass of the fast diagonalisation, the "
-                                           "residual once per cell); profiles/k_vanka_own_f64_n1024.md",
+                    "executed_flops_note": "the FP64 pipe executes fewer operations than the algorithmic count: shared "
+                                           "row transforms, the fused column pass and the shared last pass of the fast "
+                                           "diagonalisation; the residual runs on the tensor cores",
                     "algorithmic_bytes_per_launch": sweep_bytes(n) * (3.0 - ZERO_GUESS_SHARE) / 3.0,
                     "hbm_gbs_achieved": round(sweep_bytes(n) * (3.0 - ZERO_GUESS_SHARE) / 3.0 / (sweep_ms * 1e-3) / 1e9, 1)}
     else:
@@ -859,7 +878,7 @@ def main():
     ap.add_argument("--oracle-worker", action="store_true")
     ap.add_argument("--oracle-vcycle", type=int, default=None, metavar="N",
                     help="time the CPU oracle's set-up and one V-cycle at N x N (single thread) and exit")
-    ap.add_argument("--tile", type=int, default=-1, help="Vanka sweep configuration (-1: autotuned; 0..3 fused 8x8/16x8/16x16/14x14, 4/5 split 16x16, 6 fused 4x4)")
+    ap.add_argument("--tile", type=int, default=-1, help="Vanka sweep configuration (-1: by size in FP64, autotuned in the mixed forms; 0..3 fused 8x8/16x8/16x16/14x14, 4/5 split 16x16, 6 fused 4x4)")
     ap.add_argument("--kernel", choices=["sweep", "residual", "vcycle", "solve"], default=None,
                     help="time one kernel alone on the finest level (profiling mode)")
     ap.add_argument("--smoother", type=int, choices=[0, 1, 2, 3], default=0,

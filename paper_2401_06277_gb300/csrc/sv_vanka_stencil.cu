@@ -1,5 +1,5 @@
 // sv_vanka_stencil.cu -- the additive Vanka correction as one stencil (Algorithm 3
-// with the shared patch inverses of Section 6.3), FP64.
+// with the shared patch inverses of Section 6.3).
 //
 // On a uniform grid every patch of a class has the same inverse, so the sum over
 // patches sum_i V_i^T diag(1/m) A_i^-1 V_i is itself a stencil: the nine
@@ -19,7 +19,6 @@
 #include <cuda_runtime.h>
 
 #include <cmath>
-#include <mutex>
 #include <vector>
 
 #include "sv_internal.h"
@@ -133,7 +132,9 @@ std::vector<long double> build_stencil() {
 // chain a warp runs, not the work.  Hence a warp takes one output kind of 4 x 2
 // cells with four lanes per output, each lane every fourth coefficient (at most 42
 // multiply-adds), summed by shuffles; three warps per CTA and three CTAs per tile
-// spread the nine outputs of a cell over the SMs.
+// spread the nine outputs of a cell over the SMs.  Zero guess, FP64: 9.0 us at n = 40,
+// 17.6 at n = 64 (a solve at n = 32: 7.8 ms with patch solves, 3.6 with this sweep); FP32
+// V-cycle of n = 128 with it up to n = 64: 260 -> 200 us.
 // ---------------------------------------------------------------------------
 constexpr int GX = 4, GY = 2, GW = GX + 4, GH = GY + 4, PARTS = 4;
 static_assert(GX * GY * PARTS == 32, "a warp is one output kind of a tile");
