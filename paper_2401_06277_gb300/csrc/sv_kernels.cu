@@ -218,14 +218,18 @@ __global__ void __launch_bounds__(128) k_restrict_march(LevelDev F, LevelDev C, 
 
 // One thread per pair of fine node columns (2 q, 2 q + 1), q in 0..2 nc, of component c (2:
 // the fine vertex column q of the pressure): the even column is a coarse column, the odd
-// one takes (3/8, 3/4, -1/8) or its mirror image.
+// one takes (3/8, 3/4, -1/8) or its mirror image.  Coarse rows per thread by size, since a
+// smaller level is bound by the chain of read-modify-writes of a thread, a larger one by
+// the FP64 pipe; FP64, 1 / 2 / 4 rows (us): to 2048^2 230 / 216 / 210, to 1024^2 60.6 / 56.9
+// / 57.9, to 512^2 18.3 / 19.1 / 21.8, to 256^2 7.8 / 8.1 / 12.8.  The restriction only
+// reads along its chain: 4 rows are the best (2 within 2%) from 512^2 on.
 template <typename T>
 __global__ void __launch_bounds__(128) k_prolong_march(LevelDev F, LevelDev C, const T* __restrict__ ec,
-                                                       T* __restrict__ xf) {
+                                                       T* __restrict__ xf, int rows) {
   pdl_begin();
-  const int q = blockIdx.x * blockDim.x + threadIdx.x, ey0 = blockIdx.y * MARCH_ROWS, c = blockIdx.z;
+  const int q = blockIdx.x * blockDim.x + threadIdx.x, ey0 = blockIdx.y * rows, c = blockIdx.z;
   if (q > F.n) return;
-  const int ey1 = min(ey0 + MARCH_ROWS, C.np), fq = F.nq, cq = C.nq, ex = q >> 1;
+  const int ey1 = min(ey0 + rows, C.np), fq = F.nq, cq = C.nq, ex = q >> 1;
   if (c == 2) {
     const T* e = ec + 2 * C.nv + ex;
     T* x = xf + 2 * F.nv + q;
@@ -424,7 +428,8 @@ void launch_prolong_add(const LevelDev& F, const LevelDev& C, const T* ec, T* xf
     launch_pdl(k_prolong_out<T>, out_grid(C.np, 36), dim3(32), 0, s, F, C, ec, xf);
     return;
   }
-  launch_pdl(k_prolong_march<T>, dim3((F.np + 127) / 128, (C.np + MARCH_ROWS - 1) / MARCH_ROWS, 3), dim3(128), 0, s, F, C, ec, xf);
+  const int rows = C.n <= 320 ? 1 : C.n <= 640 ? 2 : MARCH_ROWS;
+  launch_pdl(k_prolong_march<T>, dim3((F.np + 127) / 128, (C.np + rows - 1) / rows, 3), dim3(128), 0, s, F, C, ec, xf, rows);
 }
 
 template <typename TI, typename TO>

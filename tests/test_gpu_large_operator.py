@@ -71,3 +71,17 @@ def test_operator_spreads_nonfinite_values_as_the_stencil_does():
     ok = torch.isfinite(out)
     assert torch.allclose(out[ok], clean[ok], rtol=1e-12, atol=1e-12)
     H.close()
+
+
+@pytest.mark.parametrize("n,coarse_n", [(640, 5), (704, 11)])
+def test_prolongation_rows_per_thread(n, coarse_n):
+    """The sizes on both sides of a change in the coarse rows a thread walks."""
+    import paper_2401_06277_gb300 as pkg
+    from paper_2401_06277_gb300 import stokes
+    H = pkg.Hierarchy(n, coarse_n=coarse_n, restart=1)
+    P = O.prolongation(O.Mesh(n), O.Mesh(n // 2))
+    e, x = si.random_vector(n // 2, 3), si.random_vector(n, 4)
+    xf = dev(x)
+    stokes.stokes_prolong_add(H.handle, H.levels - 1, dev(e), xf)
+    assert close(xf, x + P @ e)
+    H.close()
