@@ -143,12 +143,13 @@ __device__ __forceinline__ void epilogue(const Args& A, const Shared& C, int g, 
       add_digit<8>(T[8], v[1][8]);
       add_digit<-2>(T[8], v[2][8]);
     }
+    // before the arrival: it lets step s + 2 run, after which the slot takes step s + 4's
+    const int eb = C.sexp[s & 3];
     fence_before();
     __syncwarp();
     if (lane == 0) mbar_arrive(C.free + 8 * g);
     const int j = C.j0 + 2 * s + a;
     if (i > n || 2 * s + a >= C.rows) continue;
-    const int eb = C.sexp[s & 3];
     if (eb == 0x7ff) {
       for (int o = 0; o < 9; ++o) apply_cell(A, i, j, o);
       continue;
