@@ -332,20 +332,27 @@ stokes_status stokes_stats_reset(stokes_hierarchy* h);
 stokes_status stokes_stats_read(stokes_hierarchy* h, stokes_stats* out);
 
 /* Device-side failures of asynchronous work: synchronises the creation
- * stream and returns STOKES_ERR_TIMEOUT if a bounded device wait (the
- * tensor-core sweep's mbarrier waits) expired in work queued since the last
- * report, else STOKES_OK.  The flag is cleared when reported, so the
- * hierarchy stays usable.  stokes_fgmres_solve and the other synchronising
- * solves check the same flag at every iteration. */
+ * stream and returns STOKES_ERR_TIMEOUT if a bounded device wait expired in
+ * work queued since the last report, else STOKES_OK.  Waits are bounded in the
+ * tensor-core sweeps (the BF16 form's; the FP64 form's from n = 56 on), in the
+ * FP64 operator of every form from n = 160 on (stokes_apply_operator,
+ * stokes_residual, the residual inside a sweep, cycle or solve) and at the grid
+ * barriers of the persistent coarse-level launch.  After an expired wait the
+ * output of that call is void: any part of it may have been written.  The flag
+ * is cleared when reported, so the hierarchy stays usable.  stokes_fgmres_solve
+ * and the other synchronising solves check the same flag at every iteration. */
 stokes_status stokes_device_status(stokes_hierarchy* h);
 
 /* Test hooks: failures made on purpose, without faulting or hanging a GPU.
- *  - stokes_test_set_wait_limit: number of polls of the tensor-core sweep's
- *    first bounded wait (the mbarrier of the bulk copy of the patch inverse).
- *    0 makes that wait expire at once: the kernel sets the hierarchy's error
- *    flag, still waits for its copy with the full limit, frees its tensor
- *    memory and returns without writing x_out; the next synchronising call
- *    returns STOKES_ERR_TIMEOUT.  A negative value restores the default.
+ *  - stokes_test_set_wait_limit: number of polls of the bounded waits of the
+ *    tensor-core kernels: in the BF16 sweep the first one (the mbarrier of the
+ *    bulk copy of the patch inverse), in the FP64 sweep and operator every wait
+ *    between their warps.  0 makes them expire at once: the kernel sets the
+ *    hierarchy's error flag, still waits for its copies and matrix instructions
+ *    in flight with the full limit, frees its tensor memory and returns.  The
+ *    BF16 sweep then has written nothing, the FP64 kernels may have written part
+ *    of their output; the next synchronising call returns STOKES_ERR_TIMEOUT.  A
+ *    negative value restores the default.
  *  - stokes_test_set_alloc_limit: cap on the device bytes one
  *    stokes_hierarchy_create (on any thread) may allocate; beyond it the
  *    creation frees what it holds and returns STOKES_ERR_OOM.  0 removes it. */

@@ -563,7 +563,7 @@ stokes_status read_scalar(stokes_hierarchy* h, const double* dev, double* out) {
     // hierarchy stays usable
     cudaMemsetAsync(h->dev_err, 0, sizeof(int), h->stream);
     if (h->tail_bar) cudaMemsetAsync(h->tail_bar, 0, 2 * sizeof(unsigned), h->stream);
-    return fail(STOKES_ERR_TIMEOUT, "a bounded device wait expired (tensor-core sweep or grid barrier)");
+    return fail(STOKES_ERR_TIMEOUT, "a bounded device wait expired (tensor-core kernel or grid barrier)");
   }
   return STOKES_OK;
 }
@@ -1280,7 +1280,7 @@ stokes_status stokes_device_status(stokes_hierarchy* h) {
   if (flag != 0) {
     SV_TRY(cudaMemsetAsync(h->dev_err, 0, sizeof(int), h->stream), "clear error flag");
     if (h->tail_bar) SV_TRY(cudaMemsetAsync(h->tail_bar, 0, 2 * sizeof(unsigned), h->stream), "reset grid barrier");
-    return fail(STOKES_ERR_TIMEOUT, "a bounded device wait expired (tensor-core sweep or grid barrier)");
+    return fail(STOKES_ERR_TIMEOUT, "a bounded device wait expired (tensor-core kernel or grid barrier)");
   }
   return STOKES_OK;
 }
@@ -1288,6 +1288,7 @@ stokes_status stokes_device_status(stokes_hierarchy* h) {
 stokes_status stokes_test_set_wait_limit(stokes_hierarchy* h, int polls) {
   if (!h) return fail(STOKES_ERR_ARG, "null hierarchy");
   h->tc_wait_limit = (polls < 0 || polls > sv::TC_WAIT_LIMIT) ? sv::TC_WAIT_LIMIT : polls;
+  for (sv::Level& L : h->lv) L.d.wait_limit = h->tc_wait_limit;
   return STOKES_OK;
 }
 

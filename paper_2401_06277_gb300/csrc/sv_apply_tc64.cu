@@ -444,7 +444,7 @@ void launch_apply_tc64(const LevelDev& L, const double* x, const double* b, doub
   // one more than a multiple of 128 on most grids); each with its segments
   const int rem = L.np % COLS, strips = L.np / COLS + (rem > EDGE_COLS ? 1 : 0), steps = (L.np + 1) / 2;
   const int seg = segment_steps(strips, steps, sms, 3);
-  Args A{L, L.op_digits, x, b, y, L.cb / L.cl, strips, seg, L.dev_err, TC_WAIT_LIMIT};
+  Args A{L, L.op_digits, x, b, y, L.cb / L.cl, strips, seg, L.dev_err, L.wait_limit};
   count_launches(1);
   launch_pdl(k_apply_tc64, dim3(strips, (steps + seg - 1) / seg), dim3(NT), SM::BYTES, s, A);
 }

@@ -140,9 +140,11 @@ struct LevelDev {
   double zs, zsinv;
   float zsf, zsinvf;
   // levels whose FP64 operator runs on the tensor cores (sv_apply_tc64.cu): the packed
-  // integer coefficients, and the hierarchy's error flag; null elsewhere
+  // integer coefficients, the hierarchy's error flag (null elsewhere) and the polls of a
+  // bounded wait
   const unsigned char* op_digits = nullptr;
   int* dev_err = nullptr;
+  int wait_limit = TC_WAIT_LIMIT;
 };
 
 // cl and cb in the element type
@@ -262,7 +264,7 @@ struct stokes_hierarchy {
   sv::BSParams bs;
   double* host_scalars = nullptr;  // pinned host mirror of a few scalars
   int* dev_err = nullptr;          // set by kernels whose bounded waits expired
-  int tc_wait_limit = sv::TC_WAIT_LIMIT;   // first bounded wait of the tensor-core sweep (test hook)
+  int tc_wait_limit = sv::TC_WAIT_LIMIT;   // polls of the tensor-core kernels' bounded waits (test hook)
   // persistent coarse-level kernel (mixed forms): levels 0..tail_top in one launch
   int tail_top = -1;
   sv::TailOp* tail_ops = nullptr;      // device: the steps of one cycle below and at tail_top
