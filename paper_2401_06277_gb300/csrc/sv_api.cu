@@ -201,10 +201,14 @@ cudaEvent_t* timing_pair(stokes_hierarchy* h, bool finest) {
 
 // One FP64 sweep with the hierarchy's smoother (shared class factors, or the
 // stored per-patch inverses, whose sweep uses L.r as residual scratch: L.r is
-// free whenever a sweep runs).
+// free whenever a sweep runs).  A mixed hierarchy has neither L.r nor FP64 scratch: its
+// FP64 sweep (stokes_vanka_sweep alone) takes two vectors of the Krylov basis, free
+// outside a solve, or a fused tile where the split sweep was asked for.
 void sweep_f64(stokes_hierarchy* h, sv::Level& L, const double* x, const double* b, double* xo) {
+  const bool mixed = h->prm.prec != STOKES_FP64;
   if (h->prm.smoother == STOKES_SMOOTHER_BRAESS_SARAZIN || h->prm.smoother == STOKES_SMOOTHER_SCHUR_UZAWA)
-    sv::launch_bs_sweep<double>(L.d, h->bs, static_cast<double*>(h->bs_buf), L.r, x, b, xo, h->stream);
+    sv::launch_bs_sweep<double>(L.d, h->bs, mixed ? h->V + L.d.N : static_cast<double*>(h->bs_buf),
+                                mixed ? h->V : L.r, x, b, xo, h->stream);
   else if (h->prm.smoother == STOKES_SMOOTHER_PER_PATCH)
     sv::launch_simple_sweep(L.d, L.pinv, h->delta, L.r, x, b, xo, h->prm.omega, h->stream);
   else if (L.vk_cfg == sv::VANKA_CFG_TC64)
@@ -212,11 +216,12 @@ void sweep_f64(stokes_hierarchy* h, sv::Level& L, const double* x, const double*
                           L.r, h->dev_err, h->tc_wait_limit, h->stream);
   else if (L.vk_cfg == sv::VANKA_CFG_STENCIL)
     sv::launch_vanka_stencil<double>(L.d, h->stencil_G, x, b, xo, h->prm.omega, L.r, h->stream);
-  else if (sv::vanka_cfg_split(L.vk_cfg))
+  else if (sv::vanka_cfg_split(L.vk_cfg) && !mixed)
     sv::launch_vanka_split<double>(L.d, L.cd, h->fd, x, b, xo, h->prm.omega, h->delta, L.vk_cfg == sv::VANKA_CFG_SPLIT2,
                            h->stream, L.r);
   else
-    sv::launch_vanka<double>(L.d, L.cd, h->fd, x, b, xo, h->prm.omega, L.vk_cfg, h->stream);
+    sv::launch_vanka<double>(L.d, L.cd, h->fd, x, b, xo, h->prm.omega, sv::vanka_cfg_split(L.vk_cfg) ? 1 : L.vk_cfg,
+                             h->stream);
 }
 
 // Mixed-form sweep of a level with strip tiles: the interior tiles on the strip
