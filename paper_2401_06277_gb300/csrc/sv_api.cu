@@ -199,28 +199,40 @@ cudaEvent_t* timing_pair(stokes_hierarchy* h, bool finest) {
   return p;
 }
 
+// A level as the sweeps and residuals of a cycle take it: the tensor-core operator keeps
+// 71 bits below the largest values in reach and leaves nothing to FP64.  The entries of a
+// cycle are not independent, its coarse corrections join near and far ones; a Krylov
+// iteration takes what the cycle returns as it is, and its own operator keeps every entry.
+sv::LevelDev cycle_level(const sv::Level& L) {
+  sv::LevelDev d = L.d;
+  d.every_entry = false;
+  return d;
+}
+
 // One FP64 sweep with the hierarchy's smoother (shared class factors, or the
 // stored per-patch inverses, whose sweep uses L.r as residual scratch: L.r is
 // free whenever a sweep runs).  A mixed hierarchy has neither L.r nor FP64 scratch: its
 // FP64 sweep (stokes_vanka_sweep alone) takes two vectors of the Krylov basis, free
 // outside a solve, or a fused tile where the split sweep was asked for.
-void sweep_f64(stokes_hierarchy* h, sv::Level& L, const double* x, const double* b, double* xo) {
+// single: a sweep that the caller asked for.
+void sweep_f64(stokes_hierarchy* h, sv::Level& L, const double* x, const double* b, double* xo, bool single) {
+  const sv::LevelDev d = single ? L.d : cycle_level(L);
   const bool mixed = h->prm.prec != STOKES_FP64;
   if (h->prm.smoother == STOKES_SMOOTHER_BRAESS_SARAZIN || h->prm.smoother == STOKES_SMOOTHER_SCHUR_UZAWA)
-    sv::launch_bs_sweep<double>(L.d, h->bs, mixed ? h->V + L.d.N : static_cast<double*>(h->bs_buf),
+    sv::launch_bs_sweep<double>(d, h->bs, mixed ? h->V + L.d.N : static_cast<double*>(h->bs_buf),
                                 mixed ? h->V : L.r, x, b, xo, h->stream);
   else if (h->prm.smoother == STOKES_SMOOTHER_PER_PATCH)
-    sv::launch_simple_sweep(L.d, L.pinv, h->delta, L.r, x, b, xo, h->prm.omega, h->stream);
+    sv::launch_simple_sweep(d, L.pinv, h->delta, L.r, x, b, xo, h->prm.omega, h->stream);
   else if (L.vk_cfg == sv::VANKA_CFG_TC64)
-    sv::launch_vanka_tc64(L.d, h->stencil_digits, h->stencil_eu, h->stencil_ep, h->stencil_ring, x, b, xo, h->prm.omega,
+    sv::launch_vanka_tc64(d, h->stencil_digits, h->stencil_eu, h->stencil_ep, h->stencil_ring, x, b, xo, h->prm.omega,
                           L.r, h->dev_err, h->tc_wait_limit, h->stream);
   else if (L.vk_cfg == sv::VANKA_CFG_STENCIL)
-    sv::launch_vanka_stencil<double>(L.d, h->stencil_G, x, b, xo, h->prm.omega, L.r, h->stream);
+    sv::launch_vanka_stencil<double>(d, h->stencil_G, x, b, xo, h->prm.omega, L.r, h->stream);
   else if (sv::vanka_cfg_split(L.vk_cfg) && !mixed)
-    sv::launch_vanka_split<double>(L.d, L.cd, h->fd, x, b, xo, h->prm.omega, h->delta, L.vk_cfg == sv::VANKA_CFG_SPLIT2,
+    sv::launch_vanka_split<double>(d, L.cd, h->fd, x, b, xo, h->prm.omega, h->delta, L.vk_cfg == sv::VANKA_CFG_SPLIT2,
                            h->stream, L.r);
   else
-    sv::launch_vanka<double>(L.d, L.cd, h->fd, x, b, xo, h->prm.omega, sv::vanka_cfg_split(L.vk_cfg) ? 1 : L.vk_cfg,
+    sv::launch_vanka<double>(d, L.cd, h->fd, x, b, xo, h->prm.omega, sv::vanka_cfg_split(L.vk_cfg) ? 1 : L.vk_cfg,
                              h->stream);
 }
 
@@ -247,7 +259,7 @@ void timed_sweep<double>(stokes_hierarchy* h, bool finest, sv::Level& L, const d
                          double* xo) {
   cudaEvent_t* ev = timing_pair(h, finest);
   if (ev) cudaEventRecord(ev[0], h->stream);
-  sweep_f64(h, L, x, b, xo);
+  sweep_f64(h, L, x, b, xo, false);
   if (ev) cudaEventRecord(ev[1], h->stream);
 }
 
@@ -441,7 +453,7 @@ void vcycle_level(stokes_hierarchy* h, int l, const R* b, R* out) {
   // (Galerkin: P^T A_f P = A_c), so each pass starts the coarse cycle from zero
   const int passes = (l - 1 == 0) ? 1 : h->prm.cycle;
   for (int g = 0; g < passes; ++g) {
-    sv::launch_apply<R>(L.d, cur, b, Buf<R>::r(L), 1, s);
+    sv::launch_apply<R>(cycle_level(L), cur, b, Buf<R>::r(L), 1, s);
     sv::launch_restrict<R>(L.d, C.d, Buf<R>::r(L), Buf<R>::b(C), s);
     vcycle<R>(h, l - 1, Buf<R>::b(C), Buf<R>::e(C));
     sv::launch_prolong_add<R>(L.d, C.d, Buf<R>::e(C), cur, s);
@@ -1251,7 +1263,7 @@ stokes_status stokes_vanka_sweep(stokes_hierarchy* h, int level, const double* x
   if (!b || !x_out) return fail(STOKES_ERR_ARG, "null vector");
   if (x_out == x || x_out == b) return fail(STOKES_ERR_ARG, "x_out must not alias x or b");
   sv::Level& L = h->lv[level];
-  sweep_f64(h, L, x, b, x_out);
+  sweep_f64(h, L, x, b, x_out, true);
   return check_launch("vanka_sweep");
 }
 
@@ -1263,7 +1275,7 @@ stokes_status stokes_relaxation_sweep(stokes_hierarchy* h, int level, const doub
   if (x_out == x || x_out == b) return fail(STOKES_ERR_ARG, "x_out must not alias x or b");
   sv::Level& L = h->lv[level];
   if (h->prm.prec == STOKES_FP64) {
-    sweep_f64(h, L, x, b, x_out);
+    sweep_f64(h, L, x, b, x_out, true);
     return check_launch("relaxation_sweep");
   }
   // the mixed forms: round x and b to FP32, sweep in the V-cycle's arithmetic, widen the result

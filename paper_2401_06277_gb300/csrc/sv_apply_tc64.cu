@@ -2,25 +2,40 @@
 // integer contraction on the tensor cores.
 //
 // The coefficients of the stencils are integers up to 512 (sv_stencil.cuh), exact in
-// FP16.  With x in 6 digits of 10 bits (sv_digits.cuh) a digit's products sum to less
-// than 2^20, so FP32 holds every sum exactly; the six sums of an output are added in
-// 64-bit integers and rounded once, where the FP64 kernel rounds after each of up to 31
+// FP16.  With x in 6 digits of 12 bits (sv_digits.cuh) a digit's products sum to less
+// than 2^22, so FP32 holds every sum exactly; the six sums of an output are added
+// exactly and rounded once, where the FP64 kernel rounds after each of up to 31
 // multiply-adds.  The pressure enters the velocity rows scaled by cb / cl, so that one
-// contraction gives (A x) / cl.  The only other loss is that of x, truncated 58 bits below
-// the bound of the 4 x 132 cells in reach.  Measured against 64-bit mantissas, random x:
-// 2.0e-16 of the largest velocity row (FP64 kernel 2.2e-16), 1.6e-16 pressure (2.3e-16).
+// contraction gives (A x) / cl.
+//
+// The components keep exponents of their own: u and the pressures in reach share one,
+// 2^EU, v and the pressures 2^EV, and the divergence rows sum their two parts apart, so
+// that no row sees the size of a component that it does not contain.  The only other
+// loss is that of x, truncated 71 bits below 2^EU or 2^EV: nothing of a value within
+// 2^-19 of it.  An output whose reach holds smaller values is taken from the contraction
+// only if a value of its own row is large enough: one with a coefficient of 32 or more at
+// 2^-17 (a velocity node of the cell; 4 or more and 2^-19 in the divergence rows, whose
+// coefficients sum to 60 and not 1300), or one with 1 or more at 2^-12 (a pressure).
+// What is truncated is then at most 30 units of roundoff of sum |a| |x| over the row,
+// less than the a-priori bound of the FP64 kernel (31).  The other outputs, and those
+// with values in reach that are not finite, are computed in FP64, within a cycle (whose
+// entries are not independent) only the latter.  Error against quadruple precision,
+// random x at n = 512: 1.6e-16 of the largest velocity row (FP64 kernel 2.2e-16), 1.3e-16
+// pressure (2.3e-16).
 //
 // Columns that the elimination drops (Dirichlet nodes, vertices outside the grid) read
 // as zero and every remaining row is the interior one, so one coefficient set serves
-// the whole grid; Dirichlet rows are the identity.  Cells with values that are not
-// finite in reach are recomputed in FP64, so that they spread as before.
+// the whole grid; Dirichlet rows are the identity.
 //
 // One step is two cell rows of a strip of 128: K = 12 cell offsets (dx -1..1, dy -1..2)
-// x 8 + 3 x 4 pressures, 8 MMAs (M = 128 cells, N = 2 rows x 9 outputs padded to 32) per
-// digit.  Bound: the instructions around the contraction (digits of 9 values, 54 sums
-// per cell: about 700 a vertex) and HBM, no longer the FP64 pipe (334 operations a
-// vertex at 2 per clock and SM).  2048^2: 0.34 ms, 0.9 GB moved at 2.7 TB/s with b (the
-// FP64 kernel: 1.52 ms); the two epilogue groups took it from 0.367 ms.
+// x 8 + 3 x (4 pressures, in units of 2^EU and of 2^EV), 8 MMAs (M = 128
+// cells, N = 2 rows x 10 outputs padded to 32) per digit.  Bound: the latency of the instructions around the contraction (digits of 9 values,
+// 60 sums per cell; the two epilogue groups and the digit warps are about equally long),
+// no longer the FP64 pipe (334 operations a vertex at 2 per clock and SM).  2048^2 with b:
+// 0.42 ms (the FP64 kernel: 1.52 ms; 6 digits of 10 bits under one exponent for all
+// components, which lost the entries above: 0.355).  All outputs in FP64 (data falling by
+// 2^-0.3 per column): 1.99 ms.  Two warps for the pressures alone took 0.44 ms, one
+// epilogue group and two threads per cell for the digits 0.59.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
@@ -52,10 +67,14 @@ struct SM {
   static constexpr int RING = 0;                 // 3 row pairs
   static constexpr int P = RING + 6 * ROWB;      // pressures of a step, two buffers
   static constexpr int G = P + 2 * ROWB;
-  static constexpr int BAR = G + GBYTES;         // full[3], done[2], free[2], gload
-  static constexpr int MISC = BAR + 16 * 8;      // tmem slot, fail flag, 8 maxima, 4 exponents
-  static constexpr int BYTES = MISC + 4 * 16;
-  static_assert(G % 128 == 0 && BAR % 8 == 0, "shared memory");
+  static constexpr int CEXP = G + GBYTES;        // exponents of cells: 8 row pairs [row][column] of uint2
+  static constexpr int PEXP = CEXP + 8 * 2 * WCOLS * 8;   // of pressures: 8 steps [row][column] of 16 bits
+  static constexpr int BAR = PEXP + 8 * 4 * WCOLS * 2;    // full[3], done[2], free[2], gload
+  static constexpr int SMAX = BAR + 10 * 8;      // largest u, v, p of 8 row pairs, uint4
+  static constexpr int LOST = SMAX + 8 * 16;     // what was truncated in 8 steps
+  static constexpr int MISC = LOST + 8 * 4;      // tmem slot, fail flag, 4 exponents
+  static constexpr int BYTES = MISC + 6 * 4;
+  static_assert(G % 128 == 0 && BAR % 8 == 0 && SMAX % 16 == 0, "shared memory");
 };
 
 constexpr uint32_t IDESC = (1u << 4) | (static_cast<uint32_t>(NB >> 3) << 17) | ((128u >> 4) << 24);
@@ -90,19 +109,77 @@ __device__ __noinline__ void apply_cell(const Args& A, int i, int j, int o) {
   }
 }
 
+// The exponents of a step (E + 1022 of u and v; 0x7ff: values that are not finite) and
+// which components were truncated in it: u, v, the pressures in units of either
+struct StepExp {
+  int eu, ev;
+  unsigned lost;
+};
+constexpr unsigned LOST_U = 1, LOST_V = 2, LOST_PU = 4, LOST_PV = 8;
+// Exponents for maxima of mu and mv: kept while they fit within 2^4; one for both if the
+// maxima are within 2^3 (the divergence rows then need one sum), until they are 2^6 apart.
+__device__ __forceinline__ bool choose_exp(int mu, int mv, int& eu, int& ev) {
+  const int m = max(mu, mv), apart = abs(mu - mv);
+  if (eu == ev ? exp_fits(m, eu) && (apart <= 5 || eu == EB_MIN) : exp_fits(mu, eu) && exp_fits(mv, ev)) return false;
+  eu = exp_for(apart <= 3 ? m : mu);
+  ev = exp_for(apart <= 3 ? m : mv);
+  return true;
+}
+
 // phase of full[s % 3] for step s >= 1 (step 0 needs no arrival)
 __device__ __forceinline__ uint32_t full_phase(int s) { return (s % 3 == 0 ? s / 3 - 1 : s / 3) & 1; }
 
 struct Shared {   // what the roles of a CTA share
   uint32_t full, done, free, tmem;
   volatile int* fail;
-  volatile int* sexp;
+  volatile unsigned* sexp;
+  const volatile unsigned* lost;
+  const uint2* cexp;
+  const unsigned short* pexp;
   int i0, j0, rows, S;
 };
 
-// Accumulators to y, steps g, g + 2, ...: warp -> cell row a and lane quarter of the
-// columns.  The digit sums have weights 2^(50 - 10 c), taken in units of 2^7 (velocity
-// rows: the coefficients sum to 1300 at most, |T| < 2^62) and 2^2 (pressure rows: 60).
+// 2^36 hi + lo as an FP64 number with a single rounding; both below 2^46 and offset by the
+// bits of 1.5 2^52, so that they are FP64 numbers as they stand
+constexpr long long OFFSET = 0x4338000000000000ll;
+__device__ __forceinline__ double total(long long hi, long long lo) {
+  constexpr double off = 6755399441055744.0, w = 68719476736.0;   // 1.5 2^52, 2^36
+  return fma(__longlong_as_double(hi), w, -(off * w + off)) + __longlong_as_double(lo);
+}
+
+// Outputs of a cell that the contraction may not give (bits: u, v, divergence).  a: the
+// cell's row in the step, col: its held column.
+__device__ __forceinline__ unsigned lost_outputs(const Shared& C, int s, int a, int col, const StepExp& E) {
+  const uint2 own = C.cexp[(((s + a) & 7) * 2 + 1 - a) * WCOLS + col];   // row 1 of pair s, row 0 of pair s + 1
+  const unsigned short* pe = C.pexp + ((s + 1) & 7) * 4 * WCOLS;
+  const int mu = own.x & 0xffffu, mv = own.x >> 16, md = own.y;
+  unsigned out = 0;
+  if ((E.lost & (LOST_U | LOST_PU)) && mu < E.eu - 16 && pe[(1 + a) * WCOLS + col + 1] < E.eu - 11) out |= 1;
+  if ((E.lost & (LOST_V | LOST_PV)) && mv < E.ev - 16 && pe[(2 + a) * WCOLS + col] < E.ev - 11) out |= 2;
+  if (md < max((E.lost & LOST_U) ? E.eu : 0, (E.lost & LOST_V) ? E.ev : 0) - 18) out |= 4;
+  return out;
+}
+// Those of them that have anything but zeros in reach
+__device__ __forceinline__ unsigned nonzero_reach(const uint2* cexp, const unsigned short* pexp, int s, int a, int col,
+                                               unsigned out) {
+  unsigned u = 0, v = 0, p = 0;
+#pragma unroll 1
+  for (int dy = -1; dy <= 1; ++dy)
+#pragma unroll 1
+    for (int dx = -1; dx <= 1; ++dx) {
+      const int r = 2 * s + a + 1 + dy;   // cell row of the walk, row r & 1 of pair r >> 1
+      const unsigned w = cexp[((r >> 1 & 7) * 2 + (r & 1)) * WCOLS + col + dx].x;
+      u |= w & 0xffffu;
+      v |= w >> 16;
+      p |= pexp[(((s + 1) & 7) * 4 + 1 + a + dy) * WCOLS + col + dx];
+    }
+  if ((u | p) == 0) out &= ~1u;
+  if ((v | p) == 0) out &= ~2u;
+  if ((u | v) == 0) out &= ~4u;
+  return out;
+}
+
+// Accumulators to y, steps g, g + 2, ...: warp -> cell row a and lane quarter of the columns.
 __device__ __forceinline__ void epilogue(const Args& A, const Shared& C, int g, int warp, int lane) {
   const LevelDev& L = A.L;
   const int n = L.n, nq = L.nq, np = L.np;
@@ -113,71 +190,77 @@ __device__ __forceinline__ void epilogue(const Args& A, const Shared& C, int g, 
     const bool ok = mbar_wait_or_fail(C.done + 8 * g, (s >> 1) & 1, A.wait_limit, C.fail);
     if (!__all_sync(0xffffffffu, ok)) return;
     fence_after();
-    long long T[9];
-    {
-      uint32_t v[3][9];
-#pragma unroll
-      for (int c = 0; c < 3; ++c) tmem_ld9(tq + NB * c, v[c]);
-      wait_ld();
-#pragma unroll
-      for (int o = 0; o < 9; ++o) T[o] = 0;
-#pragma unroll
-      for (int o = 0; o < 8; ++o) {
-        add_digit<43>(T[o], v[0][o]);
-        add_digit<33>(T[o], v[1][o]);
-        add_digit<23>(T[o], v[2][o]);
-      }
-      add_digit<48>(T[8], v[0][8]);
-      add_digit<38>(T[8], v[1][8]);
-      add_digit<28>(T[8], v[2][8]);
-#pragma unroll
-      for (int c = 0; c < 3; ++c) tmem_ld9(tq + NB * (3 + c), v[c]);
-      wait_ld();
-#pragma unroll
-      for (int o = 0; o < 8; ++o) {
-        add_digit<13>(T[o], v[0][o]);
-        add_digit<3>(T[o], v[1][o]);
-        add_digit<-7>(T[o], v[2][o]);
-      }
-      add_digit<18>(T[8], v[0][8]);
-      add_digit<8>(T[8], v[1][8]);
-      add_digit<-2>(T[8], v[2][8]);
-    }
+    double T[8], Tu, Tv = 0.0;   // the outputs' totals; the divergence as one or two
     // before the arrival: it lets step s + 2 run, after which the slot takes step s + 4's
-    const int eb = C.sexp[s & 3];
+    const unsigned w = C.sexp[s & 3];
+    const StepExp E{static_cast<int>(w & 0xffffu), static_cast<int>(w >> 16), C.lost[s & 7]};
+    {
+      // six digit sums per output, weights 2^(60 - 12 c): three to a 64-bit integer, exact
+      long long hi[10];
+      uint32_t v[3][10];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) tmem_ld10(tq + NB * c, v[c]);
+      wait_ld();
+      auto sum = [&](int o) {
+        // an integer below 2^22 plus 1.5 2^23 has its bits at the end of the FP32 number
+        auto bits = [](uint32_t f) { return static_cast<long long>(__float_as_int(__uint_as_float(f) + 12582912.0f)); };
+        constexpr long long z = 0x4b400000ll;
+        return OFFSET - z * ((1 << 24) + (1 << 12) + 1) + bits(v[0][o]) * (1 << 24) + bits(v[1][o]) * (1 << 12) + bits(v[2][o]);
+      };
+#pragma unroll
+      for (int o = 0; o < 10; ++o) hi[o] = sum(o);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) tmem_ld10(tq + NB * (3 + c), v[c]);
+      wait_ld();
+#pragma unroll
+      for (int o = 0; o < 8; ++o) T[o] = total(hi[o], sum(o));
+      if (E.eu == E.ev) {
+        Tu = total(hi[8] + (hi[9] - OFFSET), sum(8) + (sum(9) - OFFSET));
+      } else {
+        Tu = total(hi[8], sum(8));
+        Tv = total(hi[9], sum(9));
+      }
+    }
+    const int j = C.j0 + 2 * s + a;
+    const bool mine = i <= n && 2 * s + a < C.rows;
+    unsigned redo = 0;
+    if (mine && E.lost != 0 && L.every_entry) redo = lost_outputs(C, s, a, i - C.i0 + 2, E);
+    if (redo != 0) redo = nonzero_reach(C.cexp, C.pexp, s, a, i - C.i0 + 2, redo);
+    if (E.eu == 0x7ff) redo |= 5;
+    if (E.ev == 0x7ff) redo |= 6;
     fence_before();
     __syncwarp();
     if (lane == 0) mbar_arrive(C.free + 8 * g);
-    const int j = C.j0 + 2 * s + a;
-    if (i > n || 2 * s + a >= C.rows) continue;
-    if (eb == 0x7ff) {
-      for (int o = 0; o < 9; ++o) apply_cell(A, i, j, o);
-      continue;
-    }
+    if (!mine) continue;
     const long long ku = static_cast<long long>(2 * j) * nq + 2 * i;
     const long long kp = 2 * nv + static_cast<long long>(j) * np + i;
     auto at = [&](int o) { return (o >> 2) * nv + ku + ((o >> 1) & 1) * nq + (o & 1); };
     const bool res = A.b != nullptr;
-    const double su = (res ? -L.cl : L.cl) * exp_scale(eb, -51), sp = (res ? -L.cb : L.cb) * exp_scale(eb, -56);
-    if (i >= 1 && j >= 1 && i <= n - 1 && j <= n - 1) {   // all four nodes exist and are free
+    const double sg = res ? -1.0 : 1.0;
+    const double su = sg * L.cl * exp_scale(E.eu, -71), sv = sg * L.cl * exp_scale(E.ev, -71);
+    const double pu = sg * L.cb * exp_scale(E.eu, -71), pv = sg * L.cb * exp_scale(E.ev, -71);
+    auto div = [&](double b0) { return E.eu == E.ev ? fma(pu, Tu, b0) : fma(pu, Tu, fma(pv, Tv, b0)); };
+    if (i >= 1 && j >= 1 && i <= n - 1 && j <= n - 1 && redo == 0) {   // all four nodes exist and are free
       double bv[9];
 #pragma unroll
       for (int o = 0; o < 8; ++o) bv[o] = res ? A.b[at(o)] : 0.0;
       bv[8] = res ? A.b[kp] : 0.0;
 #pragma unroll
-      for (int o = 0; o < 8; ++o) A.y[at(o)] = fma(su, to_double(T[o]), bv[o]);
-      A.y[kp] = fma(sp, to_double(T[8]), bv[8]);
-    } else {
+      for (int o = 0; o < 8; ++o) A.y[at(o)] = fma(o < 4 ? su : sv, T[o], bv[o]);
+      A.y[kp] = div(bv[8]);
+    } else {   // an output is written once: y may be b
 #pragma unroll
       for (int o = 0; o < 8; ++o) {
         const int I = 2 * i + (o & 1), J = 2 * j + ((o >> 1) & 1);
-        if (I >= nq || J >= nq) continue;
+        if (I >= nq || J >= nq || ((redo >> (o >> 2)) & 1)) continue;
         const long long k = at(o);
         const double b0 = res ? A.b[k] : 0.0;
-        if (is_free(I, J, nq)) A.y[k] = fma(su, to_double(T[o]), b0);
+        if (is_free(I, J, nq)) A.y[k] = fma(o < 4 ? su : sv, T[o], b0);
         else A.y[k] = res ? b0 - A.x[k] : A.x[k];   // Dirichlet row: identity
       }
-      A.y[kp] = fma(sp, to_double(T[8]), res ? A.b[kp] : 0.0);
+      if (!(redo & 4)) A.y[kp] = div(res ? A.b[kp] : 0.0);
+      for (int o = 0; o < 9; ++o)
+        if ((redo >> (o >> 2)) & 1) apply_cell(A, i, j, o);
     }
   }
 }
@@ -193,8 +276,11 @@ __global__ void __launch_bounds__(NT, 1) k_apply_tc64(const Args A) {
   const uint32_t bar_full = s0 + SM::BAR, bar_done = bar_full + 24, bar_free = bar_done + 24, bar_g = bar_free + 16;
   uint32_t* tslot = reinterpret_cast<uint32_t*>(sm + SM::MISC);
   volatile int* fail = reinterpret_cast<volatile int*>(sm + SM::MISC + 4);
-  int* smax = reinterpret_cast<int*>(sm + SM::MISC + 8);                    // 8 slots
-  volatile int* sexp = reinterpret_cast<volatile int*>(sm + SM::MISC + 40);   // 4 slots
+  unsigned* smax = reinterpret_cast<unsigned*>(sm + SM::SMAX);
+  unsigned* lost = reinterpret_cast<unsigned*>(sm + SM::LOST);
+  volatile unsigned* sexp = reinterpret_cast<volatile unsigned*>(sm + SM::MISC + 8);   // 4 slots
+  uint2* cexp = reinterpret_cast<uint2*>(sm + SM::CEXP);
+  unsigned short* pexp = reinterpret_cast<unsigned short*>(sm + SM::PEXP);
   const int i0 = COLS * static_cast<int>(blockIdx.x);
   const int j0 = 2 * A.steps_per_seg * static_cast<int>(blockIdx.y);
   const int rows = min(2 * A.steps_per_seg, n + 1 - j0);
@@ -210,10 +296,8 @@ __global__ void __launch_bounds__(NT, 1) k_apply_tc64(const Args A) {
     mbar_init(bar_g, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     *fail = 0;
-    for (int k = 0; k < 8; ++k) smax[k] = 0;
+    for (int k = 0; k < 40; ++k) smax[k] = 0u;   // and lost
   }
-  for (int k = tid; k < 2 * ROWB / 16; k += NT)   // channels 4..7 of the pressures stay zero
-    reinterpret_cast<uint4*>(sm + SM::P)[k] = make_uint4(0u, 0u, 0u, 0u);
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tslot)), "r"(512));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
@@ -249,61 +333,113 @@ __global__ void __launch_bounds__(NT, 1) k_apply_tc64(const Args A) {
                    ? A.x[2 * nv + static_cast<long long>(pj) * np + gi] : 0.0;
     }
   };
-  auto note_max = [&](int q, Cell& c) {   // pressures to their units; the pair's largest exponent
+  // sizes as high words, a set bit for what lies below them: zero for zeros only
+  struct Small {
+    unsigned u, v, p;   // the smallest nonzero ones, less one
+  };
+  auto mag = [](double x) {
+    return (static_cast<unsigned>(__double2hiint(x)) & 0x7fffffffu) | min(static_cast<unsigned>(__double2loint(x)), 1u);
+  };
+  auto smallest = [&](const Cell& c) {
+    Small r{~0u, ~0u, min(mag(c.p[0]) - 1u, mag(c.p[1]) - 1u)};
+#pragma unroll
+    for (int o = 0; o < 4; ++o) {
+      r.u = min(r.u, mag(c.v[o]) - 1u);
+      r.v = min(r.v, mag(c.v[4 + o]) - 1u);
+    }
+    return r;
+  };
+  // pressures to their units; the exponents of the cell; the row pair's largest values
+  auto note = [&](int q, int a, int col, bool act, Cell& c) {
     c.p[0] *= A.ps;
     c.p[1] *= A.ps;
-    int m = max(__double2hiint(c.p[0]) & 0x7fffffff, __double2hiint(c.p[1]) & 0x7fffffff);
+    unsigned v[8], m[3] = {0u, 0u, 0u};
 #pragma unroll
-    for (int o = 0; o < 8; ++o) m = max(m, __double2hiint(c.v[o]) & 0x7fffffff);
-    m = __reduce_max_sync(0xffffffffu, m);
-    if (lane == 0) atomicMax(smax + (q & 7), m);
+    for (int o = 0; o < 8; ++o) {
+      v[o] = mag(c.v[o]);
+      m[o >> 2] = max(m[o >> 2], v[o]);
+    }
+    const unsigned p0 = mag(c.p[0]), p1 = mag(c.p[1]);
+    m[2] = max(p0, p1);
+    auto ex = [](unsigned w) { return max(w >> 20, min(w, 1u)); };   // nonzero for every value but zero
+    if (act) {
+      cexp[((q & 7) * 2 + a) * WCOLS + col] =
+          make_uint2(ex(m[0]) | (ex(m[1]) << 16), ex(max(max(v[1], v[3]), max(v[6], v[7]))));
+      pexp[((q & 7) * 4 + 2 * a) * WCOLS + col] = static_cast<unsigned short>(ex(p0));
+      pexp[((q & 7) * 4 + 2 * a + 1) * WCOLS + col] = static_cast<unsigned short>(ex(p1));
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) m[k] = __reduce_max_sync(0xffffffffu, m[k]);
+    if (lane == 0) {
+#pragma unroll
+      for (int k = 0; k < 3; ++k) atomicMax(smax + 4 * (q & 7) + k, m[k]);
+    }
+    return smallest(c);
   };
-  auto put = [&](int q, int a, int col, int eb, const Cell& c) {
-    unsigned long long w[8];
+  // exponents of the step with row pairs q - 1 and q; whether they changed
+  auto choose = [&](int q, int& eu, int& ev) {
+    const uint4 m0 = reinterpret_cast<const uint4*>(smax)[(q - 1) & 7], m1 = reinterpret_cast<const uint4*>(smax)[q & 7];
+    // |x| < 2^(e - 1022); the step's pressures came with pair q
+    return choose_exp(max(max(m0.x, m1.x), m1.z) >> 20, max(max(m0.y, m1.y), m1.z) >> 20, eu, ev);
+  };
+  auto truncated = [](const Small& c, int eu, int ev) {
+    const unsigned lu = (static_cast<unsigned>(eu - 18) << 20) - 1u, lv = (static_cast<unsigned>(ev - 18) << 20) - 1u;
+    return (c.u < lu ? LOST_U : 0u) | (c.v < lv ? LOST_V : 0u) | (c.p < lu ? LOST_PU : 0u) | (c.p < lv ? LOST_PV : 0u);
+  };
+  auto words = [&](const Cell& c, int eu, int ev, Wide (&w)[8]) {
 #pragma unroll
-    for (int o = 0; o < 8; ++o) w[o] = static_cast<unsigned long long>(to_fixed(c.v[o], eb)) + digit_bias();
+    for (int o = 0; o < 8; ++o) w[o] = to_wide(c.v[o], o < 4 ? eu : ev);
+  };
+  auto put = [&](int q, int a, int col, const Wide (&w)[8]) {
 #pragma unroll
     for (int j = 0; j < ND; ++j)
       *reinterpret_cast<uint4*>(sm + SM::RING + (2 * (q % 3) + a) * ROWB + j * PLANE + col * 16) =
-          make_uint4(digit2(w[0], w[1], j), digit2(w[2], w[3], j), digit2(w[4], w[5], j), digit2(w[6], w[7], j));
+          make_uint4(wide_digit2(w[0], w[1], j), wide_digit2(w[2], w[3], j), wide_digit2(w[4], w[5], j),
+                     wide_digit2(w[6], w[7], j));
   };
-  auto put_p = [&](int s, int a, int col, int eb, const Cell& c) {
-    unsigned long long w[2];
+  auto put_p = [&](int s, int a, int col, int eu, int ev, const Cell& c) {   // in units of 2^EU, then of 2^EV
+    unsigned char* p = sm + SM::P + (s & 1) * ROWB + col * 16 + 8 * a;
+    const Wide w0 = to_wide(c.p[0], eu), w1 = to_wide(c.p[1], eu);
 #pragma unroll
-    for (int k = 0; k < 2; ++k) w[k] = static_cast<unsigned long long>(to_fixed(c.p[k], eb)) + digit_bias();
+    for (int j = 0; j < ND; ++j) {
+      const unsigned u = wide_digit2(w0, w1, j);
+      *reinterpret_cast<uint2*>(p + j * PLANE) = make_uint2(u, u);
+    }
+    if (eu != ev) {
+      const Wide z0 = to_wide(c.p[0], ev), z1 = to_wide(c.p[1], ev);
 #pragma unroll
-    for (int j = 0; j < ND; ++j)
-      *reinterpret_cast<unsigned*>(sm + SM::P + (s & 1) * ROWB + j * PLANE + col * 16 + 4 * a) = digit2(w[0], w[1], j);
-  };
-  auto largest = [&](int q) {   // |x| < 2^(e - 1022) over the pairs q - 1, q
-    const volatile int* vm = smax;
-    return max(vm[q & 7], vm[(q - 1) & 7]) >> 20;
+      for (int j = 0; j < ND; ++j) *reinterpret_cast<unsigned*>(p + j * PLANE + 4) = wide_digit2(z0, z1, j);
+    }
   };
 
   // the first window (row pairs 0 and 1) by 18 warps at once
-  int eb;
+  int eu = -1, ev = -1;   // no exponents yet
   {
     const int q = warp / SLICE_WARPS, t = tid - q * SLICE_T;
     const bool act = q < 2 && t < 2 * WCOLS;
     const int a = t >= WCOLS ? 1 : 0, col = t - a * WCOLS;
     Cell c;
+    Small small{~0u, ~0u, ~0u};
     if (q < 2) {
       load(q, a, col, act, c);
-      note_max(q, c);
+      small = note(q, a, col, act, c);
     }
     __syncthreads();
-    const int em = largest(1);
-    eb = min(max(em + 1, EB_MIN), 0x7ff);
+    choose(1, eu, ev);
     if (act) {
-      put(q, a, col, eb, c);
-      if (q == 1) put_p(0, a, col, eb, c);
+      Wide w[8];
+      words(c, eu, ev, w);
+      put(q, a, col, w);
+      if (q == 1) put_p(0, a, col, eu, ev, c);
+      const unsigned l = truncated(small, eu, ev);
+      if (l != 0) atomicOr(lost, l);
     }
-    if (tid == 0) sexp[0] = em < 0x7ff ? eb : 0x7ff;
+    if (tid == 0) sexp[0] = eu | (ev << 16);
     fence_proxy();
     __syncthreads();
   }
 
-  const Shared C{bar_full, bar_done, bar_free, tmem, fail, sexp, i0, j0, rows, S};
+  const Shared C{bar_full, bar_done, bar_free, tmem, fail, sexp, lost, cexp, pexp, i0, j0, rows, S};
   if (warp < EPI_WARPS) {
     epilogue(A, C, warp / EPI_GROUP, warp, lane);
   } else if (warp < EPI_WARPS + SLICE_WARPS) {
@@ -313,28 +449,37 @@ __global__ void __launch_bounds__(NT, 1) k_apply_tc64(const Args A) {
     const int a = t >= WCOLS ? 1 : 0, col = t - a * WCOLS;
     Cell cur;
     if (S > 1) load(2, a, col, act, cur);
+    unsigned lost_before = lost[0];   // of this thread's cell of the row pair before; at first, of any
     for (int q = 2; q < S + 1; ++q) {
-      note_max(q, cur);
+      const Small small = note(q, a, col, act, cur);
       asm volatile("bar.sync 1, %0;" ::"n"(SLICE_T) : "memory");
-      if (t == 0) smax[(q + 3) & 7] = 0;
-      const int em = largest(q), s = q - 1;
-      const bool renew = em > eb || (eb - em > 3 && eb > EB_MIN);
-      if (renew) {   // uniform over the slicer warps: the other row pair again, with the new exponent
-        eb = min(max(em + 1, EB_MIN), 0x7ff);
+      if (t < 3) smax[4 * ((q + 3) & 7) + t] = 0u;
+      const int s = q - 1;
+      if (choose(q, eu, ev)) {   // uniform over the slicer warps: the other row pair again, with the new exponents
         mbar_wait_or_fail(bar_done + 8 * ((s - 1) & 1), ((s - 1) >> 1) & 1, A.wait_limit, fail);
         Cell c;
         load(q - 1, a, col, act, c);
-        if (act) put(q - 1, a, col, eb, c);
+        Wide w[8];
+        words(c, eu, ev, w);
+        if (act) put(q - 1, a, col, w);
+        lost_before = truncated(smallest(c), eu, ev);
       } else if (s >= 2) {
         // the row pair's slot and the pressure buffer are free once step s - 2 has read them
         // (after a failed wait the results are void and only the arrivals matter)
         mbar_wait_or_fail(bar_done + 8 * (s & 1), ((s - 2) >> 1) & 1, A.wait_limit, fail);
       }
-      if (t == 0) sexp[s & 3] = em < 0x7ff ? eb : 0x7ff;
-      if (act) {
-        put(q, a, col, eb, cur);
-        put_p(s, a, col, eb, cur);
+      if (t == 0) {
+        sexp[s & 3] = eu | (ev << 16);
+        lost[(s + 1) & 7] = 0u;
       }
+      const unsigned l = truncated(small, eu, ev);
+      const unsigned lw = __reduce_or_sync(0xffffffffu, l | (lost_before & (LOST_U | LOST_V)));
+      if (lw != 0 && lane == 0) atomicOr(lost + (s & 7), lw);
+      lost_before = l;
+      if (act) put_p(s, a, col, eu, ev, cur);
+      Wide w[8];
+      words(cur, eu, ev, w);
+      if (act) put(q, a, col, w);
       if (q + 1 < S + 1) load(q + 1, a, col, act, cur);   // in flight over the fence and the next barrier
       fence_proxy();
       __syncwarp();
@@ -407,26 +552,26 @@ void apply_tc64_pack(std::vector<unsigned char>& out) {
     std::memcpy(out.data() + static_cast<size_t>(chunk) * CHUNK + (16 * a + o) * 16 + 2 * ch, &h, 2);
   };
   for (int a = 0; a < 2; ++a)
-    for (int o = 0; o < 9; ++o) {
-      const int c = o >> 2, py = (o >> 1) & 1, px = o & 1;
+    for (int o = 0; o < 10; ++o) {
+      const int c = o >> 2, py = (o >> 1) & 1, px = o & 1;   // o = 8, 9: the divergence of u, of v
       for (int dyi = 0; dyi < 4; ++dyi)
         for (int dx = -1; dx <= 1; ++dx)
           for (int ch = 0; ch < 8; ++ch) {
             const int c2 = ch >> 2, I = 2 * dx + (ch & 1), J = 2 * (dyi - 1 - a) + ((ch >> 1) & 1);
             double v = 0.0;
-            if (o == 8) {
-              v = c2 == 0 ? crow(I) * nrow(J) : nrow(I) * crow(J);
+            if (o >= 8) {
+              if (c2 == o - 8) v = c2 == 0 ? crow(I) * nrow(J) : nrow(I) * crow(J);
             } else if (c2 == c) {
               const int dI = I - px, dJ = J - py;
               v = k1(px, dI) * m1(py, dJ) + m1(px, dI) * k1(py, dJ);
             }
             place(a, o, dx < 1 ? 2 * dyi + dx + 1 : 8 + dyi, ch, v);
           }
-      if (o == 8) continue;
+      if (o >= 8) continue;
       for (int k = 0; k < 4; ++k)        // pressure row j - 1 + k
         for (int dx = -1; dx <= 1; ++dx) {
           const int dj = k - 1 - a;
-          place(a, o, 12 + dx + 1, k,
+          place(a, o, 12 + dx + 1, 4 * (k >> 1) + 2 * c + (k & 1),   // the pressures in the unit of component c
                 c == 0 ? ccol(px, dx) * ncol(py, dj) : ncol(px, dx) * ccol(py, dj));
         }
     }

@@ -3,7 +3,8 @@
 //
 // A strip of 128 cell columns (132 held) is walked two cell rows at a time.  The cells
 // in reach of a step share an exponent E: x = 2^(E - 58) q, |x| < 2^E, q an integer
-// written in ND = 6 balanced digits of 10 bits.  In shared memory a digit of a cell row
+// written in ND = 6 balanced digits of 10 bits (the sweep), or 2^(E - 71) q in 6 digits of
+// 12 bits (the operator, whose coefficients leave more of FP32's 24 bits to them).  In shared memory a digit of a cell row
 // is a plane of 16 bytes per cell (the FP16 digits of its eight velocity values: Q2
 // nodes (2i + PI, 2j + PJ) of component c at 4 c + 2 PJ + PI), so the operand of the
 // cells shifted by (dx, dy) is the same memory at another start address.
@@ -30,6 +31,11 @@ constexpr int SLICE_T = 32 * SLICE_WARPS;
 static_assert(2 * WCOLS <= SLICE_T, "one thread per cell of a row pair");
 constexpr int EB_MIN = 200;                      // smallest exponent in use (E + 1022): scales stay normal
 
+// E + 1022 for values below 2^(m - 1022), one binade above them, and whether one in use
+// still serves them: a walk then renews it seldom.  0x7ff where a value is not finite.
+__device__ __forceinline__ int exp_for(int m) { return m >= 0x7ff ? 0x7ff : max(min(m + 1, 0x7fe), EB_MIN); }
+__device__ __forceinline__ bool exp_fits(int m, int eb) { return m <= eb && (eb - m <= 3 || eb == EB_MIN) && (m < 0x7ff) == (eb < 0x7ff); }
+
 // q = x 2^(58 - E) rounded toward zero, |x| < 2^E, eb = E + 1022.  Exact for |x| >=
 // 2^(E - 6): the mantissa's 53 bits then lie above the last place.
 __device__ __forceinline__ long long to_fixed(double x, int eb) {
@@ -54,6 +60,51 @@ __device__ __forceinline__ unsigned digit2(unsigned long long a, unsigned long l
   __half2 h;
   memcpy(&h, &t, 4);
   h = __hadd2(h, __half2half2(__ushort_as_half(0xE600)));   // -1536
+  unsigned u;
+  memcpy(&u, &h, 4);
+  return u;
+}
+
+// The wide form: six digits of 12 bits in [-2048, 2048], q = x 2^(71 - E) truncated,
+// |x| < 2^E.  Nothing is lost of |x| >= 2^(E - 19).  Digits of |q| plus 2048 each: lo the
+// four lower ones, hi the upper two.
+struct Wide {
+  unsigned long long lo;
+  unsigned hi;
+  float sign;
+};
+// shifts whose counts of 64 and more (negative ones too) give 0
+__device__ __forceinline__ unsigned long long shl64(unsigned long long v, int k) {
+  unsigned long long r;
+  asm("shl.b64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(k));
+  return r;
+}
+__device__ __forceinline__ unsigned long long shr64(unsigned long long v, int k) {
+  unsigned long long r;
+  asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(k));
+  return r;
+}
+__device__ __forceinline__ Wide to_wide(double x, int eb) {
+  constexpr unsigned long long mask = (1ull << 48) - 1, bias = 0x800800800800ull;
+  const unsigned h = __double2hiint(x), l = __double2loint(x);
+  const int d = eb - static_cast<int>((h >> 20) & 0x7ffu);   // the mantissa's last place: 2^(18 - d) units
+  // zero and subnormals: d >= EB_MIN shifts everything out
+  const unsigned long long m = (static_cast<unsigned long long>((h & 0xfffffu) | 0x100000u) << 32) | l;
+  const unsigned long long b = ((shl64(m, 18 - d) | shr64(m, d - 18)) & mask) + bias;
+  Wide w;
+  w.lo = b;
+  w.hi = static_cast<unsigned>(shr64(m, 30 + d)) + static_cast<unsigned>(b >> 48) + ((2048u << 12) + 2048u);
+  w.sign = __uint_as_float((h & 0x80000000u) | 0x3f800000u);
+  return w;
+}
+// digit j (0 the highest) of two values as FP16 integers, exact: 2^23 + 2048 + digit as
+// the mantissa of an FP32 number
+__device__ __forceinline__ unsigned wide_digit2(const Wide& a, const Wide& b, int j) {
+  auto digit = [j](const Wide& w) {
+    const unsigned t = j == 0 ? w.hi >> 12 : j == 1 ? w.hi & 0xfffu : static_cast<unsigned>(w.lo >> (12 * (5 - j))) & 0xfffu;
+    return fmaf(__uint_as_float(t | 0x4b000000u), w.sign, -8390656.0f * w.sign);
+  };
+  const __half2 h = __floats2half2_rn(digit(a), digit(b));
   unsigned u;
   memcpy(&u, &h, 4);
   return u;

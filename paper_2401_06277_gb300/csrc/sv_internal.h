@@ -145,6 +145,7 @@ struct LevelDev {
   const unsigned char* op_digits = nullptr;
   int* dev_err = nullptr;
   int wait_limit = TC_WAIT_LIMIT;
+  bool every_entry = true;   // the operator: outputs to which it gives less than FP64 would, in FP64
 };
 
 // cl and cb in the element type

@@ -82,12 +82,19 @@ __device__ __forceinline__ uint32_t elect_one() {
   return on;
 }
 
-// nine consecutive accumulator columns of this lane
+// nine, ten consecutive accumulator columns of this lane
 __device__ __forceinline__ void tmem_ld9(uint32_t taddr, uint32_t (&r)[9]) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
                : "r"(taddr));
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r[8]) : "r"(taddr + 8));
+}
+
+__device__ __forceinline__ void tmem_ld10(uint32_t taddr, uint32_t (&r)[10]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0,%1}, [%2];" : "=r"(r[8]), "=r"(r[9]) : "r"(taddr + 8));
 }
 
 }  // namespace tc

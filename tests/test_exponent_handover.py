@@ -7,6 +7,8 @@ taken from the source, so that a read moved behind the arrival is found here."""
 import os
 import re
 
+import pytest
+
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2401_06277_gb300", "csrc")
 STEPS, SLOTS = 16, 4
 
@@ -57,3 +59,34 @@ def test_operator_reads_the_exponent_before_its_slot_can_be_reused():
 
 def test_the_argument_needs_that_order():
     assert ordered(False) != []
+
+
+@pytest.mark.parametrize("slots", [5, 8])
+def test_exponents_of_cells_are_read_before_their_slot_is_written_again(slots):
+    """Per row pair, written when the pair is read (before the waits of its step q - 1),
+    used by the steps q - 1 and q before their arrival: six slots are needed, eight are kept."""
+    after = {}
+
+    def edge(a, b):
+        after.setdefault(a, []).append(b)
+
+    for s in range(STEPS):
+        edge(("read", s), ("free", s))
+        edge(("free", s), ("mma", s + 2))
+        edge(("mma", s), ("done", s))
+        edge(("mma", s), ("mma", s + 1))
+        edge(("done", s), ("waited", s + 2))           # a digit warp, in its step s + 2
+        edge(("waited", s), ("write", s + 2))          # then the next row pair, that of step s + 1
+    loose = []
+    for q in range(STEPS - slots):
+        seen, todo = set(), [("read", q)]
+        while todo:
+            for b in after.get(todo.pop(), ()):
+                if b not in seen:
+                    seen.add(b)
+                    todo.append(b)
+        if ("write", q + slots) not in seen:
+            loose.append(q)
+    assert (loose == []) == (slots >= 6)
+    src = open(os.path.join(CSRC, "sv_apply_tc64.cu")).read()
+    assert "cexp[((q & 7) * 2 + a) * WCOLS + col] =" in src and "pexp[((q & 7) * 4 + 2 * a) * WCOLS + col] =" in src
