@@ -115,6 +115,9 @@ void free_all(stokes_hierarchy* h) {
   h->stencil_Gf = nullptr;
   cudaFree(h->stencil_digits);
   cudaFree(h->stencil_ring);
+  cudaFree(h->stencil_check.flags);
+  cudaFree(h->stencil_check.any);
+  h->stencil_check = sv::TC64Check{};
   h->stencil_ring = nullptr;
   h->stencil_G = nullptr;
   h->stencil_digits = nullptr;
@@ -214,7 +217,8 @@ sv::LevelDev cycle_level(const sv::Level& L) {
 // free whenever a sweep runs).  A mixed hierarchy has neither L.r nor FP64 scratch: its
 // FP64 sweep (stokes_vanka_sweep alone) takes two vectors of the Krylov basis, free
 // outside a solve, or a fused tile where the split sweep was asked for.
-// single: a sweep that the caller asked for.
+// single: a sweep that the caller asked for, whose every entry is to be as accurate as that
+// of FP64 patch solves.
 void sweep_f64(stokes_hierarchy* h, sv::Level& L, const double* x, const double* b, double* xo, bool single) {
   const sv::LevelDev d = single ? L.d : cycle_level(L);
   const bool mixed = h->prm.prec != STOKES_FP64;
@@ -223,10 +227,11 @@ void sweep_f64(stokes_hierarchy* h, sv::Level& L, const double* x, const double*
                                 mixed ? h->V : L.r, x, b, xo, h->stream);
   else if (h->prm.smoother == STOKES_SMOOTHER_PER_PATCH)
     sv::launch_simple_sweep(d, L.pinv, h->delta, L.r, x, b, xo, h->prm.omega, h->stream);
-  else if (L.vk_cfg == sv::VANKA_CFG_TC64)
+  else if (L.vk_cfg == sv::VANKA_CFG_TC64) {
+    if (single) ++h->stencil_check.call;
     sv::launch_vanka_tc64(d, h->stencil_digits, h->stencil_eu, h->stencil_ep, h->stencil_ring, x, b, xo, h->prm.omega,
-                          L.r, h->dev_err, h->tc_wait_limit, h->stream);
-  else if (L.vk_cfg == sv::VANKA_CFG_STENCIL)
+                          L.r, h->dev_err, h->tc_wait_limit, single ? h->stencil_check : sv::TC64Check{}, h->stream);
+  } else if (L.vk_cfg == sv::VANKA_CFG_STENCIL)
     sv::launch_vanka_stencil<double>(d, h->stencil_G, x, b, xo, h->prm.omega, L.r, h->stream);
   else if (sv::vanka_cfg_split(L.vk_cfg) && !mixed)
     sv::launch_vanka_split<double>(d, L.cd, h->fd, x, b, xo, h->prm.omega, h->delta, L.vk_cfg == sv::VANKA_CFG_SPLIT2,
@@ -1111,6 +1116,10 @@ stokes_status stokes_hierarchy_create(int n, double viscosity, const stokes_para
       if (e == cudaSuccess) e = dalloc(&h->stencil_ring, ring.size());
       if (e == cudaSuccess)
         e = cudaMemcpy(h->stencil_ring, ring.data(), ring.size() * sizeof(double), cudaMemcpyHostToDevice);
+      const size_t cells = static_cast<size_t>(n + 1) * (n + 1);
+      if (e == cudaSuccess) e = dalloc(&h->stencil_check.flags, cells);
+      if (e == cudaSuccess) e = dalloc(&h->stencil_check.any, 1);
+      if (e == cudaSuccess) e = cudaMemset(h->stencil_check.any, 0, sizeof(unsigned));
       if (e == cudaSuccess) e = sv::vanka_tc64_prepare();
       if (e != cudaSuccess) {
         free_all(h);

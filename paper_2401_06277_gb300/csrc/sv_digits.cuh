@@ -36,14 +36,14 @@ constexpr int EB_MIN = 200;                      // smallest exponent in use (E 
 __device__ __forceinline__ int exp_for(int m) { return m >= 0x7ff ? 0x7ff : max(min(m + 1, 0x7fe), EB_MIN); }
 __device__ __forceinline__ bool exp_fits(int m, int eb) { return m <= eb && (eb - m <= 3 || eb == EB_MIN) && (m < 0x7ff) == (eb < 0x7ff); }
 
-// q = x 2^(58 - E) rounded toward zero, |x| < 2^E, eb = E + 1022.  Exact for |x| >=
+// q = x 2^(58 - E) rounded to nearest, |x| < 2^E, eb = E + 1022.  Exact for |x| >=
 // 2^(E - 6): the mantissa's 53 bits then lie above the last place.
 __device__ __forceinline__ long long to_fixed(double x, int eb) {
   const unsigned hi = __double2hiint(x), lo = __double2loint(x);
   const int e = (hi >> 20) & 0x7ff, d = eb - e;
   const unsigned long long m = (static_cast<unsigned long long>((hi & 0xfffffu) | 0x100000u) << 32) | lo;
-  unsigned long long v = (m << 5) >> min(d, 63);    // 0 for d > 58
-  if (e == 0) v = 0;                                // zero, or subnormal
+  // zero and subnormals: d >= EB_MIN shifts everything out
+  const unsigned long long v = (((m << 6) >> min(d, 63)) + 1) >> 1;
   return static_cast<int>(hi) < 0 ? -static_cast<long long>(v) : static_cast<long long>(v);
 }
 

@@ -115,6 +115,15 @@ constexpr int TAIL_SPIN_LIMIT = 1 << 22;   // polls (about 64 ns apart) of a gri
 constexpr int BS_TYPE = 26, BS_TAB = NCLASS * BS_TYPE;
 std::vector<double> bs_schur_table();
 
+// Which outputs the contraction gives less than FP64 patch solves would (a byte per cell:
+// 1 velocities, 2 pressure), for the FP64 pass that follows, and the number of the last
+// call that found any.  A null `flags` leaves them as they are.
+struct TC64Check {
+  unsigned char* flags = nullptr;
+  unsigned* any = nullptr;
+  unsigned call = 0;
+};
+
 struct BSParams {
   const double* tab = nullptr;    // bs_schur_table on the device, in FP64
   const float* tabf = nullptr;    // and in FP32
@@ -243,6 +252,7 @@ struct stokes_hierarchy {
   unsigned char* stencil_digits = nullptr;   // and its interior cell type as tensor-core digits
   double* stencil_ring = nullptr;            // and the table of the cells near the boundary
   int stencil_eu = 0, stencil_ep = 0;        // exponents of the digits (tc64_pack)
+  sv::TC64Check stencil_check;               // single sweeps: outputs left to FP64 (finest-level size)
   unsigned char* op_digits = nullptr;        // integer coefficients of the tensor-core operator
   double* coarse_G = nullptr;    // N0 x N0 dense inverse of the bordered coarse system
   int N0 = 0;
@@ -376,7 +386,7 @@ bool tc64_pack(std::vector<unsigned char>& out, int* eu, int* ep);
 cudaError_t vanka_tc64_prepare();
 void launch_vanka_tc64(const LevelDev& L, const unsigned char* Gp, int eu, int ep, const double* Gd, const double* x,
                        const double* b, double* xo, double omega, double* rscratch, int* err, int wait_limit,
-                       cudaStream_t s);
+                       const TC64Check& check, cudaStream_t s);
 
 // FP64 operator / residual (b null: y = A x) as an exact digit contraction on the tensor
 // cores (sv_apply_tc64.cu); launch_apply<double> takes it on levels with L.op_digits.

@@ -8,7 +8,7 @@
 // therefore split into small integers whose products and sums FP32 holds exactly
 // (an error-free splitting, as in Ozaki, Ogita, Oishi and Rump, "Error-free
 // transformations of matrix multiplication", Numerical Algorithms 59, 2012):
-//   residual      r = 2^(E - 58) q, |r| < 2^E, q truncated to an integer, in
+//   residual      r = 2^(E - 58) q, |r| < 2^E, q rounded to an integer, in
 //                 6 balanced digits of 10 bits: q = sum_j d_j 1024^(5 - j), |d_j| <= 512
 //   coefficients  G = 2^(e_o - 62) g (e_o per output kind), 7 balanced digits of 9 bits,
 //                 |g_i| <= 256
@@ -18,9 +18,17 @@
 // 42) are kept; those left out are below 2^-64 of the largest product.  The 27
 // integers of an output are added in 64-bit integers (unit 2^16, the pressure's 2^14, of
 // the last digit pair's) and rounded to FP64 at the end.  A residual loses what lies 58
-// bits below the bound of the 6 x 132 cells in reach, at most 2^-54 of the largest of
+// bits below the bound 2^E of the 6 x 132 cells in reach, at most 2^-55 of the largest of
 // them; measured, a sweep's error against 64-bit mantissas is 2.6e-16 of the largest
 // velocity (FP64 patch solves: 7e-16 to 1.4e-15) and 2.0e-16 for the pressure (2.6e-16).
+//
+// Outputs whose own patches hold only much smaller residuals would lose by that against
+// FP64 patch solves, whose error follows their patches.  A single sweep therefore checks
+// its cells: where nothing within 2^-8 of 2^E (2^-10 for the pressure, whose coefficients
+// sum to less) lies in the patches of an output, that output is computed in FP64 by a
+// second launch (k_vanka_fp64_cells).  What is lost elsewhere is below 2^-51 of the largest
+// residual of the output's patches times the sum of its coefficients, less than the
+// measured error of FP64 patch solves.  The sweeps of a cycle do without.
 //
 // Decomposition.  A CTA owns a strip of 128 cell columns and walks up it two cell rows
 // at a time.  The digits of the cells lie in shared memory as planes [cell row][digit]
@@ -51,6 +59,8 @@
 // reads keep shared memory 97% busy, so the other warps' shared-memory accesses wait;
 // hence the two epilogue groups (0.55 -> 0.50 ms) and one barrier for two digit planes
 // (0.50 -> 0.49).  Small levels are bound by the prologue: 12.9 us at n = 64, 13.9 at 128.
+// With the check 0.53 ms, and where it finds cells, of a random residual none, of a
+// right-hand side with boundary data the strips along the walls: 2.5 ms; all cells 12.9 ms.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
@@ -88,9 +98,11 @@ struct SM {
   static constexpr int RING = 0;                         // 6 cell rows
   static constexpr int P = RING + 6 * ROWB;              // pressures of the step: [digit][column] 16 B
   static constexpr int G = P + ROWB;
-  static constexpr int BAR = (G + GBYTES + 7) / 8 * 8;                 // full[3] (plane pairs), done[2][6] (by step parity), free[3], gload
-  static constexpr int MISC = BAR + 22 * 8;              // tmem slot, fail flag, 8 maxima, 4 exponents
-  static constexpr int BYTES = MISC + 4 * 16;
+  static constexpr int CEXP = G + GBYTES;                // exponents of cells: 8 row pairs [row][column] of 16 bits
+  static constexpr int PEXP = CEXP + 8 * 2 * WCOLS * 2;  // of pressures: 8 row pairs [row][column]
+  static constexpr int BAR = (PEXP + 8 * 4 * WCOLS * 2 + 7) / 8 * 8;   // full[3] (plane pairs), done[2][6] (by step parity), free[3], gload
+  static constexpr int MISC = BAR + 22 * 8;              // tmem slot, fail flag, 8 maxima, 8 minima, 4 exponents
+  static constexpr int BYTES = MISC + 24 * 4;
   static_assert(G % 16 == 0 && BAR % 8 == 0 && BYTES <= 227 * 1024, "shared memory");
 };
 
@@ -125,6 +137,7 @@ struct Args {
   int steps_per_seg;
   int* err;
   int wait_limit;
+  const TC64Check check;      // flags null: every output is taken as it is
 };
 
 // FP64 dot products of the cells outside [3, n - 3]^2: three cell rows below and above,
@@ -172,24 +185,38 @@ __device__ __forceinline__ int cell_type(int n, const Band& b) {
 // each: 10,000 clocks of a sub-partition's FP64 unit).  PARTS = 4: one cell, four lanes per
 // output, for the grids on which the longest unit, not the work, sets the time.
 template <int PARTS>
-__device__ __forceinline__ void ring_velocity(const Args& A, int unit, int lane) {
+__device__ __forceinline__ void cell_velocity(const Args& A, const Band& b, int lane) {
   static_assert(PARTS == 1 || PARTS == 4, "lanes: 8 outputs x 4 cells or 4 parts");
   const LevelDev& L = A.L;
   const int n = L.n, nq = L.nq, np = L.np, o = lane & 7, part = PARTS == 4 ? lane >> 3 : 0;
   const long long nv = L.nv;
-  const Band b = band_of(n, unit, 4 / PARTS, PARTS == 4 ? 0 : lane >> 3);
   const double* g = A.Gd + static_cast<size_t>(cell_type(n, b)) * RT_TYPE + o;
+  const int px = o & 1, py = (o >> 1) & 1;
   double a0 = 0.0, a1 = 0.0;
-  for (int rJ = b.J0 + part; rJ <= b.J1; rJ += PARTS) {
+  auto node = [&](int rJ, int rI) {
     const int J = 2 * b.j - 4 + rJ;
-    const double* rr = A.r + static_cast<long long>(J) * nq + 2 * b.i - 4;
-    const double* gr = g + rJ * 144;
+    const double* rr = A.r + static_cast<long long>(J) * nq + 2 * b.i - 4 + rI;
+    const double* gr = g + (rJ * 9 + rI) * 16;
+    const bool ok = b.in && is_free(2 * b.i - 4 + rI, J, nq);
+    const double r0 = ok ? __ldg(rr) : 0.0, r1 = ok ? __ldg(rr + nv) : 0.0;
+    a0 = fma(__ldg(gr), r0, a0);
+    a1 = fma(__ldg(gr + 8), r1, a1);
+  };
+  if (PARTS == 1) {
+    for (int rJ = b.J0; rJ <= b.J1; ++rJ) {
 #pragma unroll 3
-    for (int rI = b.I0; rI <= b.I1; ++rI) {
-      const bool ok = b.in && is_free(2 * b.i - 4 + rI, J, nq);
-      const double r0 = ok ? __ldg(rr + rI) : 0.0, r1 = ok ? __ldg(rr + nv + rI) : 0.0;
-      a0 = fma(__ldg(gr + rI * 16), r0, a0);
-      a1 = fma(__ldg(gr + rI * 16 + 8), r1, a1);
+      for (int rI = b.I0; rI <= b.I1; ++rI) node(rJ, rI);
+    }
+  } else {   // every fourth node of the window (four wide at least)
+    int rJ = b.J0, rI = b.I0 + part;
+#pragma unroll 3
+    for (int e = (b.J1 - b.J0 + 1) * (b.I1 - b.I0 + 1) - part; e > 0; e -= PARTS) {
+      node(rJ, rI);
+      rI += PARTS;
+      if (rI > b.I1) {
+        rI -= b.I1 - b.I0 + 1;
+        ++rJ;
+      }
     }
   }
   double ap = 0.0;
@@ -205,18 +232,17 @@ __device__ __forceinline__ void ring_velocity(const Args& A, int unit, int lane)
     d += __shfl_xor_sync(0xffffffffu, d, 8);
     d += __shfl_xor_sync(0xffffffffu, d, 16);
   }
-  const int I = 2 * b.i + (o & 1), J = 2 * b.j + ((o >> 1) & 1);
+  const int I = 2 * b.i + px, J = 2 * b.j + py;
   if (part != 0 || !b.in || I >= nq || J >= nq) return;
   const long long k = (o >> 2) * nv + static_cast<long long>(J) * nq + I;
   const double xv = A.x != nullptr ? A.x[k] : 0.0;
   A.xo[k] = is_free(I, J, nq) ? fma(A.su, d, xv) : fma(A.omega, A.r[k], xv);
 }
 
-__device__ __forceinline__ void ring_pressure(const Args& A, int unit, int lane) {
+__device__ __forceinline__ void cell_pressure(const Args& A, const Band& b) {
   const LevelDev& L = A.L;
   const int n = L.n, nq = L.nq;
   const long long nv = L.nv;
-  const Band b = band_of(n, unit, 32, lane);
   const double* g = A.Gd + static_cast<size_t>(cell_type(n, b)) * RT_TYPE + 171 * 8;
   double a0 = 0.0, a1 = 0.0;
   for (int rJ = max(2, b.J0); rJ <= min(6, b.J1); ++rJ) {
@@ -242,9 +268,9 @@ __device__ __forceinline__ void ring(const Args& A, int slot, int slots, int lan
   const int n = A.L.n, wide = n > RING_PARTS_MAX_N;
   const int uv = ring_units(n, wide ? 4 : 1), up = ring_units(n, 32);
   for (int u = slot; u < uv + up; u += slots) {
-    if (u >= uv) ring_pressure(A, u - uv, lane);
-    else if (wide) ring_velocity<1>(A, u, lane);
-    else ring_velocity<4>(A, u, lane);
+    if (u >= uv) cell_pressure(A, band_of(n, u - uv, 32, lane));
+    else if (wide) cell_velocity<1>(A, band_of(n, u, 4, lane >> 3), lane);
+    else cell_velocity<4>(A, band_of(n, u, 1, 0), lane);
   }
 }
 
@@ -252,9 +278,43 @@ struct Shared {   // what the roles of a CTA share
   uint32_t full, done, free, tmem;
   volatile int* fail;
   volatile int* sexp;
+  const unsigned short* cexp;
+  const unsigned short* pexp;
   int i0, j0, rows, S;
 };
 
+// Outputs of a cell to which the contraction gives too little (bits: velocities, pressure):
+// the patches that hold it have no residual within 2^-8 of 2^E (pressure: 2^-10).  Every
+// velocity output lies in patches that hold the nodes of the 3 x 3 cells around and the
+// pressures of the vertices i, i + 1 and j, j + 1; the pressure's patch the nodes of the
+// cells i - 1, i and j - 1, j and its own pressure.  a: the cell's row in the step, col:
+// its held column.
+__device__ __forceinline__ unsigned too_small(const Shared& C, int s, int a, int col, int eb) {
+  auto cell = [&](int r, int c) -> int { return C.cexp[(((r >> 1) & 7) * 2 + (r & 1)) * WCOLS + c]; };
+  const int r = 2 * s + 2 + a;   // cell row of the walk, row r & 1 of pair r >> 1
+  int mp = cell(r, col);
+  if (mp >= eb - 7) return 0;
+  const unsigned short* p = C.pexp + (((s + 2) & 7) * 4 + 1 + a) * WCOLS + col;
+  mp = max(mp, static_cast<int>(p[0]));
+  if (mp >= eb - 7) return 0;
+  mp = max(max(mp, cell(r, col - 1)), max(cell(r - 1, col), cell(r - 1, col - 1)));
+  int mu = max(mp, max(max(cell(r + 1, col - 1), cell(r + 1, col)), max(cell(r + 1, col + 1), cell(r, col + 1))));
+  mu = max(max(mu, cell(r - 1, col + 1)), static_cast<int>(max(max(p[1], p[WCOLS]), p[WCOLS + 1])));
+  return (mu < eb - 7 ? 1u : 0u) | (mp < eb - 9 ? 2u : 0u);
+}
+// Whether its reach holds anything but zeros
+__device__ __forceinline__ bool any_residual(const Shared& C, int s, int a, int col) {
+  unsigned m = 0;
+#pragma unroll 1
+  for (int r = 2 * s + a; r <= 2 * s + a + 4; ++r)
+#pragma unroll 1
+    for (int c = col - 2; c <= col + 2; ++c) m |= C.cexp[(((r >> 1) & 7) * 2 + (r & 1)) * WCOLS + c];
+#pragma unroll 1
+  for (int k = 0; k < 3; ++k)
+#pragma unroll 1
+    for (int c = col - 1; c <= col + 1; ++c) m |= C.pexp[(((s + 2) & 7) * 4 + a + k) * WCOLS + c];
+  return m != 0;
+}
 // One chain's accumulators: T[o] += the digit sums (gi, c) with weight 2^(59 - 9 gi - 10 c),
 // in units of 2^16 (velocities) and 2^14 (pressure): the sums of |G| / 2^e_o are below 5
 // and 1.4, so |T| < 2^62.  Weights below the unit are rounded one by one (about a dozen).
@@ -306,14 +366,22 @@ __device__ __forceinline__ void epilogue(const Args& A, const Shared& C, int g, 
           chain(std::integral_constant<int, 4>{}) && chain(std::integral_constant<int, 5>{})))
       return;
     const int j = C.j0 + 2 * s + a;
-    if (i > n - 3 || 2 * s + a >= C.rows) continue;
+    const bool mine = i <= n - 3 && 2 * s + a < C.rows;
+    const int es = C.sexp[s & 3], eb = es & 0xffff;   // the sign: values were rounded
+    if (A.check.flags != nullptr) {
+      unsigned redo = 0;
+      if (mine && es < 0) redo = too_small(C, s, a, i - C.i0 + 2, eb);
+      if (redo != 0 && !any_residual(C, s, a, i - C.i0 + 2)) redo = 0;
+      if (mine) A.check.flags[static_cast<long long>(j) * np + i] = static_cast<unsigned char>(redo);
+      if (mine && redo != 0) *A.check.any = A.check.call;
+    }
+    if (!mine) continue;
     const long long ku = static_cast<long long>(2 * j) * nq + 2 * i;
     const long long kp = 2 * nv + static_cast<long long>(j) * np + i;
     auto at = [&](int o) { return o == 8 ? kp : (o >> 2) * nv + ku + ((o >> 1) & 1) * nq + (o & 1); };
     double xv[9];
 #pragma unroll
     for (int o = 0; o < 9; ++o) xv[o] = A.x != nullptr ? A.x[at(o)] : 0.0;
-    const int eb = C.sexp[s & 3];   // NaN where a residual of the window is not finite
     const double qu = A.qu * exp_scale(eb, UNIT_U - 75), qp = A.qp * exp_scale(eb, UNIT_P - 75);
 #pragma unroll
     for (int o = 0; o < 9; ++o) A.xo[at(o)] = fma(o == 8 ? qp : qu, to_double(T[o]), xv[o]);
@@ -332,8 +400,11 @@ __global__ void __launch_bounds__(NT, 1) k_vanka_tc64(const Args A) {
                  bar_g = bar_free + 8 * MMA_WARPS;
   uint32_t* tslot = reinterpret_cast<uint32_t*>(sm + SM::MISC);
   volatile int* fail = reinterpret_cast<volatile int*>(sm + SM::MISC + 4);
-  int* smax = reinterpret_cast<int*>(sm + SM::MISC + 8);                    // 8 slots
-  volatile int* sexp = reinterpret_cast<volatile int*>(sm + SM::MISC + 40);   // 4 slots
+  unsigned* smax = reinterpret_cast<unsigned*>(sm + SM::MISC + 8);                    // 8 slots
+  unsigned* smin = reinterpret_cast<unsigned*>(sm + SM::MISC + 40);                   // 8 slots
+  volatile int* sexp = reinterpret_cast<volatile int*>(sm + SM::MISC + 72);   // 4 slots
+  unsigned short* cexp = reinterpret_cast<unsigned short*>(sm + SM::CEXP);
+  unsigned short* pexp = reinterpret_cast<unsigned short*>(sm + SM::PEXP);
   if (static_cast<int>(blockIdx.x) >= A.ctas) {
     if (warp < RING_CTA_WARPS)
       ring(A, RING_WARPS * A.ctas + (blockIdx.x - A.ctas) * RING_CTA_WARPS + warp,
@@ -355,7 +426,10 @@ __global__ void __launch_bounds__(NT, 1) k_vanka_tc64(const Args A) {
     mbar_init(bar_g, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     *fail = 0;
-    for (int k = 0; k < 8; ++k) smax[k] = 0;
+    for (int k = 0; k < 8; ++k) {
+      smax[k] = 0u;
+      smin[k] = ~0u;
+    }
   }
   for (int k = tid; k < ROWB / 16; k += NT)   // channels 4..7 of the pressures stay zero
     reinterpret_cast<uint4*>(sm + SM::P)[k] = make_uint4(0u, 0u, 0u, 0u);
@@ -394,14 +468,35 @@ __global__ void __launch_bounds__(NT, 1) k_vanka_tc64(const Args A) {
       c.p[k] = (act && q >= 2 && gi <= n && pj <= n) ? A.r[2 * nv + static_cast<long long>(pj) * np + gi] : 0.0;
     }
   };
-  auto note_max = [&](int q, Cell& c) {   // pressures to their units; the pair's largest exponent
+  // pressures to their units; the pair's largest value (high word); with a check also the
+  // smallest nonzero one, and the exponents of the cell and its pressures
+  auto note = [&](int q, int a, int col, bool act, Cell& c) {
     c.p[0] *= A.rps;
     c.p[1] *= A.rps;
-    int m = max(__double2hiint(c.p[0]) & 0x7fffffff, __double2hiint(c.p[1]) & 0x7fffffff);
+    auto high = [](double x) { return static_cast<unsigned>(__double2hiint(x)) & 0x7fffffffu; };
+    unsigned m = 0u;
 #pragma unroll
-    for (int o = 0; o < 8; ++o) m = max(m, __double2hiint(c.v[o]) & 0x7fffffff);
-    m = __reduce_max_sync(0xffffffffu, m);
-    if (lane == 0) atomicMax(smax + (q & 7), m);
+    for (int o = 0; o < 8; ++o) m = max(m, high(c.v[o]));
+    const unsigned all = __reduce_max_sync(0xffffffffu, max(m, max(high(c.p[0]), high(c.p[1]))));
+    if (lane == 0) atomicMax(smax + (q & 7), all);
+    if (A.check.flags != nullptr) {
+      auto mag = [&](double x) { return high(x) | min(static_cast<unsigned>(__double2loint(x)), 1u); };   // zero for zeros only
+      auto ex = [](unsigned w) { return static_cast<unsigned short>(max(w >> 20, min(w, 1u))); };
+      const unsigned p0 = mag(c.p[0]), p1 = mag(c.p[1]);
+      unsigned l = min(p0 - 1u, p1 - 1u), v = 0u;
+#pragma unroll
+      for (int o = 0; o < 8; ++o) {
+        v = max(v, mag(c.v[o]));
+        l = min(l, mag(c.v[o]) - 1u);
+      }
+      if (act) {
+        cexp[((q & 7) * 2 + a) * WCOLS + col] = ex(v);
+        pexp[((q & 7) * 4 + 2 * a) * WCOLS + col] = ex(p0);
+        pexp[((q & 7) * 4 + 2 * a + 1) * WCOLS + col] = ex(p1);
+      }
+      l = __reduce_min_sync(0xffffffffu, l);
+      if (lane == 0) atomicMin(smin + (q & 7), l);
+    }
   };
   auto words = [&](const Cell& c, int eb, unsigned long long (&w)[8]) {
 #pragma unroll
@@ -419,8 +514,14 @@ __global__ void __launch_bounds__(NT, 1) k_vanka_tc64(const Args A) {
     *reinterpret_cast<unsigned*>(sm + SM::P + j * PLANE + col * 16 + 4 * a) = digit2(w[0], w[1], j);
   };
   auto largest = [&](int q) {   // |x| < 2^(e - 1022) over the pairs q - 2 .. q
-    const volatile int* vm = smax;
-    return max(vm[q & 7], max(vm[(q - 1) & 7], vm[(q - 2) & 7])) >> 20;
+    const volatile unsigned* vm = smax;
+    return static_cast<int>(max(vm[q & 7], max(vm[(q - 1) & 7], vm[(q - 2) & 7])) >> 20);
+  };
+  auto step_exp = [&](int q, int eb) {   // with the sign if a value of the pairs q - 2 .. q has bits below 2^(E - 58)
+    if (A.check.flags == nullptr) return eb;
+    const volatile unsigned* vm = smin;
+    const unsigned l = min(vm[q & 7], min(vm[(q - 1) & 7], vm[(q - 2) & 7]));
+    return eb | (l < (static_cast<unsigned>(eb - 5) << 20) - 1u ? static_cast<int>(0x80000000u) : 0);
   };
 
   // the first window (row pairs 0, 1, 2) by 27 warps at once
@@ -432,11 +533,11 @@ __global__ void __launch_bounds__(NT, 1) k_vanka_tc64(const Args A) {
     Cell c;
     if (q < 3) {
       load(q, a, col, act, c);
-      note_max(q, c);
+      note(q, a, col, act, c);
     }
     __syncthreads();
     const int em = largest(2);
-    eb = min(max(em + 1, EB_MIN), 0x7ff);
+    eb = exp_for(em);
     if (act) {
       unsigned long long w[8], wp[2];
       words(c, eb, w);
@@ -447,12 +548,12 @@ __global__ void __launch_bounds__(NT, 1) k_vanka_tc64(const Args A) {
         if (q == 2) put_p(a, col, j, wp);
       }
     }
-    if (tid == 0) sexp[0] = em < 0x7ff ? eb : 0x7ff;
+    if (tid == 0) sexp[0] = step_exp(2, eb);
     fence_proxy();
     __syncthreads();
   }
 
-  const Shared C{bar_full, bar_done, bar_free, tmem, fail, sexp, i0, j0, rows, S};
+  const Shared C{bar_full, bar_done, bar_free, tmem, fail, sexp, cexp, pexp, i0, j0, rows, S};
   if (warp < EPI_WARPS) {
     epilogue(A, C, warp / EPI_GROUP, warp, lane);
   } else if (warp < EPI_WARPS + SLICE_WARPS) {
@@ -463,14 +564,17 @@ __global__ void __launch_bounds__(NT, 1) k_vanka_tc64(const Args A) {
     Cell cur;
     if (S > 1) load(3, a, col, act, cur);
     for (int q = 3; q < S + 2; ++q) {
-      note_max(q, cur);
+      note(q, a, col, act, cur);
       asm volatile("bar.sync 1, %0;" ::"n"(SLICE_T) : "memory");
-      if (t == 0) smax[(q + 3) & 7] = 0;
+      if (t == 0) {
+        smax[(q + 3) & 7] = 0u;
+        smin[(q + 3) & 7] = ~0u;
+      }
       const int em = largest(q), s = q - 2;
       unsigned long long w[8], wp[2];
-      const bool renew = em > eb || (eb - em > 3 && eb > EB_MIN);
+      const bool renew = !exp_fits(em, eb);
       if (renew) {   // uniform over the slicer warps: the window again, once the step before has read it
-        eb = min(max(em + 1, EB_MIN), 0x7ff);
+        eb = exp_for(em);
         for (int j = 0; j < ND; ++j)
           mbar_wait_or_fail(bar_done + 8 * (ND * ((s - 1) & 1) + j), ((s - 1) >> 1) & 1, A.wait_limit, fail);
         for (int qq = q - 2; qq < q; ++qq) {
@@ -483,7 +587,7 @@ __global__ void __launch_bounds__(NT, 1) k_vanka_tc64(const Args A) {
           }
         }
       }
-      if (t == 0) sexp[s & 3] = em < 0x7ff ? eb : 0x7ff;
+      if (t == 0) sexp[s & 3] = step_exp(q, eb);
       words(cur, eb, w);
       words_p(cur, eb, wp);
       if (q + 1 < S + 2) load(q + 1, a, col, act, cur);   // in flight while the planes are written
@@ -563,6 +667,55 @@ __global__ void __launch_bounds__(NT, 1) k_vanka_tc64(const Args A) {
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
 }
 
+// The pressure of one interior cell by a warp
+__device__ __forceinline__ void warp_pressure(const Args& A, int i, int j, int lane) {
+  const LevelDev& L = A.L;
+  const double* g = A.Gd + static_cast<size_t>(3 * VS_POS + 3) * RT_TYPE + 171 * 8;
+  const long long kp = 2 * L.nv + static_cast<long long>(j) * L.np + i;
+  double d = 0.0;
+  if (lane < 25) {   // all nodes are free
+    const double* r = A.r + static_cast<long long>(2 * j - 2 + lane / 5) * L.nq + 2 * i - 2 + lane % 5;
+    d = fma(__ldg(g + 2 * lane + 1), __ldg(r + L.nv), __ldg(g + 2 * lane) * __ldg(r));
+  } else if (lane == 25) {
+    d = A.rps * __ldg(g + 50) * __ldg(A.r + kp);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+  if (lane == 0) A.xo[kp] = fma(A.sp, d, A.x != nullptr ? A.x[kp] : 0.0);
+}
+// The outputs that the contraction leaves to FP64: a warp looks at 32 cells of a row and
+// computes the flagged ones one at a time (many pressures by a lane each).  A cell costs
+// about fifty times what it costs in the contraction, so they are spread over the whole GPU
+// here, not done where they are found: residuals that are large along a wall flag all cells
+// of the strips there.
+__global__ void __launch_bounds__(128) k_vanka_fp64_cells(const Args A) {
+  pdl_begin();
+  if (*A.check.any != A.check.call) return;
+  const int n = A.L.n, lane = threadIdx.x & 31, w = n - 5, per = (w + 31) / 32;
+  Band b;
+  b.I0 = b.J0 = 0;
+  b.I1 = b.J1 = 8;
+  for (int u = blockIdx.x * 4 + (threadIdx.x >> 5); u < w * per; u += gridDim.x * 4) {
+    // columns shifted by a row each, or a warp would stay in the same ones
+    const int i = 3 + 32 * ((u + u / per) % per) + lane, j = 3 + u / per;
+    const unsigned redo = i <= n - 3 ? A.check.flags[static_cast<long long>(j) * A.L.np + i] : 0u;
+    const unsigned vel = __ballot_sync(0xffffffffu, redo & 1u), pres = __ballot_sync(0xffffffffu, redo & 2u);
+    b.j = j;
+    b.in = true;
+    for (unsigned m = vel; m != 0; m &= m - 1) {
+      b.i = __shfl_sync(0xffffffffu, i, __ffs(m) - 1);
+      cell_velocity<4>(A, b, lane);
+    }
+    if (__popc(pres) > 6) {
+      b.i = i;
+      if (redo & 2u) cell_pressure(A, b);
+      __syncwarp();
+    } else {
+      for (unsigned m = pres; m != 0; m &= m - 1) warp_pressure(A, __shfl_sync(0xffffffffu, i, __ffs(m) - 1), j, lane);
+    }
+  }
+}
+
 }  // namespace
 
 // Digits of the interior cell type in the K order of the kernel's MMAs.  Row 18 i + 9 a
@@ -620,7 +773,7 @@ cudaError_t vanka_tc64_prepare() {
 
 void launch_vanka_tc64(const LevelDev& L, const unsigned char* Gp, int eu, int ep, const double* Gd, const double* x,
                        const double* b, double* xo, double omega, double* rscratch, int* err, int wait_limit,
-                       cudaStream_t s) {
+                       const TC64Check& check, cudaStream_t s) {
   const double* r = b;
   if (x != nullptr) {
     launch_apply<double>(L, x, b, rscratch, 1, s);
@@ -634,10 +787,14 @@ void launch_vanka_tc64(const LevelDev& L, const unsigned char* Gp, int eu, int e
   // SMs left over compute cells near the boundary
   const int ctas = strips * ((steps + seg - 1) / seg), extra = ctas < sms ? sms - ctas : 0;
   Args A{L, Gp, Gd, x, r, xo, omega / L.cl, omega / L.cb, std::ldexp(omega / L.cl, eu), std::ldexp(omega / L.cb, ep),
-         L.cl / L.cb, omega, strips, ctas, seg, err, wait_limit};
+         L.cl / L.cb, omega, strips, ctas, seg, err, wait_limit, check};
   count_launches(1);
   g_tc_launches.fetch_add(1, std::memory_order_relaxed);
   launch_pdl(k_vanka_tc64, dim3(ctas + extra), dim3(NT), SM::BYTES, s, A);
+  if (check.flags != nullptr) {
+    count_launches(1);
+    launch_pdl(k_vanka_fp64_cells, dim3(4 * sms), dim3(128), 0, s, A);
+  }
 }
 
 }  // namespace sv

@@ -90,3 +90,39 @@ def test_exponents_of_cells_are_read_before_their_slot_is_written_again(slots):
     assert (loose == []) == (slots >= 6)
     src = open(os.path.join(CSRC, "sv_apply_tc64.cu")).read()
     assert "cexp[((q & 7) * 2 + a) * WCOLS + col] =" in src and "pexp[((q & 7) * 4 + 2 * a) * WCOLS + col] =" in src
+
+
+@pytest.mark.parametrize("slots", [5, 8])
+def test_sweep_reads_the_exponents_of_cells_before_their_slot_is_written_again(slots):
+    """The sweep: six chains a step, chains c and c + 3 take turns in an accumulator, the
+    epilogue reads the pairs s .. s + 2 after the last of them.  Pair q is written at the
+    begin of step q - 2, each step waiting for all chains of the step before it."""
+    after = {}
+
+    def edge(a, b):
+        after.setdefault(a, []).append(b)
+
+    for s in range(STEPS):
+        for c in range(6):
+            edge(("done", s, c), ("free", s, c))
+            edge(("free", s, c), ("free", s, c + 1) if c < 5 else ("read", s))
+            use_next = ("mma", s, c + 3) if c < 3 else ("mma", s + 1, c - 3)
+            edge(("free", s, c), use_next)
+            edge(("mma", s, c), ("done", s, c))
+            edge(("done", s, c), ("waited", s + 1))
+        edge(("read", s), ("free", s + 2, 0))          # the group's next step
+        edge(("waited", s), ("write", s + 3))
+    loose = []
+    for q in range(2, STEPS - slots - 2):
+        for s in (q - 2, q - 1, q):                    # the steps that use pair q
+            seen, todo = set(), [("read", s)]
+            while todo:
+                for b in after.get(todo.pop(), ()):
+                    if b not in seen:
+                        seen.add(b)
+                        todo.append(b)
+            if ("write", q + slots) not in seen:
+                loose.append((q, s))
+    assert (loose == []) == (slots == 8)
+    src = open(os.path.join(CSRC, "sv_vanka_tc64.cu")).read()
+    assert "cexp[((q & 7) * 2 + a) * WCOLS + col] =" in src and "pexp[((q & 7) * 4 + 2 * a) * WCOLS + col] =" in src
