@@ -50,7 +50,8 @@
 // The exponent E is shared by the cells in reach of a step.  It follows the residual:
 // when the largest of the window leaves [2^(E-4), 2^E), the digits of the window are
 // rewritten with a new E.  A residual that is not finite makes the cells of the step
-// NaN.  Every wait is bounded; on expiry the kernel sets *err and returns.
+// NaN, in a single sweep only the dofs of the patches that hold it.  Every wait is
+// bounded; on expiry the kernel sets *err and returns.
 //
 // Bound: the tensor pipe and its operand reads.  An MMA of M = 128 takes N / 2 clocks
 // from N = 128 on and about 38 + 0.22 N below, so the chains of a step take 25 clocks per
@@ -191,13 +192,13 @@ __device__ __forceinline__ void cell_velocity(const Args& A, const Band& b, int 
   const int n = L.n, nq = L.nq, np = L.np, o = lane & 7, part = PARTS == 4 ? lane >> 3 : 0;
   const long long nv = L.nv;
   const double* g = A.Gd + static_cast<size_t>(cell_type(n, b)) * RT_TYPE + o;
-  const int px = o & 1, py = (o >> 1) & 1;
+  const int px = o & 1, py = (o >> 1) & 1;   // the patches with an odd node lie to its right: from 2 px, 2 py on
   double a0 = 0.0, a1 = 0.0;
   auto node = [&](int rJ, int rI) {
     const int J = 2 * b.j - 4 + rJ;
     const double* rr = A.r + static_cast<long long>(J) * nq + 2 * b.i - 4 + rI;
     const double* gr = g + (rJ * 9 + rI) * 16;
-    const bool ok = b.in && is_free(2 * b.i - 4 + rI, J, nq);
+    const bool ok = b.in && rI >= 2 * px && rJ >= 2 * py && is_free(2 * b.i - 4 + rI, J, nq);
     const double r0 = ok ? __ldg(rr) : 0.0, r1 = ok ? __ldg(rr + nv) : 0.0;
     a0 = fma(__ldg(gr), r0, a0);
     a1 = fma(__ldg(gr + 8), r1, a1);
@@ -223,7 +224,7 @@ __device__ __forceinline__ void cell_velocity(const Args& A, const Band& b, int 
 #pragma unroll
   for (int k = part; k < 9; k += PARTS) {
     const int pi = b.i + k % 3 - 1, pj = b.j + k / 3 - 1;
-    const bool ok = b.in && pi >= 0 && pj >= 0 && pi <= n && pj <= n;
+    const bool ok = b.in && k % 3 >= px && k / 3 >= py && pi >= 0 && pj >= 0 && pi <= n && pj <= n;
     const double r0 = ok ? __ldg(A.r + 2 * nv + static_cast<long long>(pj) * np + pi) : 0.0;
     ap = fma(__ldg(g + 162 * 8 + k * 8), r0, ap);
   }
@@ -372,6 +373,7 @@ __device__ __forceinline__ void epilogue(const Args& A, const Shared& C, int g, 
       unsigned redo = 0;
       if (mine && es < 0) redo = too_small(C, s, a, i - C.i0 + 2, eb);
       if (redo != 0 && !any_residual(C, s, a, i - C.i0 + 2)) redo = 0;
+      if (eb == 0x7ff) redo = 3;                      // values that are not finite
       if (mine) A.check.flags[static_cast<long long>(j) * np + i] = static_cast<unsigned char>(redo);
       if (mine && redo != 0) *A.check.any = A.check.call;
     }

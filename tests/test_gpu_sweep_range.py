@@ -7,6 +7,7 @@ import numpy as np
 import pytest
 import torch
 
+import stokes_inputs as si
 from oracle import rounding as RB
 from oracle import stokes_oracle as O
 
@@ -60,4 +61,29 @@ def test_sweep_keeps_every_entry(form):
     bound = RB.sweep_error_bound(lv, None, b * scale, 0.7) * 2.0 ** -29
     got = H.sweep(None, torch.from_numpy(b).cuda()).cpu().numpy() * scale
     assert (np.abs(got - want) <= bound).all(), (np.abs(got - want) / np.maximum(bound, 1e-300)).max()
+    H.close()
+
+
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+@pytest.mark.parametrize("where", ["u", "p", "near the wall"])
+def test_sweep_spreads_nonfinite_values_as_the_patches_do(where, bad):
+    """Exactly the dofs of the patches that hold the bad residual are not finite; the others
+    are what they are without it."""
+    import paper_2401_06277_gb300 as pkg
+    n, nq, lv = N, 2 * N + 1, level()
+    H = pkg.Hierarchy(N, coarse_n=5, restart=1)
+    b = si.random_vector(n, 9)
+    k = {"u": 101 * nq + 101, "p": 2 * nq * nq + 50 * (n + 1) + 61, "near the wall": nq * nq + 101 * nq + 3}[where]
+    clean = H.sweep(None, torch.from_numpy(b).cuda()).cpu().numpy()
+    b[k] = bad
+    out = H.sweep(None, torch.from_numpy(b).cuda()).cpu().numpy()
+    hit = np.zeros(len(b), dtype=bool)
+    for dofs in lv.patch_dofs[(lv.patch_dofs == k).any(axis=1)]:
+        hit[dofs[dofs >= 0]] = True
+    free = np.zeros((nq, nq), dtype=bool)
+    free[1:-1, 1:-1] = True
+    hit &= np.concatenate([free.ravel(), free.ravel(), np.ones((n + 1) ** 2, dtype=bool)])   # Dirichlet rows are identities
+    assert not np.isfinite(out[hit]).any()
+    assert np.isfinite(out[~hit]).all()
+    assert np.abs(out - clean)[~hit].max() <= 1e-13 * np.abs(clean).max()
     H.close()
