@@ -750,20 +750,14 @@ stokes_status fgmres(stokes_hierarchy* h, const double* b, double* x, int* iters
   return STOKES_OK;
 }
 
-// Tile shape of the sweep per level and precision: fixed by params.tile, or
-// (tile = -1) the fastest of the shapes on that level, timed with CUDA events
-// on the hierarchy's stream.  Every level with sweeps is tuned: on the small
-// ones the 4 x 4 tile spreads the FP64 patch solves over more SMs.
-template <typename R>
+// Tile shape of the FP32 sweep of a level of the mixed forms (tile = -1): the fastest of
+// the shapes there, timed with CUDA events on the hierarchy's stream.
 cudaError_t tune_level(stokes_hierarchy* h, sv::Level& L, int* cfg) {
   cudaStream_t s = h->stream;
-  R* x = Buf<R>::x0(L);
-  R* b = Buf<R>::b(L);
-  R* xo = Buf<R>::x1(L);
-  const R* cd = nullptr;
+  float *x = L.xf0, *b = L.bf, *xo = L.xf1;
   cudaError_t e;
-  if ((e = cudaMemsetAsync(x, 0, L.d.N * sizeof(R), s)) != cudaSuccess) return e;
-  if ((e = cudaMemsetAsync(b, 0, L.d.N * sizeof(R), s)) != cudaSuccess) return e;
+  if ((e = cudaMemsetAsync(x, 0, L.d.N * sizeof(float), s)) != cudaSuccess) return e;
+  if ((e = cudaMemsetAsync(b, 0, L.d.N * sizeof(float), s)) != cudaSuccess) return e;
   cudaEvent_t e0, e1;
   if ((e = cudaEventCreate(&e0)) != cudaSuccess) return e;
   if ((e = cudaEventCreate(&e1)) != cudaSuccess) {
@@ -771,31 +765,22 @@ cudaError_t tune_level(stokes_hierarchy* h, sv::Level& L, int* cfg) {
     return e;
   }
   float best = 1e30f;
-  // candidates: the fused tile shapes; in FP64 also the split sweep; in the mixed
-  // forms, on levels with interior strips, also the strip sweep with its ring
-  const bool tc = (sizeof(R) == 4) && L.strip;
-  constexpr int CAND_TC = sv::VANKA_CFG_4 + 1;   // the strip sweep (mixed forms), tuning index only
+  // candidates: the fused tile shapes, the split sweep and, on levels with interior
+  // strips, the strip sweep with its ring
+  const bool tc = L.strip;
+  constexpr int CAND_TC = sv::VANKA_CFG_4 + 1;   // the strip sweep, tuning index only
   const int ncand = tc ? CAND_TC + 1 : sv::VANKA_CFG_4 + 1;
   int best_c = 0;
   for (int c = 0; c < ncand; ++c) {
     if (tc && c == sv::VANKA_CFG_14) continue;   // where the strip tiles fit, 14x14 means the strip sweep
     auto run = [&]() {
-      if constexpr (sizeof(R) == 8) {
-        if (sv::vanka_cfg_split(c))
-          sv::launch_vanka_split<double>(L.d, L.cd, h->fd, x, b, xo, h->prm.omega, h->delta,
-                                         c == sv::VANKA_CFG_SPLIT2, s, L.r);
-        else
-          sv::launch_vanka<double>(L.d, L.cd, h->fd, x, b, xo, h->prm.omega, c, s);
-      } else {
-        if (c == CAND_TC) {
-          tc_sweep(h, L, x, b, xo, s);
-        } else if (sv::vanka_cfg_split(c)) {
-          sv::launch_vanka_split<float>(L.d, L.cdf, h->fdf, x, b, xo, h->prm.omega, h->deltaf,
-                                        c == sv::VANKA_CFG_SPLIT2, s, nullptr);
-        } else {
-          sv::launch_vanka<float>(L.d, L.cdf, h->fdf, x, b, xo, h->prm.omega, c, s);
-        }
-      }
+      if (c == CAND_TC)
+        tc_sweep(h, L, x, b, xo, s);
+      else if (sv::vanka_cfg_split(c))
+        sv::launch_vanka_split<float>(L.d, L.cdf, h->fdf, x, b, xo, h->prm.omega, h->deltaf, c == sv::VANKA_CFG_SPLIT2,
+                                      s, nullptr);
+      else
+        sv::launch_vanka<float>(L.d, L.cdf, h->fdf, x, b, xo, h->prm.omega, c, s);
     };
     // one untimed run, then the best of three timed trials: a trial is a few sweeps
     // on large levels and more on small ones, where one sweep lasts microseconds and
@@ -824,7 +809,6 @@ cudaError_t tune_level(stokes_hierarchy* h, sv::Level& L, int* cfg) {
   } else {
     *cfg = best_c;
   }
-  (void)cd;
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (e != cudaSuccess) return e;
@@ -855,14 +839,14 @@ cudaError_t choose_tiles(stokes_hierarchy* h) {
     L.vk_cfg = L.vk_cfg_f = (L.d.n < 64) ? 0 : 1;
     if (&L == &h->lv.front()) continue;   // the coarsest level is solved exactly: no sweeps
     if (static_cast<int>(&L - &h->lv.front()) <= h->tail_top) continue;   // swept by the persistent launch
-    // only the precision the V-cycle runs in is tuned (the FP64 sweep of a
-    // mixed hierarchy serves stokes_vanka_sweep alone and keeps 16x8)
+    // a level with sweeps has n >= 8 (coarse_n >= 4): the stencil's positions do not overlap.
+    // The FP64 sweep of a mixed hierarchy serves stokes_vanka_sweep alone and keeps its tile.
+    static_assert(sv::VS_MIN_N <= 8, "smallest level with sweeps");
     cudaError_t e = cudaSuccess;
-    if (h->prm.prec == STOKES_FP64 && L.d.n >= sv::VS_MIN_N)
+    if (h->prm.prec == STOKES_FP64)
       L.vk_cfg = (h->stencil_digits && L.d.n >= TC64_MIN_N) ? sv::VANKA_CFG_TC64 : sv::VANKA_CFG_STENCIL;
-    else if (h->prm.prec == STOKES_FP64) e = tune_level<double>(h, L, &L.vk_cfg);
-    else if (h->stencil_Gf && L.d.n >= sv::VS_MIN_N && L.d.n <= STENCIL_F32_MAX_N) L.vk_cfg_f = sv::VANKA_CFG_STENCIL;
-    else e = tune_level<float>(h, L, &L.vk_cfg_f);   // strip sweep vs SIMT shapes
+    else if (h->stencil_Gf && L.d.n <= STENCIL_F32_MAX_N) L.vk_cfg_f = sv::VANKA_CFG_STENCIL;
+    else e = tune_level(h, L, &L.vk_cfg_f);   // strip sweep vs SIMT shapes
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

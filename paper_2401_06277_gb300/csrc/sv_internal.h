@@ -349,10 +349,10 @@ void launch_rhs_transpose(const LevelDev& L, const double* lam, double* g, cudaS
 // in [skip_lo, skip_hi] are left to the tensor-core kernel (empty by default).
 constexpr int VANKA_NCFG = 4;
 constexpr int VANKA_CFG_14 = 3;
-constexpr int VANKA_CFG_SPLIT = 4;   // FP64 only: own-patch solves + separate update (launch_vanka_split)
+constexpr int VANKA_CFG_SPLIT = 4;   // own-patch solves + separate update (launch_vanka_split)
 constexpr int VANKA_CFG_SPLIT2 = 5;  // the same, compiled for two CTAs per SM (at most 128 registers)
 constexpr int VANKA_CFG_4 = 6;       // fused 4x4 tiles: small levels, spread over more SMs
-constexpr int VANKA_CFG_STENCIL = 7; // FP64 only: the residual, then the composite stencil (launch_vanka_stencil)
+constexpr int VANKA_CFG_STENCIL = 7; // the residual, then the composite stencil (launch_vanka_stencil)
 constexpr int VANKA_CFG_TC64 = 8;    // FP64 only: the composite stencil on the tensor cores (launch_vanka_tc64)
 inline bool vanka_cfg_split(int cfg) { return cfg == VANKA_CFG_SPLIT || cfg == VANKA_CFG_SPLIT2; }
 template <typename R>

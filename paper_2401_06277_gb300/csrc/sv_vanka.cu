@@ -20,9 +20,10 @@
 //
 // In FP64 the kernel is bound by the FP64 pipe on GB300 (2 DFMA / clk / SM).
 // The tile shape trades halo recomputation against shared memory per CTA and
-// is chosen per level by a timing autotuner at hierarchy creation (mixed forms; in
-// FP64 the default is the composite stencil, sv_vanka_stencil.cu and sv_vanka_tc64.cu,
-// and these kernels serve grids too small for it and the configurations asked for).
+// is chosen per level by a timing autotuner at hierarchy creation (mixed forms above 64^2;
+// in FP64, and in the mixed forms up to there, the default is the composite stencil,
+// sv_vanka_stencil.cu and sv_vanka_tc64.cu, and the FP64 kernels here serve the
+// configurations asked for, the coarsest level and the FP64 sweep of a mixed hierarchy).
 //
 // Issue-slot economies: window rows load one warp per row with compile-time
 // extents; on tiles whose owned vertices lie in 1..n-1 the update sums each
