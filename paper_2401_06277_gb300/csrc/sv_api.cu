@@ -1004,8 +1004,10 @@ stokes_status stokes_hierarchy_create(int n, double viscosity, const stokes_para
         e = cudaGetLastError();
       }
     }
-    // patch corrections of the per-patch-inverse and the split sweeps (finest-level size)
-    if (e == cudaSuccess && prm.prec == STOKES_FP64 && k + 1 == sizes.size())
+    // patch corrections of the per-patch-inverse and the split sweeps (finest-level size);
+    // in FP64 only where one of them was asked for, 1.7 GB at 2048^2
+    if (e == cudaSuccess && prm.prec == STOKES_FP64 && k + 1 == sizes.size() &&
+        (prm.smoother == STOKES_SMOOTHER_PER_PATCH || sv::vanka_cfg_split(prm.tile)))
       e = dalloc(&h->delta, std::max(sv::patch_delta_doubles(L.d), sv::split_delta_doubles(L.d)));
     if (e == cudaSuccess && prm.prec != STOKES_FP64 && k + 1 == sizes.size())
       e = dalloc(&h->deltaf, std::max(sv::patch_delta_doubles(L.d), sv::split_delta_doubles(L.d)));
