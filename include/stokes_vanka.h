@@ -335,7 +335,7 @@ stokes_status stokes_stats_read(stokes_hierarchy* h, stokes_stats* out);
  * stream and returns STOKES_ERR_TIMEOUT if a bounded device wait expired in
  * work queued since the last report, else STOKES_OK.  Waits are bounded in the
  * tensor-core sweeps (the BF16 form's; the FP64 form's from n = 56 on), in the
- * FP64 operator of every form from n = 160 on (stokes_apply_operator,
+ * FP64 operator of every form from n = 192 on (stokes_apply_operator,
  * stokes_residual, the residual inside a sweep, cycle or solve) and at the grid
  * barriers of the persistent coarse-level launch.  After an expired wait the
  * output of that call is void: any part of it may have been written.  The flag

@@ -820,9 +820,10 @@ cudaError_t tune_level(stokes_hierarchy* h, sv::Level& L, int* cfg) {
 // n = 64 its 1125 multiply-adds per vertex exceed those of the tiled patch solves.
 constexpr int STENCIL_F32_MAX_N = 64;
 // Levels whose FP64 operator is the tensor-core contraction (smaller ones: FP64, one
-// output per thread): 8.4 us at n = 128 in FP64, 11.4 us at n = 256 by the contraction
-// (57 us in FP64 before it).
-constexpr int OP_TC64_MIN_N = 160;
+// output per thread).  FP64 / contraction (us): n = 160 12.1 / 14.6, 176 13.8 / 14.6,
+// 192 16.6 / 14.0, 256 26.7 / 14.4: the contraction takes two to three steps per CTA there
+// whatever the size.
+constexpr int OP_TC64_MIN_N = 192;
 // The FP64 sweep by size: the composite stencil as FP64 dot products below TC64_MIN_N, as
 // the tensor-core contraction from there on.  One zero-guess sweep, FP64 dot products /
 // tensor cores (us): n = 48 10.9 / 13.0, 56 14.3 / 12.9, 64 17.6 / 12.9, 128 52.4 / 13.9.

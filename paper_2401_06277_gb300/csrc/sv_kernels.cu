@@ -383,19 +383,17 @@ dim3 grid2(int nx, int ny, dim3 blk) {
 
 template <typename T>
 void launch_apply(const LevelDev& L, const T* x, const T* b, T* y, int residual, cudaStream_t s) {
-  if constexpr (sizeof(T) == 8) {
-    if (L.op_digits != nullptr) {
-      launch_apply_tc64(L, x, residual ? b : nullptr, y, s);
-      return;
-    }
-  }
-  count_launches(1);
-  if (L.np <= OUT_MAX_NP) {
+  const bool tc64 = sizeof(T) == 8 && L.op_digits != nullptr;
+  if (!tc64) count_launches(1);
+  if constexpr (sizeof(T) == 8) {   // FP64: up to the size from which on the contraction is faster (OP_TC64_MIN_N)
+    if (tc64) launch_apply_tc64(L, x, residual ? b : nullptr, y, s);
+    else launch_pdl(k_apply_out<T>, out_grid(L.np, 9), dim3(32), 0, s, L, x, b, y, residual);
+  } else if (L.np <= OUT_MAX_NP) {
     launch_pdl(k_apply_out<T>, out_grid(L.np, 9), dim3(32), 0, s, L, x, b, y, residual);
-    return;
+  } else {
+    dim3 blk(32, 8);
+    launch_pdl(k_apply<T>, dim3(grid2(L.np, L.np, blk)), dim3(blk), 0, s, L, x, b, y, residual);
   }
-  dim3 blk(32, 8);
-  launch_pdl(k_apply<T>, dim3(grid2(L.np, L.np, blk)), dim3(blk), 0, s, L, x, b, y, residual);
 }
 
 void launch_rhs(const LevelDev& L, const double* f, const double* ud, double* b, cudaStream_t s) {

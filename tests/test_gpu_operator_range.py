@@ -1,4 +1,4 @@
-"""The tensor-core FP64 operator (n >= 160) entry by entry, for data whose size changes
+"""The tensor-core FP64 operator (n >= 192) entry by entry, for data whose size changes
 within a strip of 128 cells or differs between the components.
 
 Bar: 66 u sum |a| |x| per row (u = 2^-53), plus 4 u |b|.  31 u is the a-priori bound of
@@ -106,8 +106,8 @@ FORMS = ["plain", "columns up", "columns down", "rows up", "rows down", "spikes"
 @pytest.mark.parametrize("form", FORMS)
 def test_operator_keeps_every_entry(form, nu):
     import paper_2401_06277_gb300 as pkg
-    n = 160
-    H = pkg.Hierarchy(n, viscosity=nu, coarse_n=5, restart=1)
+    n = 192
+    H = pkg.Hierarchy(n, viscosity=nu, coarse_n=6, restart=1)
     rng = np.random.default_rng(FORMS.index(form))
     x = field(n, form, rng)
     want, size = apply_ref(n, nu, x)
@@ -124,4 +124,15 @@ def test_operator_keeps_every_entry(form, nu):
     from paper_2401_06277_gb300 import stokes
     stokes.stokes_residual(H.handle, H.levels - 1, bd, xd, bd)
     assert np.array_equal(bd.cpu().numpy(), got)
+    H.close()
+
+
+@pytest.mark.parametrize("n,coarse_n", [(128, 4), (144, 9), (160, 5), (176, 11), (192, 6), (208, 13), (224, 7)])
+def test_operator_on_both_sides_of_the_size_rule(n, coarse_n):
+    import paper_2401_06277_gb300 as pkg
+    H = pkg.Hierarchy(n, coarse_n=coarse_n, restart=1)
+    x = field(n, "plain", np.random.default_rng(n))
+    want, size = apply_ref(n, 1.0, x)
+    got = H.apply(torch.from_numpy(x).cuda()).cpu().numpy()
+    assert (np.abs(got - want) <= 66.0 * U * size).all()
     H.close()

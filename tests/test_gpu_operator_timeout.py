@@ -1,4 +1,4 @@
-"""An expired wait of the tensor-core FP64 operator (n >= 160) is reported, by the direct
+"""An expired wait of the tensor-core FP64 operator (n >= 192) is reported, by the direct
 calls and by a mixed-precision hierarchy, and the next call is right again."""
 import numpy as np
 import pytest
@@ -15,8 +15,8 @@ pytestmark = pytest.mark.gpu
 def test_expired_operator_wait_is_reported_and_recovered(prec, call):
     import paper_2401_06277_gb300 as pkg
     from paper_2401_06277_gb300 import stokes
-    n = 160
-    H = pkg.Hierarchy(n, coarse_n=5, prec=getattr(stokes, prec), restart=1)
+    n = 192
+    H = pkg.Hierarchy(n, coarse_n=6, prec=getattr(stokes, prec), restart=1)
     x, b = si.random_vector(n, 1), si.random_vector(n, 2)
     xd, bd = torch.from_numpy(x).cuda(), torch.from_numpy(b).cuda()
     run = (lambda: H.apply(xd)) if call == "apply" else (lambda: H.residual(bd, xd))
