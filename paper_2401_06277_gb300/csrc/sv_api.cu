@@ -490,7 +490,7 @@ void bt_vcycle(stokes_hierarchy* h, int blk, int l, const double* b, double* out
   const double om = (blk == 0) ? h->prm.bt_omega_u : h->prm.bt_omega_p;
   auto resid = [&](const double* x, double* r) {
     if (blk == 0)
-      sv::launch_apply<double>(L.d, x, b, r, 1, s);
+      sv::launch_apply<double>(cycle_level(L), x, b, r, 1, s);
     else
       sv::launch_mass_resid(L.d, x, b, r, s);
   };
@@ -538,12 +538,12 @@ void bt_precondition(stokes_hierarchy* h, const double* r, double* z) {
     sv::launch_add(z, F.e, N, s);
   }
   // 2. L du = r_u - B^T dp: rhs = r - A (0, dp) on the velocity rows
-  sv::launch_apply<double>(F.d, z, r, rhs, 1, s);
+  sv::launch_apply<double>(cycle_level(F), z, r, rhs, 1, s);
   cudaMemsetAsync(acc, 0, N * sizeof(double), s);
   for (int c = 0; c < h->prm.bt_cycles; ++c) {
     const double* in = rhs;
     if (c > 0) {
-      sv::launch_apply<double>(F.d, acc, rhs, tmp, 1, s);
+      sv::launch_apply<double>(cycle_level(F), acc, rhs, tmp, 1, s);
       in = tmp;
     }
     bt_vcycle(h, 0, top, in, F.e);
