@@ -28,9 +28,10 @@
 // the whole grid; Dirichlet rows are the identity.
 //
 // One step is two cell rows of a strip of 128: K = 12 cell offsets (dx -1..1, dy -1..2)
-// x 8 + 3 x (4 pressures, in units of 2^EU and of 2^EV), 8 MMAs (M = 128
-// cells, N = 2 rows x 10 outputs padded to 32) per digit.  Bound: the latency of the instructions around the contraction (digits of 9 values,
-// 60 sums per cell; the two epilogue groups and the digit warps are about equally long),
+// x 8 + 3 x (4 pressures, in units of 2^EU and of 2^EV), 8 MMAs (M = 128 cells, N = 2
+// rows x 10 outputs padded to 32) per digit.  Bound: the latency of the instructions
+// around the contraction (digits of 9 values, 60 sums per cell; the two epilogue groups
+// and the digit warps are about equally long),
 // no longer the FP64 pipe (334 operations a vertex at 2 per clock and SM).  2048^2 with b:
 // 0.42 ms (the FP64 kernel: 1.52 ms; 6 digits of 10 bits under one exponent for all
 // components, which lost the entries above: 0.355).  All outputs in FP64 (data falling by
@@ -93,7 +94,7 @@ struct Args {
 };
 
 // Output o of cell (i, j) in FP64, out of line: the columns past the last strip and the
-// cells with non-finite values in reach
+// outputs that the contraction leaves
 __device__ __noinline__ void apply_cell(const Args& A, int i, int j, int o) {
   const int res = A.b != nullptr;
   switch (o) {
@@ -107,6 +108,12 @@ __device__ __noinline__ void apply_cell(const Args& A, int i, int j, int o) {
     case 7: ops::apply_out<double, 1, 1, 1>(A.L, A.x, A.b, A.y, res, i, j); break;
     default: ops::apply_out<double, 2, 0, 0>(A.L, A.x, A.b, A.y, res, i, j); break;
   }
+}
+
+// Those with their bit (u, v, divergence); out of line too, for the registers (424 -> 415 us)
+__device__ __noinline__ void apply_cells(const Args& A, int i, int j, unsigned redo) {
+  for (int o = 0; o < 9; ++o)
+    if ((redo >> (o >> 2)) & 1) apply_cell(A, i, j, o);
 }
 
 // The exponents of a step (E + 1022 of u and v; 0x7ff: values that are not finite) and
@@ -236,9 +243,8 @@ __device__ __forceinline__ void epilogue(const Args& A, const Shared& C, int g, 
     const long long kp = 2 * nv + static_cast<long long>(j) * np + i;
     auto at = [&](int o) { return (o >> 2) * nv + ku + ((o >> 1) & 1) * nq + (o & 1); };
     const bool res = A.b != nullptr;
-    const double sg = res ? -1.0 : 1.0;
-    const double su = sg * L.cl * exp_scale(E.eu, -71), sv = sg * L.cl * exp_scale(E.ev, -71);
-    const double pu = sg * L.cb * exp_scale(E.eu, -71), pv = sg * L.cb * exp_scale(E.ev, -71);
+    const double tu = exp_scale(E.eu, -71), tv = exp_scale(E.ev, -71), cl = res ? -L.cl : L.cl, cb = res ? -L.cb : L.cb;
+    const double su = cl * tu, sv = cl * tv, pu = cb * tu, pv = cb * tv;
     auto div = [&](double b0) { return E.eu == E.ev ? fma(pu, Tu, b0) : fma(pu, Tu, fma(pv, Tv, b0)); };
     if (i >= 1 && j >= 1 && i <= n - 1 && j <= n - 1 && redo == 0) {   // all four nodes exist and are free
       double bv[9];
@@ -259,8 +265,7 @@ __device__ __forceinline__ void epilogue(const Args& A, const Shared& C, int g, 
         else A.y[k] = res ? b0 - A.x[k] : A.x[k];   // Dirichlet row: identity
       }
       if (!(redo & 4)) A.y[kp] = div(res ? A.b[kp] : 0.0);
-      for (int o = 0; o < 9; ++o)
-        if ((redo >> (o >> 2)) & 1) apply_cell(A, i, j, o);
+      if (redo != 0) apply_cells(A, i, j, redo);
     }
   }
 }
@@ -386,11 +391,10 @@ __global__ void __launch_bounds__(NT, 1) k_apply_tc64(const Args A) {
     const unsigned lu = (static_cast<unsigned>(eu - 18) << 20) - 1u, lv = (static_cast<unsigned>(ev - 18) << 20) - 1u;
     return (c.u < lu ? LOST_U : 0u) | (c.v < lv ? LOST_V : 0u) | (c.p < lu ? LOST_PU : 0u) | (c.p < lv ? LOST_PV : 0u);
   };
-  auto words = [&](const Cell& c, int eu, int ev, Wide (&w)[8]) {
+  auto put = [&](int q, int a, int col, int eu, int ev, const Cell& c) {
+    Wide w[8];
 #pragma unroll
     for (int o = 0; o < 8; ++o) w[o] = to_wide(c.v[o], o < 4 ? eu : ev);
-  };
-  auto put = [&](int q, int a, int col, const Wide (&w)[8]) {
 #pragma unroll
     for (int j = 0; j < ND; ++j)
       *reinterpret_cast<uint4*>(sm + SM::RING + (2 * (q % 3) + a) * ROWB + j * PLANE + col * 16) =
@@ -427,9 +431,7 @@ __global__ void __launch_bounds__(NT, 1) k_apply_tc64(const Args A) {
     __syncthreads();
     choose(1, eu, ev);
     if (act) {
-      Wide w[8];
-      words(c, eu, ev, w);
-      put(q, a, col, w);
+      put(q, a, col, eu, ev, c);
       if (q == 1) put_p(0, a, col, eu, ev, c);
       const unsigned l = truncated(small, eu, ev);
       if (l != 0) atomicOr(lost, l);
@@ -459,9 +461,7 @@ __global__ void __launch_bounds__(NT, 1) k_apply_tc64(const Args A) {
         mbar_wait_or_fail(bar_done + 8 * ((s - 1) & 1), ((s - 1) >> 1) & 1, A.wait_limit, fail);
         Cell c;
         load(q - 1, a, col, act, c);
-        Wide w[8];
-        words(c, eu, ev, w);
-        if (act) put(q - 1, a, col, w);
+        if (act) put(q - 1, a, col, eu, ev, c);
         lost_before = truncated(smallest(c), eu, ev);
       } else if (s >= 2) {
         // the row pair's slot and the pressure buffer are free once step s - 2 has read them
@@ -476,10 +476,10 @@ __global__ void __launch_bounds__(NT, 1) k_apply_tc64(const Args A) {
       const unsigned lw = __reduce_or_sync(0xffffffffu, l | (lost_before & (LOST_U | LOST_V)));
       if (lw != 0 && lane == 0) atomicOr(lost + (s & 7), lw);
       lost_before = l;
-      if (act) put_p(s, a, col, eu, ev, cur);
-      Wide w[8];
-      words(cur, eu, ev, w);
-      if (act) put(q, a, col, w);
+      if (act) {
+        put_p(s, a, col, eu, ev, cur);
+        put(q, a, col, eu, ev, cur);
+      }
       if (q + 1 < S + 1) load(q + 1, a, col, act, cur);   // in flight over the fence and the next barrier
       fence_proxy();
       __syncwarp();

@@ -369,7 +369,7 @@ __global__ void k_coarse(const double* __restrict__ G, int N0, const double* __r
   if (lane == 0) e[row] = s;
 }
 
-// Levels whose per-vertex kernels run one output per thread.  At np = 129 the operator
+// Levels whose FP32 operator and transfers run one output per thread.  At np = 129 the operator
 // has 4680 such warps for 608 sub-partitions; above, a thread per vertex fills them.  The
 // prolongation's 36 outputs per coarse element fill them from half that size.
 constexpr int OUT_MAX_NP = 129;
