@@ -252,7 +252,7 @@ def job_throughput(ws, units_local: float, ms_local: float) -> tuple[float, floa
 # kernel at 1024 x 1024 (ncu --set full, summaries in profiles/); at other sizes the
 # bench scales them by the number of dofs (the traffic of a sweep is proportional)
 TRAFFIC_1024 = {
-    "fp64": {"bytes": 154744064 + 45769472 + 157928448 + 45379072, "tile": "stencil-tc",
+    "fp64": {"bytes": 154690048 + 43019520 + 157865472 + 48066560, "tile": "stencil-tc",
              "source": "profiles/tc64_kernels_f64_n1024.md (k_apply_tc64 residual + k_vanka_tc64, a sweep from a "
                        "non-zero iterate; writes still in L2 at kernel end are not counted)"},
     "mixed": {"bytes": 77614592 + 7096320, "tile": "14x14",

@@ -78,7 +78,8 @@ typedef struct {
   stokes_precision prec;  /*                                          (FP64) */
   int tile;         /* Vanka sweep configuration: -1 = chosen per level, in
                        the FP64 form by its size (stokes_level_tile), in the
-                       mixed forms by timing at creation; fused tiles of 0 = 8x8, 1 = 16x8,
+                       mixed forms by its size up to n = 64 and by timing at
+                       creation above; fused tiles of 0 = 8x8, 1 = 16x8,
                        2 = 16x16, 3 = 14x14 vertices (mixed forms: 3 = the
                        strip sweep of the interior tiles where they fit --
                        BF16 tensor-core patch GEMMs, or FP32 patch solves --
@@ -179,9 +180,10 @@ stokes_status stokes_level_n(const stokes_hierarchy* h, int level, int* n_level)
 /* Sweep configuration used on a level (see stokes_params.tile).  With tile = -1 the
  * FP64 form takes, on levels with sweeps, 7 (n < 56: the residual, then the sum of all
  * patch solves as one stencil of FP64 dot products) or 8 (above: the same stencil as an
- * exact integer contraction on the tensor cores); both are chosen by size only and are
- * not values of stokes_params.tile.  In the mixed
- * forms, 3 on a level where the interior strips fit means the strip sweep
+ * integer contraction on the tensor cores, exact but for the rounding of its operands,
+ * stokes_vanka_sweep); the mixed forms take 7, in FP32, up to n = 64.  Both are chosen
+ * by size only and are not values of stokes_params.tile.  In the mixed
+ * forms above n = 64, 3 on a level where the interior strips fit means the strip sweep
  * (tensor-core GEMMs in the BF16 form, FP32 patch solves in the FP32 form) with
  * its 14x14 SIMT ring; the autotuner may choose a SIMT shape (0..2, 6) there
  * instead. */
@@ -195,7 +197,10 @@ stokes_status stokes_level_tile(const stokes_hierarchy* h, int level, int* tile)
 stokes_status stokes_assemble_rhs(stokes_hierarchy* h, const double* f_nodal,
                                   const double* u_dirichlet, double* b);
 
-/* y = A x on level `level` (Section 2.2, the block matrix A). */
+/* y = A x on level `level` (Section 2.2, the block matrix A), in FP64: every entry within
+ * 31 u sum_k |a_jk| |x_k| (u = 2^-53) and one rounding, whatever the sizes of the other
+ * entries.  From n = 192 on the tensor cores form it from x in integer digits, and FP64
+ * where those would give an entry less. */
 stokes_status stokes_apply_operator(stokes_hierarchy* h, int level, const double* x, double* y);
 
 /* r = b - A x on level `level` (the residual step of Algorithm 1). */
@@ -206,7 +211,12 @@ stokes_status stokes_residual(stokes_hierarchy* h, int level, const double* b, c
  * x_out = x + sum_i V_i^T W_i A_i^-1 V_i (b - A x), W_i = omega diag(1/m_j),
  * every patch using the same residual.  x == NULL means x = 0.  x_out must not
  * alias x or b.  Runs in the hierarchy's precision for levels of the
- * preconditioner; this entry point always uses FP64. */
+ * preconditioner; this entry point always uses FP64.  Every entry is as accurate as
+ * that of FP64 patch solves, and a residual that is not finite reaches the dofs of its
+ * patches only; where the tensor cores run the sweep (n >= 56, stokes_level_tile), a
+ * second launch recomputes in FP64 what they would give less.  It costs little when
+ * there is nothing to recompute and up to 25 sweeps when residuals differ by more than
+ * 2^8 within 128 cells everywhere. */
 stokes_status stokes_vanka_sweep(stokes_hierarchy* h, int level, const double* x,
                                  const double* b, double* x_out);
 
@@ -248,7 +258,9 @@ stokes_status stokes_initial_guess(stokes_hierarchy* h, const double* b, double*
  * guess (Algorithm 1; a W-cycle with params.cycle = 2), or, with
  * params.precond = 1, one application of the block-triangular preconditioner
  * (Section 3.4, Algorithm 5) -- the preconditioner FGMRES applies.  r and z
- * have length N(n); they must not alias. */
+ * have length N(n); they must not alias.  In the FP64 form the sweeps and residuals of
+ * a cycle on the tensor cores round their operands 58 and 71 bits below the largest of
+ * 132 x 6 and 132 x 4 cells (FP64 numbers carry 53 bits each) and recompute nothing. */
 stokes_status stokes_vcycle_apply(stokes_hierarchy* h, const double* r, double* z);
 
 /* Solve A x = b by FGMRES(restart) right-preconditioned with the V-cycle
