@@ -260,7 +260,9 @@ stokes_status stokes_initial_guess(stokes_hierarchy* h, const double* b, double*
  * (Section 3.4, Algorithm 5) -- the preconditioner FGMRES applies.  r and z
  * have length N(n); they must not alias.  In the FP64 form the sweeps and residuals of
  * a cycle on the tensor cores round their operands 58 and 71 bits below the largest of
- * 132 x 6 and 132 x 4 cells (FP64 numbers carry 53 bits each) and recompute nothing. */
+ * 132 x 6 and 132 x 4 cells (FP64 numbers carry 53 bits each), take what lies below
+ * 2^-880 as zero and recompute nothing; a residual that is not finite reaches all cells
+ * of its step there. */
 stokes_status stokes_vcycle_apply(stokes_hierarchy* h, const double* r, double* z);
 
 /* Solve A x = b by FGMRES(restart) right-preconditioned with the V-cycle
